@@ -22,6 +22,7 @@
 // column as zero and give the pinned phi_e row the identity.
 #include <algorithm>
 
+#include "lanes.h"
 #include "problem.h"
 
 namespace knp {
@@ -59,50 +60,106 @@ __global__ void k_op_w(OpArgs A, const double* __restrict__ x, double* __restric
     w[c] = A.z[0] * A.tau[reg][0] * x01.x + A.z[1] * A.tau[reg][1] * x01.y + A.z[2] * A.tau[reg][2] * x23.x;
 }
 
-// y = rowscale .* (b - A x)  (b, rowscale optional); needs w = k_op_w(x)
+// y = rowscale .* (b - A x)  (b, rowscale optional) on the fields of row r that a lane holds in out
+template <int F>
+__device__ __forceinline__ void op_store(int64_t k, const double* out, double* __restrict__ y,
+                                         const double* __restrict__ rowscale, const double* __restrict__ b) {
+    double o[F];
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+        o[f] = out[f];
+        if (b) o[f] = b[k + f] - o[f];
+        if (rowscale) o[f] *= rowscale[k + f];
+    }
+    if constexpr (F == 4) {
+        double2* yp = reinterpret_cast<double2*>(y + k);
+        yp[0] = make_double2(o[0], o[1]);
+        yp[1] = make_double2(o[2], o[3]);
+    } else {
+#pragma unroll
+        for (int f = 0; f < F; ++f) y[k + f] = o[f];
+    }
+}
+
+// y = rowscale .* (b - A x)  (b, rowscale optional), L lanes per row (lanes.h). One thread per row
+// needs w = k_op_w(x); with more lanes the kernel is bound by its chain of loads, so it forms w from
+// the x it gathers anyway (three FMAs per entry) and saves the node pass. The loads of OP_BATCH
+// entries are issued together.
+template <int L>
+constexpr int OP_BATCH = L == 1 ? 1 : 3;
+template <int L>
 __global__ void __launch_bounds__(128) k_op_apply(OpArgs A, const double* __restrict__ x, double* __restrict__ y,
                                                   const double* __restrict__ rowscale, const double* __restrict__ b) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= A.n) return;
-    int64_t s = r / SELL_C;
-    int64_t base = A.slice_ptr[s] + r % SELL_C;
-    int64_t w = (A.slice_ptr[s + 1] - A.slice_ptr[s]) / SELL_C;
+    constexpr int F = LANE_FIELDS<L>, U = OP_BATCH<L>;
+    const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t r = gid / L;
+    const int t = (int)(gid % L);
+    if (L == 1 && r >= A.n) return;   // with more lanes, all of a warp take part in the shuffles
+    const int64_t row = r < A.n ? r : A.n - 1;
+    const int reg = row < A.N_i ? 0 : 1;
+    const int64_t s = row / SELL_C;
+    const int64_t base = A.slice_ptr[s] + row % SELL_C;
+    const int w = (int)((A.slice_ptr[s + 1] - A.slice_ptr[s]) / SELL_C);
+    const int64_t ne = A.n_entries;
+    const int32_t* cp = A.col + base;
+    const double *g0 = A.g + base, *e0 = A.e + base, *ap = A.a + base;
     double ag[KI] = {0, 0, 0}, ae[KI] = {0, 0, 0}, aw = 0.0;
-    for (int64_t k = 0; k < w; ++k) {
-        int64_t pos = base + k * SELL_C;
-        int64_t c = A.col[pos];
-        const double2* xp = reinterpret_cast<const double2*>(x + 4 * c);
-        double2 x01 = xp[0], x23 = xp[1];
-        double phi = (c == A.pin) ? 0.0 : x23.y;
-        ag[0] += A.g[pos] * x01.x;
-        ag[1] += A.g[A.n_entries + pos] * x01.y;
-        ag[2] += A.g[2 * A.n_entries + pos] * x23.x;
-        aw += A.a[pos] * A.w[c];
-        ae[0] += A.e[pos] * phi;
-        ae[1] += A.e[A.n_entries + pos] * phi;
-        ae[2] += A.e[2 * A.n_entries + pos] * phi;
+    int32_t c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = t + u * L < w ? cp[(t + u * L) * SELL_C] : 0;
+    for (int k = t; k < w; k += U * L) {
+        double2 x01[U], x23[U];
+        double gv[U][KI], ev[U][KI], av[U], wv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * L < w) {
+                const int q = (k + u * L) * SELL_C;
+                const double2* xp = reinterpret_cast<const double2*>(x + 4 * (int64_t)c[u]);
+                x01[u] = xp[0];
+                x23[u] = xp[1];
+                if (L == 1) wv[u] = A.w[c[u]];
+#pragma unroll
+                for (int i = 0; i < KI; ++i) {
+                    gv[u][i] = g0[i * ne + q];
+                    ev[u][i] = e0[i * ne + q];
+                }
+                av[u] = ap[q];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * L < w) {
+                const double phi = (c[u] == A.pin) ? 0.0 : x23[u].y;
+                if (L > 1)
+                    wv[u] = A.z[0] * A.tau[reg][0] * x01[u].x + A.z[1] * A.tau[reg][1] * x01[u].y +
+                            A.z[2] * A.tau[reg][2] * x23[u].x;
+                ag[0] += gv[u][0] * x01[u].x;
+                ag[1] += gv[u][1] * x01[u].y;
+                ag[2] += gv[u][2] * x23[u].x;
+                aw += av[u] * wv[u];
+#pragma unroll
+                for (int i = 0; i < KI; ++i) ae[i] += ev[u][i] * phi;
+            }
+            const int q = k + (U + u) * L;
+            c[u] = q < w ? cp[q * SELL_C] : 0;
+        }
     }
-    for (int t = A.xptr[r]; t < A.xptr[r + 1]; ++t) {
-        int64_t c = A.xcol[t];
-        double phi = (c == A.pin) ? 0.0 : x[4 * c + 3];
-        for (int k = 0; k < KI; ++k) ae[k] += A.xe[k * A.n_cross + t] * phi;
+    for (int u = A.xptr[row] + t; u < A.xptr[row + 1]; u += L) {
+        int64_t cc = A.xcol[u];
+        double phi = (cc == A.pin) ? 0.0 : x[4 * cc + 3];
+        for (int k = 0; k < KI; ++k) ae[k] += A.xe[k * A.n_cross + u] * phi;
     }
-    double out[4];
+    double out[4], mine[F];
     out[3] = aw;
     for (int k = 0; k < KI; ++k) {
         out[k] = ag[k] + ae[k];
         out[3] += A.z[k] * ae[k];
     }
-    if (r == A.pin) out[3] = x[4 * r + 3];
-    if (b) {
-        for (int k = 0; k < 4; ++k) out[k] = b[4 * r + k] - out[k];
-    }
-    if (rowscale) {
-        for (int k = 0; k < 4; ++k) out[k] *= rowscale[4 * r + k];
-    }
-    double2* yp = reinterpret_cast<double2*>(y + 4 * r);
-    yp[0] = make_double2(out[0], out[1]);
-    yp[1] = make_double2(out[2], out[3]);
+    lane_reduce4<double, L>(out, t, mine);
+    if (r >= A.n || t >= 4) return;
+    const int f0 = lane_field<L>(t);
+    if (r == A.pin && f0 + F == 4) mine[F - 1] = x[4 * r + 3];
+    op_store<F>(4 * r + f0, mine, y, rowscale, b);
 }
 
 // g^k = m + tau_r^k a per stored entry (padding included, where m = a = 0)
@@ -124,50 +181,74 @@ __global__ void k_fold_g(int64_t n, int64_t N_i, int64_t ne, const int64_t* __re
 // y = rowscale .* (b - A^T x): the transposed node block of entry (j, l) is
 //     c^k row:  (m + tau^k a) x^k_j + z_k tau^k a x^phi_j,   phi row:  sum_k e^k (x^k_j + z_k x^phi_j)
 // with m, a, e symmetric on same-region entries; the cross-region part uses the transposed list.
+template <int L>
 __global__ void __launch_bounds__(128) k_op_apply_t(OpArgs A, const double* __restrict__ x, double* __restrict__ y,
                                                     const double* __restrict__ rowscale,
                                                     const double* __restrict__ b) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= A.n) return;
-    const int reg = r < A.N_i ? 0 : 1;
-    int64_t s = r / SELL_C;
-    int64_t base = A.slice_ptr[s] + r % SELL_C;
-    int64_t w = (A.slice_ptr[s + 1] - A.slice_ptr[s]) / SELL_C;
+    constexpr int F = LANE_FIELDS<L>, U = OP_BATCH<L>;
+    const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t r = gid / L;
+    const int t = (int)(gid % L);
+    if (L == 1 && r >= A.n) return;
+    const int64_t row = r < A.n ? r : A.n - 1;
+    const int reg = row < A.N_i ? 0 : 1;
+    const int64_t s = row / SELL_C;
+    const int64_t base = A.slice_ptr[s] + row % SELL_C;
+    const int w = (int)((A.slice_ptr[s + 1] - A.slice_ptr[s]) / SELL_C);
+    const int64_t ne = A.n_entries;
+    const int32_t* cp = A.col + base;
+    const double *mp = A.m + base, *e0 = A.e + base, *ap0 = A.a + base;
     double am[KI] = {0, 0, 0}, aa[KI] = {0, 0, 0}, ap = 0.0, ae = 0.0;
-    for (int64_t k = 0; k < w; ++k) {
-        int64_t pos = base + k * SELL_C;
-        int64_t c = A.col[pos];
-        const double2* xp = reinterpret_cast<const double2*>(x + 4 * c);
-        double2 x01 = xp[0], x23 = xp[1];
-        double xc[KI] = {x01.x, x01.y, x23.x};
-        double phi = (c == A.pin) ? 0.0 : x23.y;
-        double mv = A.m[pos], av = A.a[pos];
-        for (int q = 0; q < KI; ++q) {
-            am[q] += mv * xc[q];
-            aa[q] += av * xc[q];
-            ae += A.e[q * A.n_entries + pos] * (xc[q] + A.z[q] * phi);
+    int32_t c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = t + u * L < w ? cp[(t + u * L) * SELL_C] : 0;
+    for (int k = t; k < w; k += U * L) {
+        double2 x01[U], x23[U];
+        double ev[U][KI], mv[U], av[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * L < w) {
+                const int q = (k + u * L) * SELL_C;
+                const double2* xp = reinterpret_cast<const double2*>(x + 4 * (int64_t)c[u]);
+                x01[u] = xp[0];
+                x23[u] = xp[1];
+#pragma unroll
+                for (int i = 0; i < KI; ++i) ev[u][i] = e0[i * ne + q];
+                mv[u] = mp[q];
+                av[u] = ap0[q];
+            }
         }
-        ap += av * phi;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * L < w) {
+                const double xc[KI] = {x01[u].x, x01[u].y, x23[u].x};
+                const double phi = (c[u] == A.pin) ? 0.0 : x23[u].y;
+#pragma unroll
+                for (int i = 0; i < KI; ++i) {
+                    am[i] += mv[u] * xc[i];
+                    aa[i] += av[u] * xc[i];
+                    ae += ev[u][i] * (xc[i] + A.z[i] * phi);
+                }
+                ap += av[u] * phi;
+            }
+            const int q = k + (U + u) * L;
+            c[u] = q < w ? cp[q * SELL_C] : 0;
+        }
     }
-    for (int t = A.xtptr[r]; t < A.xtptr[r + 1]; ++t) {
-        int64_t j = A.xtrow[t];
-        int64_t idx = A.xtidx[t];
+    for (int u = A.xtptr[row] + t; u < A.xtptr[row + 1]; u += L) {
+        int64_t j = A.xtrow[u];
+        int64_t idx = A.xtidx[u];
         double phi = (j == A.pin) ? 0.0 : x[4 * j + 3];
         for (int q = 0; q < KI; ++q) ae += A.xe[q * A.n_cross + idx] * (x[4 * j + q] + A.z[q] * phi);
     }
-    double out[4];
+    double out[4], mine[F];
     for (int q = 0; q < KI; ++q) out[q] = am[q] + A.tau[reg][q] * (aa[q] + A.z[q] * ap);
     out[3] = ae;
-    if (r == A.pin) out[3] = x[4 * r + 3];
-    if (b) {
-        for (int q = 0; q < 4; ++q) out[q] = b[4 * r + q] - out[q];
-    }
-    if (rowscale) {
-        for (int q = 0; q < 4; ++q) out[q] *= rowscale[4 * r + q];
-    }
-    double2* yp = reinterpret_cast<double2*>(y + 4 * r);
-    yp[0] = make_double2(out[0], out[1]);
-    yp[1] = make_double2(out[2], out[3]);
+    lane_reduce4<double, L>(out, t, mine);
+    if (r >= A.n || t >= 4) return;
+    const int f0 = lane_field<L>(t);
+    if (r == A.pin && f0 + F == 4) mine[F - 1] = x[4 * r + 3];
+    op_store<F>(4 * r + f0, mine, y, rowscale, b);
 }
 
 }  // namespace
@@ -197,15 +278,25 @@ void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale
     for (int r = 0; r < 2; ++r)
         for (int k = 0; k < KI; ++k) A.tau[r][k] = p->sp.reg[r].tau[k];
     for (int k = 0; k < KI; ++k) A.z[k] = p->sp.z[k];
-    unsigned blocks = (unsigned)((A.n + 127) / 128);
+    const int lanes = row_lanes(A.n, (double)A.n_entries / (double)std::max<int64_t>(A.n, 1));
+    const unsigned blocks = (unsigned)((A.n * lanes + 127) / 128);
     ProfScope ps(&p->prof, KC_SPMV, st);
+    count_launch();
     if (transpose) {
+        if (lanes == 1)
+            k_op_apply_t<1><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+        else if (lanes == 4)
+            k_op_apply_t<4><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+        else
+            k_op_apply_t<8><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+    } else if (lanes == 1) {
         count_launch();
-        k_op_apply_t<<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
-    } else {
-        count_launch(2);
         k_op_w<<<(unsigned)((A.n + 255) / 256), 256, 0, st>>>(A, x, p->op_w.p);
-        k_op_apply<<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+        k_op_apply<1><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+    } else if (lanes == 4) {
+        k_op_apply<4><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+    } else {
+        k_op_apply<8><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
     }
     KNP_CUDA(cudaGetLastError());
 }

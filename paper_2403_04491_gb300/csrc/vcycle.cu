@@ -24,6 +24,7 @@
 
 #include "amg.h"
 #include "amg_gpu.h"
+#include "lanes.h"
 #include "problem.h"
 #include "vcycle.h"
 
@@ -63,19 +64,73 @@ struct Coef4 {
     double c1[4], c2[4];
 };
 
-// Row product of a sliced-ELL operator (one thread per row)
-template <class T>
-__device__ __forceinline__ void sell_row(int64_t r, const int64_t* __restrict__ sp, const int32_t* __restrict__ col,
-                                         const T* __restrict__ val, const T* __restrict__ x, T acc[4]) {
-    int64_t s = r / SELL_C;
-    int64_t base = sp[s] + r % SELL_C;
-    int64_t w = (sp[s + 1] - sp[s]) / SELL_C;
+__device__ __forceinline__ double pick4(const double c[4], int f) {
+    return f == 0 ? c[0] : f == 1 ? c[1] : f == 2 ? c[2] : c[3];
+}
+
+// N consecutive fields of a node (4: one vector access)
+template <class T, int N>
+struct VN {
+    T v[N];
+    __device__ __forceinline__ static VN load(const T* p) {
+        VN o;
+        if constexpr (N == 4) {
+            const V4<T> a = V4<T>::load(p);
+#pragma unroll
+            for (int f = 0; f < 4; ++f) o.v[f] = a.v[f];
+        } else {
+#pragma unroll
+            for (int f = 0; f < N; ++f) o.v[f] = p[f];
+        }
+        return o;
+    }
+    __device__ __forceinline__ void store(T* p) const {
+        if constexpr (N == 4) {
+            V4<T>{{v[0], v[1], v[2], v[3]}}.store(p);
+        } else {
+#pragma unroll
+            for (int f = 0; f < N; ++f) p[f] = v[f];
+        }
+    }
+};
+
+// Row product of a sliced-ELL operator by L lanes: lane t adds entries t, t + L, ... The loads of
+// U entries (and the columns of the next batch) are issued together, so that a lane waits
+// for memory once or twice per batch instead of twice per entry; the order of the sums is that of
+// the entries.
+template <class T, int L>
+__device__ __forceinline__ void sell_row(int64_t r, int t, const int64_t* __restrict__ sp,
+                                         const int32_t* __restrict__ col, const T* __restrict__ val,
+                                         const T* __restrict__ x, T acc[4]) {
+    const int64_t s = r / SELL_C;
+    const int64_t base = sp[s] + r % SELL_C;
+    const int w = (int)((sp[s + 1] - sp[s]) / SELL_C);
+    constexpr int U = L == 1 ? 1 : 4;
+    const int32_t* cp = col + base;
+    const T* vp = val + 4 * base;
     acc[0] = acc[1] = acc[2] = acc[3] = T(0);
-    for (int64_t k = 0; k < w; ++k) {
-        int64_t pos = base + k * SELL_C;
-        V4<T> a = V4<T>::load(val + 4 * pos);
-        V4<T> xv = V4<T>::load(x + 4 * (int64_t)col[pos]);
-        for (int f = 0; f < 4; ++f) acc[f] += a.v[f] * xv.v[f];
+    int32_t c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = t + u * L < w ? cp[(t + u * L) * SELL_C] : 0;
+    for (int k = t; k < w; k += U * L) {
+        V4<T> a[U], xv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * L < w) {
+                a[u] = V4<T>::load(vp + 4 * ((k + u * L) * SELL_C));
+                xv[u] = V4<T>::load(x + 4 * (int64_t)c[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = k + (U + u) * L;
+            c[u] = q < w ? cp[q * SELL_C] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * L < w)
+                for (int f = 0; f < 4; ++f) acc[f] += a[u].v[f] * xv[u].v[f];
+        }
     }
 }
 
@@ -110,10 +165,6 @@ __device__ __forceinline__ T csr_row_field(bool active, int64_t r, int slot, int
     return acc;
 }
 
-__device__ __forceinline__ double pick4(const double c[4], int f) {
-    return f == 0 ? c[0] : f == 1 ? c[1] : f == 2 ? c[2] : c[3];
-}
-
 // The coarse correction's input at node i: t = s .* v - (A Z y)_i. Row i of A Z y: its same-region
 // phi columns hold its own group's constant (the row sums RS), its cross-region entries their
 // groups' constants; the potential row is sum_k z_k of the concentration rows' terms, and the
@@ -135,11 +186,12 @@ __device__ __forceinline__ void defl_input(int64_t i, const double* __restrict__
     t[3] = s[4 * i + 3] * v[4 * i + 3] - out3;
 }
 
-// first Chebyshev step from x = 0: d = c2 D^-1 b, x = d. On the finest level b = s .* v (double
+// first Chebyshev step from x = 0: d = c2 D^-1 b, x = d (d stored if a second step reads it). On the finest level b = s .* v (double
 // input), or s .* v - A Z y inside the coarse correction (df.y set).
 template <class T>
 __global__ void k_cheb_first(int64_t n, const double* __restrict__ v, const double* __restrict__ s, T* __restrict__ b,
-                             const T* __restrict__ dinv, Coef4 c, T* __restrict__ x, T* __restrict__ d, DeflFuse df) {
+                             const T* __restrict__ dinv, Coef4 c, T* __restrict__ x, T* __restrict__ d, DeflFuse df,
+                             int write_d) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     V4<T> bb;
@@ -156,37 +208,40 @@ __global__ void k_cheb_first(int64_t n, const double* __restrict__ v, const doub
     }
     V4<T> di = V4<T>::load(dinv + 4 * i), dd;
     for (int f = 0; f < 4; ++f) dd.v[f] = (T)c.c2[f] * di.v[f] * bb.v[f];
-    dd.store(d + 4 * i);
+    if (write_d) dd.store(d + 4 * i);
     dd.store(x + 4 * i);
 }
 
-// Chebyshev update of one row given acc = (A x_in)_row
-template <class T>
-__device__ __forceinline__ void cheb_update(int64_t i, const T acc[4], const T* __restrict__ x_in,
-                                            const T* __restrict__ b, const T* __restrict__ dinv, const Coef4& c,
-                                            T* __restrict__ d, T* __restrict__ x_out) {
-    V4<T> bb = V4<T>::load(b + 4 * i), di = V4<T>::load(dinv + 4 * i), dd = V4<T>::load(d + 4 * i),
-          xx = V4<T>::load(x_in + 4 * i);
-    for (int f = 0; f < 4; ++f) {
-        dd.v[f] = (T)c.c1[f] * dd.v[f] + (T)c.c2[f] * di.v[f] * (bb.v[f] - acc[f]);
-        xx.v[f] += dd.v[f];
-    }
-    dd.store(d + 4 * i);
-    xx.store(x_out + 4 * i);
-}
-
-// Chebyshev step: r = b - A x_in; d = c1 d + c2 D^-1 r; x_out = x_in + d
-template <class T>
+// Chebyshev step: r = b - A x_in; d = c1 d + c2 D^-1 r; x_out = x_in + d. The first step of a sweep
+// (c1 = 0) does not read d, the last one does not store it.
+template <class T, int L>
 __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __restrict__ sp,
                                                    const int32_t* __restrict__ col, const T* __restrict__ val,
                                                    const T* __restrict__ x_in, const T* __restrict__ b,
                                                    const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
-                                                   T* __restrict__ x_out) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    T acc[4];
-    sell_row<T>(i, sp, col, val, x_in, acc);
-    cheb_update<T>(i, acc, x_in, b, dinv, c, d, x_out);
+                                                   T* __restrict__ x_out, int read_d, int write_d) {
+    constexpr int F = LANE_FIELDS<L>;
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = g / L;
+    const int t = (int)(g % L);
+    if (L == 1 && i >= n) return;   // with more lanes, all of a warp take part in the shuffles
+    T acc[4], ax[F];
+    sell_row<T, L>(i < n ? i : n - 1, t, sp, col, val, x_in, acc);
+    lane_reduce4<T, L>(acc, t, ax);
+    if (i >= n || t >= 4) return;
+    const int f0 = lane_field<L>(t);
+    const int64_t k = 4 * i + f0;
+    VN<T, F> bb = VN<T, F>::load(b + k), di = VN<T, F>::load(dinv + k), xx = VN<T, F>::load(x_in + k), dd;
+    if (read_d) {
+        dd = VN<T, F>::load(d + k);
+        for (int f = 0; f < F; ++f)
+            dd.v[f] = (T)pick4(c.c1, f0 + f) * dd.v[f] + (T)pick4(c.c2, f0 + f) * di.v[f] * (bb.v[f] - ax[f]);
+    } else {
+        for (int f = 0; f < F; ++f) dd.v[f] = (T)pick4(c.c2, f0 + f) * di.v[f] * (bb.v[f] - ax[f]);
+    }
+    for (int f = 0; f < F; ++f) xx.v[f] += dd.v[f];
+    if (write_d) dd.store(d + k);
+    xx.store(x_out + k);
 }
 
 template <class T, int S>
@@ -194,43 +249,44 @@ __global__ void __launch_bounds__(128) k_cheb_csr(int64_t n, const int64_t* __re
                                                   const int32_t* __restrict__ col, const T* __restrict__ val,
                                                   const T* __restrict__ x_in, const T* __restrict__ b,
                                                   const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
-                                                  T* __restrict__ x_out) {
+                                                  T* __restrict__ x_out, int read_d, int write_d) {
     int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
     int64_t i = g / (4 * S);
     int lane = (int)(g % (4 * S)), f = lane & 3;
     T acc = csr_row_field<T, S>(i < n, i, lane >> 2, f, ptr, col, val, x_in);
     if (lane < 4 && i < n) {
         const int64_t k = 4 * i + f;
-        T dd = (T)pick4(c.c1, f) * d[k] + (T)pick4(c.c2, f) * dinv[k] * (b[k] - acc);
-        d[k] = dd;
+        T dd = (T)pick4(c.c2, f) * dinv[k] * (b[k] - acc);
+        if (read_d) dd = (T)pick4(c.c1, f) * d[k] + dd;
+        if (write_d) d[k] = dd;
         x_out[k] = x_in[k] + dd;
     }
 }
 
-template <class T>
+// y = b - A x on a sliced-ELL level (b == nullptr: y = A x)
+template <class T, int L>
 __global__ void __launch_bounds__(128) k_resid_sell(int64_t n, const int64_t* __restrict__ sp,
                                                     const int32_t* __restrict__ col, const T* __restrict__ val,
                                                     const T* __restrict__ x, const T* __restrict__ b,
-                                                    T* __restrict__ r) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    T acc[4];
-    sell_row<T>(i, sp, col, val, x, acc);
-    V4<T> bb = V4<T>::load(b + 4 * i);
-    for (int f = 0; f < 4; ++f) bb.v[f] -= acc[f];
-    bb.store(r + 4 * i);
-}
-
-// y = A x on a sliced-ELL level
-template <class T>
-__global__ void __launch_bounds__(128) k_sell_apply(int64_t n, const int64_t* __restrict__ sp,
-                                                    const int32_t* __restrict__ col, const T* __restrict__ val,
-                                                    const T* __restrict__ x, T* __restrict__ y) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    T acc[4];
-    sell_row<T>(i, sp, col, val, x, acc);
-    V4<T>{{acc[0], acc[1], acc[2], acc[3]}}.store(y + 4 * i);
+                                                    T* __restrict__ y) {
+    constexpr int F = LANE_FIELDS<L>;
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = g / L;
+    const int t = (int)(g % L);
+    if (L == 1 && i >= n) return;
+    T acc[4], ax[F];
+    sell_row<T, L>(i < n ? i : n - 1, t, sp, col, val, x, acc);
+    lane_reduce4<T, L>(acc, t, ax);
+    if (i >= n || t >= 4) return;
+    const int64_t k = 4 * i + lane_field<L>(t);
+    VN<T, F> out;
+    if (b) {
+        out = VN<T, F>::load(b + k);
+        for (int f = 0; f < F; ++f) out.v[f] -= ax[f];
+    } else {
+        for (int f = 0; f < F; ++f) out.v[f] = ax[f];
+    }
+    out.store(y + k);
 }
 
 template <class T, int S>
@@ -359,6 +415,7 @@ template <class T>
 struct DevLevel {
     int64_t n = 0, nnz = 0;
     bool sell = false;
+    int lanes = 1;   // lanes per row of the sliced-ELL kernels
     // sliced ELL (every level whose padding is small)
     DArray<int64_t> sp;
     DArray<int32_t> scol;
@@ -480,6 +537,7 @@ static void upload_hierarchy(AmgDev<T>& D, const HostHierarchy& H, int degree, i
         L->n = n;
         L->nnz = HL.A.nnz();
         L->sell = upload_sell(*L, HL.A, st);
+        L->lanes = row_lanes(n, n ? (double)L->nnz / (double)n : 1.0);
         if (!L->sell) L->A.upload(HL.A, st);
         L->dinv.upload(cast_vec<T>(HL.dinv), st);
         for (int f = 0; f < 4; ++f) {
@@ -565,6 +623,7 @@ static void take_hierarchy(AmgDev<T>& D, GpuHierarchy& H, int degree, int pre, c
         L->n = n;
         L->nnz = G->A.nnz;
         L->sell = take_sell(*L, G->A, st);
+        L->lanes = row_lanes(n, n ? (double)L->nnz / (double)n : 1.0);
         if (!L->sell) L->A.take(G->A, st);
         take_values(L->dinv, G->dinv, 4 * n, st);
         for (int f = 0; f < 4; ++f) {
@@ -640,30 +699,50 @@ void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, in
         default: KERNEL<T, 32><<<nblk((grid_rows) * 128, 128), 128, 0, st>>>(__VA_ARGS__); break;         \
     }
 
+// sliced-ELL kernels with the level's lanes per row
+#define KNP_LANE_DISPATCH(lanes, KERNEL, rows, ...)                                               \
+    switch (lanes) {                                                                              \
+        case 1: KERNEL<T, 1><<<nblk(rows, 128), 128, 0, st>>>(__VA_ARGS__); break;                \
+        case 4: KERNEL<T, 4><<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
+        default: KERNEL<T, 8><<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;         \
+    }
+
+// Chebyshev step k of a sweep of `steps` steps
 template <class T>
-static void cheb_step(DevLevel<T>& L, const Coef4& c, Profiler* pr, bool fine, cudaStream_t st) {
+static void launch_cheb(const DevLevel<T>& L, const T* x_in, const T* b, const Coef4& c, T* d, T* x_out, int k,
+                        int steps, cudaStream_t st) {
+    count_launch();
+    const int read_d = k > 0, write_d = k + 1 < steps;
+    if (L.sell) {
+        KNP_LANE_DISPATCH(L.lanes, k_cheb_sell, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x_in, b, L.dinv.p, c, d, x_out,
+                          read_d, write_d);
+    } else {
+        KNP_SLOT_DISPATCH(L.A.slots, k_cheb_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x_in, b, L.dinv.p, c, d,
+                         x_out, read_d, write_d);
+    }
+}
+
+template <class T>
+static void launch_resid(const DevLevel<T>& L, const T* x, const T* b, T* r, cudaStream_t st) {
     count_launch();
     if (L.sell) {
-        ProfScope ps(fine ? pr : nullptr, KC_CHEB_FINE, st);
-        k_cheb_sell<T><<<nblk(L.n, 128), 128, 0, st>>>(L.n, L.sp.p, L.scol.p, L.sval.p, L.x.p, L.b.p, L.dinv.p, c,
-                                                       L.d.p, L.x2.p);
+        KNP_LANE_DISPATCH(L.lanes, k_resid_sell, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x, b, r);
     } else {
-        ProfScope ps(fine ? pr : nullptr, KC_CHEB_FINE, st);
-        KNP_SLOT_DISPATCH(L.A.slots, k_cheb_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, L.x.p, L.b.p, L.dinv.p, c,
-                         L.d.p, L.x2.p);
+        KNP_SLOT_DISPATCH(L.A.slots, k_resid_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x, b, r);
     }
+}
+
+template <class T>
+static void cheb_step(DevLevel<T>& L, const Coef4& c, int k, int steps, Profiler* pr, bool fine, cudaStream_t st) {
+    ProfScope ps(fine ? pr : nullptr, KC_CHEB_FINE, st);
+    launch_cheb(L, L.x.p, L.b.p, c, L.d.p, L.x2.p, k, steps, st);
     std::swap(L.x.p, L.x2.p);
 }
 
 template <class T>
 static void residual(DevLevel<T>& L, Profiler* pr, bool fine, cudaStream_t st) {
-    count_launch();
     ProfScope ps(fine ? pr : nullptr, KC_RESID_FINE, st);
-    if (L.sell) {
-        k_resid_sell<T><<<nblk(L.n, 128), 128, 0, st>>>(L.n, L.sp.p, L.scol.p, L.sval.p, L.x.p, L.b.p, L.r.p);
-    } else {
-        KNP_SLOT_DISPATCH(L.A.slots, k_resid_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, L.x.p, L.b.p, L.r.p);
-    }
+    launch_resid(L, L.x.p, L.b.p, L.r.p, st);
 }
 
 template <class T>
@@ -678,10 +757,11 @@ static void smooth(DevLevel<T>& L, const std::vector<Coef4>& cs, int degree, boo
     int k0 = 0;
     if (zero_start) {
         count_launch();
-        k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, L.b.p, L.dinv.p, cs[0], L.x.p, L.d.p, df);
+        k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, L.b.p, L.dinv.p, cs[0], L.x.p, L.d.p, df,
+                                                         degree > 1);
         k0 = 1;
     }
-    for (int k = k0; k < degree; ++k) cheb_step(L, cs[k], pr, fine, st);
+    for (int k = k0; k < degree; ++k) cheb_step(L, cs[k], k, degree, pr, fine, st);
 }
 
 template <class T>
@@ -694,7 +774,7 @@ static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, co
             // single-level hierarchy: build b from the scaled input first
             Coef4 c0{};
             count_launch();
-            k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, L.b.p, L.dinv.p, c0, L.x.p, L.d.p, df);
+            k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, L.b.p, L.dinv.p, c0, L.x.p, L.d.p, df, 0);
         }
         count_launch();
         k_coarse<T><<<nblk(4 * D.nc * 32, 256), 256, 0, st>>>(D.nc, D.cinv.p, L.b.p, L.x.p);
@@ -741,8 +821,7 @@ void p0_apply(knp_problem* p, const double* x, double* y) {
     KNP_REQUIRE(p->amg && p->amg->h64, KNP_ERR_STATE, "P_0 products need the FP64 hierarchy");
     DevLevel<double>& L = *static_cast<AmgDev<double>*>(p->amg->h64)->L[0];
     KNP_REQUIRE(L.sell, KNP_ERR_STATE, "the finest level is not sliced ELL");
-    count_launch();
-    k_sell_apply<double><<<nblk(L.n, 128), 128, 0, p->stream>>>(L.n, L.sp.p, L.scol.p, L.sval.p, x, y);
+    launch_resid<double>(L, x, nullptr, y, p->stream);
     KNP_CUDA(cudaGetLastError());
 }
 
@@ -862,15 +941,8 @@ struct NaWork {
 inline size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 template <class T>
-static void na_cheb_step(DevLevel<T>& L, NaWork<T>& w, const Coef4& c, cudaStream_t st) {
-    count_launch();
-    if (L.sell) {
-        k_cheb_sell<T><<<nblk(L.n, 128), 128, 0, st>>>(L.n, L.sp.p, L.scol.p, L.sval.p, w.x, w.b, L.dinv.p, c, w.d,
-                                                       w.x2);
-    } else {
-        KNP_SLOT_DISPATCH(L.A.slots, k_cheb_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, w.x, w.b, L.dinv.p, c, w.d,
-                         w.x2);
-    }
+static void na_cheb_step(DevLevel<T>& L, NaWork<T>& w, const Coef4& c, int k, int steps, cudaStream_t st) {
+    launch_cheb(L, w.x, w.b, c, w.d, w.x2, k, steps, st);
     std::swap(w.x, w.x2);
 }
 
@@ -884,7 +956,7 @@ static void na_vcycle_rec(AmgDev<T>& D, std::vector<NaWork<T>>& W, int l, const 
         if (v) {
             Coef4 c0{};
             count_launch();
-            k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, w.b, L.dinv.p, c0, w.x, w.d, DeflFuse{});
+            k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, w.b, L.dinv.p, c0, w.x, w.d, DeflFuse{}, 0);
         }
         count_launch();
         k_coarse<T><<<nblk(4 * D.nc * 32, 256), 256, 0, st>>>(D.nc, D.cinv.p, w.b, w.x);
@@ -894,20 +966,16 @@ static void na_vcycle_rec(AmgDev<T>& D, std::vector<NaWork<T>>& W, int l, const 
     NaWork<T>& wc = W[l + 1];
     const std::vector<Coef4>& cs = D.coef[l];
     count_launch();
-    k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, w.b, L.dinv.p, cs[0], w.x, w.d, DeflFuse{});
-    for (int k = 1; k < D.pre; ++k) na_cheb_step(L, w, cs[k], st);
-    count_launch();
-    if (L.sell) {
-        k_resid_sell<T><<<nblk(L.n, 128), 128, 0, st>>>(L.n, L.sp.p, L.scol.p, L.sval.p, w.x, w.b, w.r);
-    } else {
-        KNP_SLOT_DISPATCH(L.A.slots, k_resid_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, w.x, w.b, w.r);
-    }
+    k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, w.b, L.dinv.p, cs[0], w.x, w.d, DeflFuse{},
+                                                     D.pre > 1);
+    for (int k = 1; k < D.pre; ++k) na_cheb_step(L, w, cs[k], k, D.pre, st);
+    launch_resid(L, w.x, w.b, w.r, st);
     count_launch();
     KNP_SLOT_DISPATCH(L.R.slots, k_csr4, C.n, C.n, L.R.ptr.p, L.R.col.p, L.R.val.p, w.r, wc.b, 0);
     na_vcycle_rec(D, W, l + 1, nullptr, nullptr, st);
     count_launch();
     KNP_SLOT_DISPATCH(L.P.slots, k_csr4, L.n, L.n, L.P.ptr.p, L.P.col.p, L.P.val.p, wc.x, w.x, 1);
-    for (int k = 0; k < D.degree; ++k) na_cheb_step(L, w, cs[k], st);
+    for (int k = 0; k < D.degree; ++k) na_cheb_step(L, w, cs[k], k, D.degree, st);
 }
 
 // Lays the work vectors out in the static array; returns the bytes needed (and fills W when
