@@ -25,8 +25,6 @@
 #include <algorithm>
 #include <chrono>
 #include <map>
-#include <mutex>
-#include <unordered_map>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -40,21 +38,31 @@ namespace knp {
 
 namespace {
 
-constexpr int RED_BLOCKS = 608;   // 4 x 152 SMs: the most blocks a reduction kernel launches
+constexpr int RED_BLOCKS = 152;   // the most blocks a reduction kernel launches: one per SM (152 SMs)
 constexpr int RED_THREADS = 256;
 constexpr int MAXV = 32;          // restart + 2
-constexpr int MAXW = 3 * MAXV;    // partial-sum slots per block
+constexpr int MAXW = 3 * MAXV;    // the most sums a reduction kernel forms
+constexpr int PART_LD = RED_BLOCKS + 8;   // partial[k * PART_LD + b]: block b's share of sum k
 // device scalars: [0, MAXV) first-pass dots, [MAXV, 2 MAXV) second-pass dots, [2 MAXV, 2 MAXV +
-// MAXW) reference norms, 2 MAXV + MAXW the skip flag, then the six stopping-test norms
+// MAXW) reference norms, 2 MAXV + MAXW the skip flag, then the six stopping-test norms, then the
+// second-pass flag of the Arnoldi step
 constexpr int CHK_OFF = 2 * MAXV + MAXW + 1;
-constexpr int DOTS_LEN = CHK_OFF + 6;
+constexpr int SECOND_OFF = CHK_OFF + 6;
+constexpr int DOTS_LEN = SECOND_OFF + 1;
 constexpr int CHECK_EVERY = 8;         // steps between exact evaluations of the stopping test, at most
                                        // (8 against 4: 0.8-1.4% less time per step on the 3D and 2D
                                        // workloads, iteration counts equal or +2 in 290)
 constexpr double CHECK_MARGIN = 10.0;  // evaluate once a prediction is within this factor of passing
 
-// Every kernel below is instantiated for a compile-time vector count NV, so that the
-// accumulators and basis values stay in registers (a runtime count put them on the stack).
+// What bounds these kernels: an FP64 instruction holds an SM's FP64 pipe for 16 cycles per warp, so
+// what counts is the number of warp instructions, not only the vector elements: a reduction's adds
+// and any scalar that every thread works out for itself cost as much as vector work. Hence one block
+// of 8 warps per SM whose threads take two elements (16 bytes) of each vector at a time, so that the
+// 31 adds of a warp's reduction are paid by 8 warps per SM and not by 32; scalars are formed once per
+// block; and each kernel sums the partial results of the one before it in its prologue (about 1 us)
+// instead of a reduction launch (4.8 us) between them.
+// Every kernel is instantiated for a compile-time vector count NV, so that the accumulators and
+// basis values stay in registers (a runtime count put them on the stack).
 
 // One halving step of a warp reduce-scatter of C values per lane (C even): lanes with bit O
 // set keep the upper half and receive their partner's upper half, the others the lower half.
@@ -69,232 +77,352 @@ __device__ __forceinline__ void warp_halve(double* v, int lane, int O) {
     }
 }
 
-// Block sums of NT values per thread into partial[blockIdx.x][0..NT). Inside a warp the NT
-// values (padded to C, a multiple of 32) are reduce-scattered in five halving steps, which
-// leave lane L with the warp sums of values [L C/32, (L+1) C/32): about C shuffles and adds
-// per lane instead of 5 NT for a butterfly per value (the adds are FP64, the scarce pipe).
+// Warp sums of C values per lane (C a power of two up to 32): C - 1 adds of a reduce-scatter, then
+// one for each halving of the lanes that are left. Returns the sum of value lane / (32 / C).
+template <int C>
+__device__ __forceinline__ double warp_sums(double* v, int lane) {
+    if constexpr (C == 32) warp_halve<32>(v, lane, 16);
+    if constexpr (C >= 16) warp_halve<16>(v, lane, C == 32 ? 8 : 16);
+    if constexpr (C >= 8) warp_halve<8>(v, lane, C == 32 ? 4 : C == 16 ? 8 : 16);
+    if constexpr (C >= 4) warp_halve<4>(v, lane, C == 32 ? 2 : C == 16 ? 4 : C == 8 ? 8 : 16);
+    if constexpr (C >= 2) warp_halve<2>(v, lane, C == 32 ? 1 : C == 16 ? 2 : C == 8 ? 4 : C == 4 ? 8 : 16);
+    double s = v[0];
+#pragma unroll
+    for (int o = 16 / C; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+template <int NT>
+constexpr int POW2 = NT <= 1 ? 1 : NT <= 2 ? 2 : NT <= 4 ? 4 : NT <= 8 ? 8 : NT <= 16 ? 16 : 32;
+
+// Block sums of NT values per thread (NT <= 32) into partial[k * PART_LD + blockIdx.x]
 template <int NT>
 __device__ __forceinline__ void block_reduce_store(const double (&acc)[NT], double* __restrict__ partial) {
-    constexpr int C = (NT + 31) / 32 * 32;
-    constexpr int PER = C / 32;
+    constexpr int C = POW2<NT>;
+    static_assert(NT <= 32, "at most 32 sums");
     __shared__ double sh[RED_THREADS / 32][C];
     const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
     double v[C];
 #pragma unroll
     for (int k = 0; k < C; ++k) v[k] = k < NT ? acc[k] : 0.0;
-    warp_halve<C>(v, lane, 16);
-    warp_halve<C / 2>(v, lane, 8);
-    warp_halve<C / 4>(v, lane, 4);
-    warp_halve<C / 8>(v, lane, 2);
-    warp_halve<C / 16>(v, lane, 1);
-#pragma unroll
-    for (int m = 0; m < PER; ++m) sh[wid][lane * PER + m] = v[m];
+    const double s = warp_sums<C>(v, lane);
+    if (lane % (32 / C) == 0) sh[wid][lane / (32 / C)] = s;
     __syncthreads();
     if (threadIdx.x < NT) {
-        double s = 0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) s += sh[w][threadIdx.x];
-        partial[(int64_t)blockIdx.x * MAXW + threadIdx.x] = s;
+        double t = 0;
+        for (int w = 0; w < RED_THREADS / 32; ++w) t += sh[w][threadIdx.x];
+        partial[threadIdx.x * PART_LD + blockIdx.x] = t;
     }
 }
 
-// partial[b][k] = block b's share of <V_k, w> for k < NV, and of <w, w> at k = NV
+// out[k] = sum over blocks of partial[k * PART_LD + b], k < nt, by one block of RED_THREADS: each
+// warp takes four sums at a time. Every block of a kernel gets the same bits. out is shared memory.
+__device__ __forceinline__ void sum_partials(const double* __restrict__ partial, int nblocks, int nt, double* out) {
+    const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
+    for (int k0 = 4 * wid; k0 < nt; k0 += 4 * (RED_THREADS / 32)) {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int b = lane; b < nblocks; b += 32) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (k0 + q < nt) v[q] += partial[(k0 + q) * PART_LD + b];
+        }
+        const double s = warp_sums<4>(v, lane);
+        if (lane % 8 == 0 && k0 + lane / 8 < nt) out[k0 + lane / 8] = s;
+    }
+    __syncthreads();
+}
+
+// Two neighbouring elements of a vector; vectors are 4 n doubles, 16-byte aligned
+__device__ __forceinline__ double2 ld2(const double* __restrict__ p, int64_t i2) {
+    return reinterpret_cast<const double2*>(p)[i2];
+}
+__device__ __forceinline__ void st2(double* __restrict__ p, int64_t i2, double2 v) {
+    reinterpret_cast<double2*>(p)[i2] = v;
+}
+
+// Pairs per thread and sweep: few vectors leave too few bytes in flight with one
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n4, const double* __restrict__ V, int64_t ldv,
-                                                      const double* __restrict__ w, double* __restrict__ partial) {
+constexpr int PAIRS = NV <= 3 ? 4 : NV <= 7 ? 2 : 1;
+
+// partial sums of <V_k, w> for k < NV, and of <w, w> at k = NV
+template <int NV>
+__global__ void __launch_bounds__(RED_THREADS, 1) k_mdot(int64_t n4, const double* __restrict__ V, int64_t ldv,
+                                                         const double* __restrict__ w, double* __restrict__ partial) {
+    constexpr int E = PAIRS<NV>;
     double acc[NV + 1];
 #pragma unroll
     for (int k = 0; k <= NV; ++k) acc[k] = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        double wi = w[i];
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
+    for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n2; i += E * stride) {
+        double2 wi[E], vk[E][NV > 0 ? NV : 1];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] += V[k * ldv + i] * wi;
-        acc[NV] += wi * wi;
+        for (int e = 0; e < E; ++e) {
+            const bool in = e == 0 || i + e * stride < n2;
+            wi[e] = in ? ld2(w, i + e * stride) : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) vk[e][k] = in ? ld2(V + k * ldv, i + e * stride) : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (e > 0 && i + e * stride >= n2) break;
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                acc[k] += vk[e][k].x * wi[e].x;
+                acc[k] += vk[e][k].y * wi[e].y;
+            }
+            acc[NV] += wi[e].x * wi[e].x;
+            acc[NV] += wi[e].y * wi[e].y;
+        }
     }
     block_reduce_store<NV + 1>(acc, partial);
 }
 
-// S^2-weighted dots split by group: slot NG*k + g holds group g's part of <V_k, w>_S and slots
-// NG*NV + g hold <w, w>_S. Groups: 0 = concentrations (fields 0..2), 1 = potentials (field 3);
-// with NG = 3, group 2 takes the extracellular potentials (elements at or past n4i).
-template <int NV, int NG>
-__global__ void __launch_bounds__(RED_THREADS) k_mdot_split(int64_t n4, const double* __restrict__ V, int64_t ldv,
-                                                            const double* __restrict__ w, const double* __restrict__ s,
-                                                            int64_t n4i, double* __restrict__ partial) {
-    double acc[NV + 1];
-    double out[NG * (NV + 1)];
-#pragma unroll
-    for (int k = 0; k <= NV; ++k) acc[k] = 0.0;
-#pragma unroll
-    for (int k = 0; k < NG * (NV + 1); ++k) out[k] = 0.0;
-    // the grid stride is a multiple of 4, so every thread keeps the same field; a thread of the
-    // potential field crosses the region boundary at most once, which flushes its sums
-    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool phi = (i0 & 3) == 3;
-    int grp = phi ? ((NG == 3 && i0 >= n4i) ? 2 : 1) : 0;
-    for (int64_t i = i0; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        if (NG == 3 && phi && grp == 1 && i >= n4i) {
-#pragma unroll
-            for (int k = 0; k <= NV; ++k) {
-                out[NG * k + 1] += acc[k];
-                acc[k] = 0.0;
-            }
-            grp = 2;
+// Sums of squares per group of an element-wise quantity: groups 0 = concentrations (fields 0..2), 1 =
+// potentials (field 3); with NG = 3, group 2 takes the extracellular potentials (elements at or past
+// n4i). A thread's pairs are all fields (0, 1) or all fields (2, 3), since the grid stride is even, and
+// its potentials cross the region boundary at most once.
+template <int NG>
+struct GroupSums {
+    double a = 0.0, b = 0.0, before = 0.0;   // first and second element of the pair; b up to the boundary
+    bool past = false;
+    __device__ __forceinline__ void add(int64_t i2, int64_t n4i, double x, double y) {
+        if (NG == 3 && !past && 2 * i2 >= n4i) {
+            before = b;
+            b = 0.0;
+            past = true;
         }
-        double wi = w[i] * s[i] * s[i];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] += V[k * ldv + i] * wi;
-        acc[NV] += wi * w[i];
+        a += x * x;
+        b += y * y;
     }
-#pragma unroll
-    for (int k = 0; k <= NV; ++k) {
-        if (grp == 0) out[NG * k] += acc[k];
-        if (grp == 1) out[NG * k + 1] += acc[k];
-        if (NG == 3 && grp == 2) out[NG * k + NG - 1] += acc[k];
+    // out[0..NG): this thread's sums; hi: its pairs are fields (2, 3)
+    __device__ __forceinline__ void get(bool hi, double* out) const {
+        out[0] = hi ? a : a + (NG == 3 ? before + b : b);
+        out[1] = !hi ? 0.0 : NG == 3 ? (past ? before : b) : b;
+        if (NG == 3) out[NG - 1] = hi && past ? b : 0.0;
     }
-    block_reduce_store<NG * (NV + 1)>(out, partial);
+};
+
+// partial sums of ||s .* w||^2 per group (the stopping test's reference norms)
+template <int NG>
+__global__ void __launch_bounds__(RED_THREADS) k_group_norms(int64_t n4, const double* __restrict__ w,
+                                                             const double* __restrict__ s, int64_t n4i,
+                                                             double* __restrict__ partial) {
+    GroupSums<NG> g;
+    const int64_t n2 = n4 / 2, i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
+    for (int64_t i = i0; i < n2; i += (int64_t)gridDim.x * RED_THREADS) {
+        const double2 wi = ld2(w, i), si = ld2(s, i);
+        g.add(i, n4i, wi.x * si.x, wi.y * si.y);
+    }
+    double out[NG];
+    g.get((i0 & 1) != 0, out);
+    block_reduce_store<NG>(out, partial);
 }
 
-// S^2-weighted squared norms, by group, of two combinations of the columns of Z:
+// Partial sums of the S^2-weighted squared norms, by group, of two combinations of the columns of Z:
 // u = sum_k c[k] Z_k and v = sum_k y[k] Z_k (y[NV-1] is the newest column's, often 0).
 // Slot g holds group g's part of ||u||_S^2 and slot NG + g that of ||v||_S^2 (groups as above).
-// Without with_y only u is formed (v's slots stay zero): half the FP64 work.
+// Without with_y only u is formed (v's slots are zero): half the FP64 work.
 template <int NV, int NG>
-__global__ void __launch_bounds__(RED_THREADS) k_combo_norms(int64_t n4, const double* __restrict__ Z, int64_t ldz,
-                                                             const double* __restrict__ cy, const double* __restrict__ s,
-                                                             int64_t n4i, double* __restrict__ partial, int with_y) {
-    double ck[NV > 0 ? NV : 1], yk[NV > 0 ? NV : 1];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        ck[k] = cy[k];
-        yk[k] = cy[MAXV + k];
+__global__ void __launch_bounds__(RED_THREADS, 1) k_combo_norms(int64_t n4, const double* __restrict__ Z, int64_t ldz,
+                                                                const double* __restrict__ cy,
+                                                                const double* __restrict__ s, int64_t n4i,
+                                                                double* __restrict__ partial, int with_y) {
+    constexpr int E = PAIRS<NV>;
+    __shared__ double ck[NV > 0 ? NV : 1], yk[NV > 0 ? NV : 1];
+    if ((int)threadIdx.x < NV) {
+        ck[threadIdx.x] = cy[threadIdx.x];
+        yk[threadIdx.x] = cy[MAXV + threadIdx.x];
     }
-    double out[2 * NG];
+    __syncthreads();
+    GroupSums<NG> gu, gv;
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
+    const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
+    for (int64_t i = i0; i < n2; i += E * stride) {
+        double2 zk[E][NV > 0 ? NV : 1], w[E];
 #pragma unroll
-    for (int k = 0; k < 2 * NG; ++k) out[k] = 0.0;
-    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool phi = (i0 & 3) == 3;   // the grid stride is a multiple of 4
-    for (int64_t i = i0; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        double u = 0.0, v = 0.0;
-        if (with_y) {
+        for (int e = 0; e < E; ++e) {
+            const bool in = e == 0 || i + e * stride < n2;
+            w[e] = in ? ld2(s, i + e * stride) : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) zk[e][k] = in ? ld2(Z + k * ldz, i + e * stride) : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (e > 0 && i + e * stride >= n2) break;
+            double2 u = make_double2(0.0, 0.0);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
-                const double zk = Z[k * ldz + i];
-                u += ck[k] * zk;
-                v += yk[k] * zk;
+                u.x += ck[k] * zk[e][k].x;
+                u.y += ck[k] * zk[e][k].y;
             }
-        } else {
+            gu.add(i + e * stride, n4i, u.x * w[e].x, u.y * w[e].y);
+            if (with_y) {
+                double2 v = make_double2(0.0, 0.0);
 #pragma unroll
-            for (int k = 0; k < NV; ++k) u += ck[k] * Z[k * ldz + i];
-        }
-        const double w = s[i];
-        u *= w;
-        v *= w;
-        const int grp = phi ? ((NG == 3 && i >= n4i) ? 2 : 1) : 0;
-#pragma unroll
-        for (int q = 0; q < NG; ++q) {
-            if (grp == q) {
-                out[q] += u * u;
-                out[NG + q] += v * v;
+                for (int k = 0; k < NV; ++k) {
+                    v.x += yk[k] * zk[e][k].x;
+                    v.y += yk[k] * zk[e][k].y;
+                }
+                gv.add(i + e * stride, n4i, v.x * w[e].x, v.y * w[e].y);
             }
         }
     }
+    double out[2 * NG];
+    gu.get((i0 & 1) != 0, out);
+    gv.get((i0 & 1) != 0, out + NG);
     block_reduce_store<2 * NG>(out, partial);
 }
 
-// w' = w - sum_k h[k] V_k (in place); partial sums of <V_k, w'> and <w', w'>. h holds the first
-// pass's dots and, at h[NV], <w, w>. When the first pass kept at least REORTH_KEEP of w's squared
-// norm (|w'|^2 = <w,w> - |h|^2 >= REORTH_KEEP <w,w>), w' is orthogonal to the basis to about
-// eps / sqrt(REORTH_KEEP) and the second pass is skipped: only <w', w'> is formed, the dots stay
-// zero, and k_orth_final then just normalises. This is the Daniel-Gragg-Kaufman-Stewart test with
-// a looser threshold than its usual 1/2: on the FGMRES workloads here the first pass keeps
-// 8-20% of |w|^2, the second pass found nothing to remove in 85-99% of the steps, and FP64 issue
-// (not bandwidth) bounds these kernels on GB300.
+// w' = w - sum_k h[k] V_k (in place), h the sums of the first pass's partial dots (pdots); partial sums
+// of <V_k, w'> and <w', w'>. Block 0 stores h to dots and the flag below to dots[SECOND_OFF]. When the
+// first pass kept at least REORTH_KEEP of w's squared norm (|w'|^2 = <w,w> - |h|^2 >= REORTH_KEEP
+// <w,w>), w' is orthogonal to the basis to about eps / sqrt(REORTH_KEEP) and the second pass is
+// skipped: only <w', w'> is formed, and k_orth_final then just normalises. This is the
+// Daniel-Gragg-Kaufman-Stewart test with a looser threshold than its usual 1/2: on the FGMRES
+// workloads here the first pass keeps 8-20% of |w|^2, the second pass found nothing to remove in
+// 85-99% of the steps, and FP64 issue (not bandwidth) bounds these kernels on GB300.
 constexpr double REORTH_KEEP = 1e-4;
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS) k_orth_update_dot(int64_t n4, const double* __restrict__ V, int64_t ldv,
-                                                                 const double* __restrict__ h, double* __restrict__ w,
-                                                                 double* __restrict__ partial) {
-    double acc[NV + 1], hk[NV > 0 ? NV : 1];
-    double hh = 0.0;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        hk[k] = h[k];
-        hh += hk[k] * hk[k];
+__global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, const double* __restrict__ V,
+                                                                    int64_t ldv, const double* __restrict__ pdots,
+                                                                    int nblocks, double* __restrict__ dots,
+                                                                    double* __restrict__ w,
+                                                                    double* __restrict__ partial) {
+    constexpr int E = PAIRS<NV>;
+    __shared__ double h[NV + 1];
+    __shared__ int second_s;
+    sum_partials(pdots, nblocks, NV + 1, h);
+    if (threadIdx.x == 0) {
+        double hh = 0.0;
+        for (int k = 0; k < NV; ++k) hh += h[k] * h[k];
+        second_s = h[NV] - hh < REORTH_KEEP * h[NV];
+        if (blockIdx.x == 0) dots[SECOND_OFF] = second_s ? 1.0 : 0.0;
     }
-    const double ww = h[NV];
-    const bool second = ww - hh < REORTH_KEEP * ww;
+    if (blockIdx.x == 0 && threadIdx.x <= NV) dots[threadIdx.x] = h[threadIdx.x];
+    __syncthreads();
+    const bool second = second_s != 0;
+    double hk[NV > 0 ? NV : 1];
 #pragma unroll
-    for (int k = 0; k <= NV; ++k) acc[k] = 0.0;
+    for (int k = 0; k < NV; ++k) hk[k] = h[k];
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
+    const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
     if (second) {
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-            double vk[NV > 0 ? NV : 1];
-            double wi = w[i];
+        double acc[NV + 1];
+#pragma unroll
+        for (int k = 0; k <= NV; ++k) acc[k] = 0.0;
+        for (int64_t i = i0; i < n2; i += stride) {
+            double2 vk[NV > 0 ? NV : 1];
+            double2 wi = ld2(w, i);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
-                vk[k] = V[k * ldv + i];
-                wi -= hk[k] * vk[k];
+                vk[k] = ld2(V + k * ldv, i);
+                wi.x -= hk[k] * vk[k].x;
+                wi.y -= hk[k] * vk[k].y;
             }
-            w[i] = wi;
+            st2(w, i, wi);
 #pragma unroll
-            for (int k = 0; k < NV; ++k) acc[k] += vk[k] * wi;
-            acc[NV] += wi * wi;
+            for (int k = 0; k < NV; ++k) {
+                acc[k] += vk[k].x * wi.x;
+                acc[k] += vk[k].y * wi.y;
+            }
+            acc[NV] += wi.x * wi.x;
+            acc[NV] += wi.y * wi.y;
         }
+        block_reduce_store<NV + 1>(acc, partial);
     } else {
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-            double wi = w[i];
+        double acc[1] = {0.0};
+        for (int64_t i = i0; i < n2; i += E * stride) {
+            double2 wi[E], vk[E][NV > 0 ? NV : 1];
 #pragma unroll
-            for (int k = 0; k < NV; ++k) wi -= hk[k] * V[k * ldv + i];
-            w[i] = wi;
-            acc[NV] += wi * wi;
+            for (int e = 0; e < E; ++e) {
+                const bool in = e == 0 || i + e * stride < n2;
+                wi[e] = in ? ld2(w, i + e * stride) : make_double2(0.0, 0.0);
+#pragma unroll
+                for (int k = 0; k < NV; ++k)
+                    vk[e][k] = in ? ld2(V + k * ldv, i + e * stride) : make_double2(0.0, 0.0);
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (e > 0 && i + e * stride >= n2) break;
+#pragma unroll
+                for (int k = 0; k < NV; ++k) {
+                    wi[e].x -= hk[k] * vk[e][k].x;
+                    wi[e].y -= hk[k] * vk[e][k].y;
+                }
+                st2(w, i + e * stride, wi[e]);
+                acc[0] += wi[e].x * wi[e].x;
+                acc[0] += wi[e].y * wi[e].y;
+            }
         }
+        block_reduce_store<1>(acc, partial + NV * PART_LD);
     }
-    block_reduce_store<NV + 1>(acc, partial);
 }
 
-// v_{j+1} = (w' - sum_k h2[k] V_k) / eta with eta^2 = <w',w'> - |h2|^2 (in place). When the second
+// v_{j+1} = (w' - sum_k h2[k] V_k) / eta with eta^2 = <w',w'> - |h2|^2 (in place), h2 the sums of the
+// second pass's partial dots (pdots; only <w', w'> without a second pass). When the second
 // Gram-Schmidt pass found nothing to remove (|h2| <= ORTH_SKIP * |w'|), the subtraction is skipped,
 // V is not read, eta = |w'|, and flag[0] = 1 tells the host to keep h1 alone in the Hessenberg column.
+// Block 0 stores h2 to dots2.
 constexpr double ORTH_SKIP = 1e-10;
 template <int NV>
 __global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const double* __restrict__ V, int64_t ldv,
-                                                            const double* __restrict__ h2, double* __restrict__ w,
+                                                            const double* __restrict__ pdots, int nblocks,
+                                                            const double* __restrict__ second,
+                                                            double* __restrict__ dots2, double* __restrict__ w,
                                                             double* __restrict__ flag) {
-    double hk[NV > 0 ? NV : 1];
-    double hh = 0.0;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        hk[k] = h2[k];
-        hh += hk[k] * hk[k];
+    __shared__ double h2[NV + 1];
+    __shared__ double inv_s;
+    __shared__ int skip_s;
+    if (second[0] != 0.0) {
+        sum_partials(pdots, nblocks, NV + 1, h2);
+    } else {
+        if ((int)threadIdx.x < NV) h2[threadIdx.x] = 0.0;
+        sum_partials(pdots + NV * PART_LD, nblocks, 1, h2 + NV);
     }
-    const double s2 = h2[NV];
-    const bool skip = hh <= ORTH_SKIP * ORTH_SKIP * s2;
-    const double e2 = skip ? s2 : s2 - hh;
-    const double inv_eta = e2 > 0 ? 1.0 / sqrt(e2) : 0.0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) flag[0] = skip ? 1.0 : 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        double wi = w[i];
-        if (!skip) {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) wi -= hk[k] * V[k * ldv + i];
+    if (threadIdx.x == 0) {
+        const double s2 = h2[NV];
+        double hh = 0.0;
+        if (second[0] != 0.0)
+            for (int k = 0; k < NV; ++k) hh += h2[k] * h2[k];
+        const bool skip = hh <= ORTH_SKIP * ORTH_SKIP * s2;
+        const double e2 = skip ? s2 : s2 - hh;
+        inv_s = e2 > 0 ? rsqrt(e2) : 0.0;
+        skip_s = skip;
+        if (blockIdx.x == 0) flag[0] = skip ? 1.0 : 0.0;
+    }
+    if (blockIdx.x == 0 && threadIdx.x <= NV) dots2[threadIdx.x] = h2[threadIdx.x];
+    __syncthreads();
+    const double inv_eta = inv_s;
+    const bool skip = skip_s != 0;
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
+    const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
+    if (skip) {
+        for (int64_t i = i0; i < n2; i += 2 * stride) {
+            const bool two = i + stride < n2;
+            double2 a = ld2(w, i), b = two ? ld2(w, i + stride) : a;
+            st2(w, i, make_double2(a.x * inv_eta, a.y * inv_eta));
+            if (two) st2(w, i + stride, make_double2(b.x * inv_eta, b.y * inv_eta));
         }
-        w[i] = wi * inv_eta;
+    } else {
+        for (int64_t i = i0; i < n2; i += stride) {
+            double2 wi = ld2(w, i);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const double2 vk = ld2(V + k * ldv, i);
+                wi.x -= h2[k] * vk.x;
+                wi.y -= h2[k] * vk.y;
+            }
+            st2(w, i, make_double2(wi.x * inv_eta, wi.y * inv_eta));
+        }
     }
 }
 
-// out[k] = sum_b partial[b][k]
-__global__ void k_reduce(const double* __restrict__ partial, int nblocks, int nv, double* __restrict__ out) {
-    int k = blockIdx.x;
-    if (k >= nv) return;
-    double s = 0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += partial[(int64_t)b * MAXW + k];
-    __shared__ double sh[256];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[k] = sh[0];
+// out[k] = sum over blocks of partial[k * PART_LD + b] (one block)
+__global__ void __launch_bounds__(RED_THREADS) k_reduce(const double* __restrict__ partial, int nblocks, int nv,
+                                                        double* __restrict__ out) {
+    __shared__ double sh[MAXW];
+    sum_partials(partial, nblocks, nv, sh);
+    if (threadIdx.x < nv) out[threadIdx.x] = sh[threadIdx.x];
 }
 
 // x += sum_k y[k] Z_k
@@ -304,58 +432,40 @@ __global__ void __launch_bounds__(RED_THREADS) k_update_x(int64_t n4, const doub
     double yk[NZ > 0 ? NZ : 1];
 #pragma unroll
     for (int k = 0; k < NZ; ++k) yk[k] = y[k];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        double s = x[i];
+    const int64_t n2 = n4 / 2;
+    for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n2; i += (int64_t)gridDim.x * RED_THREADS) {
+        double2 s = ld2(x, i);
 #pragma unroll
-        for (int k = 0; k < NZ; ++k) s += yk[k] * Z[k * ldz + i];
-        x[i] = s;
+        for (int k = 0; k < NZ; ++k) {
+            const double2 z = ld2(Z + k * ldz, i);
+            s.x += yk[k] * z.x;
+            s.y += yk[k] * z.y;
+        }
+        st2(x, i, s);
     }
 }
 
-// Blocks of a grid-stride reduction kernel: one full wave, i.e. the blocks that are resident at
-// once given this kernel's registers (from the occupancy calculator), at most RED_BLOCKS. A fixed
-// grid that is not a multiple of the resident blocks leaves a partly filled last wave that costs
-// as much as a full one (3 resident blocks per SM and 608 blocks ran these kernels 2x slower).
-int red_grid(const void* fn) {
-    static std::mutex mu;
-    static std::unordered_map<const void*, int> cache;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find(fn);
-    if (it != cache.end()) return it->second;
-    int dev = 0, sms = 0, per_sm = 0;
-    KNP_CUDA(cudaGetDevice(&dev));
-    KNP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    KNP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, RED_THREADS, 0));
-    const int g = std::max(1, std::min(RED_BLOCKS, per_sm * sms));
-    cache.emplace(fn, g);
-    return g;
+// Blocks of a reduction kernel: one per SM, fewer when a block's threads would not have two pairs each.
+// (Partial sums of more blocks cost more in the next kernel's prologue than the added warps gain.)
+int red_grid(int64_t n4) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (n4 + 4 * RED_THREADS - 1) / (4 * RED_THREADS)));
+}
+// Blocks of a kernel that leaves no partial sums: two pairs per thread, up to four blocks per SM
+unsigned vec_grid(int64_t n4) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(608, (n4 + 4 * RED_THREADS - 1) / (4 * RED_THREADS)));
 }
 
 #define KNP_NV_CASES(X) \
     X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16) X(17) X(18) X(19) \
     X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30) X(31)
 
-#define KNP_NV_CASE_k_mdot(N) \
-    case N: nb_red = red_grid((const void*)&k_mdot<N>); k_mdot<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_mdot_split2(N) \
-    case N: nb_red = red_grid((const void*)&k_mdot_split<N, 2>); k_mdot_split<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_mdot_split3(N) \
-    case N: nb_red = red_grid((const void*)&k_mdot_split<N, 3>); k_mdot_split<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_combo_norms2(N) \
-    case N: nb_red = red_grid((const void*)&k_combo_norms<N, 2>); k_combo_norms<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_combo_norms3(N) \
-    case N: nb_red = red_grid((const void*)&k_combo_norms<N, 3>); k_combo_norms<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_orth_update_dot(N)                                                        \
-    case N:                                                                                     \
-        nb_red = red_grid((const void*)&k_orth_update_dot<N>);                                  \
-        k_orth_update_dot<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS);                         \
-        break;
-#define KNP_NV_CASE_k_orth_final(N) \
-    case N: nb_red = red_grid((const void*)&k_orth_final<N>); k_orth_final<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_update_x(N) \
-    case N: nb_red = red_grid((const void*)&k_update_x<N>); k_update_x<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-// Launch KERNEL<nv><<<nb_red, RED_THREADS, 0, st>>>(args) for a runtime nv in [0, 31]; nb_red
-// (a variable of the caller) receives the grid, which the following k_reduce sums over
+#define KNP_NV_CASE_k_mdot(N) case N: k_mdot<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_combo_norms2(N) case N: k_combo_norms<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_combo_norms3(N) case N: k_combo_norms<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_update_dot(N) case N: k_orth_update_dot<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_final(N) case N: k_orth_final<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_update_x(N) case N: k_update_x<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+// Launch KERNEL<nv> with the caller's grid (nb_red or nb_vec) for a runtime nv in [0, 31]
 #define KNP_LAUNCH_NV(nv, KERNEL)                                                                    \
     do {                                                                                             \
         switch (nv) {                                                                                \
@@ -388,6 +498,10 @@ struct GmresWork {
     // reductions, the copy of the dots to hh) as a CUDA graph per (j, transposed)
     std::map<std::pair<int, bool>, cudaGraphExec_t> arnoldi;
     cudaStream_t cap = nullptr;     // capture stream (the problem's stream may be the legacy one)
+    // partial sums: of an Arnoldi step's two passes, each read by the kernel after it, and the others'
+    double* pass1() { return partial.p; }
+    double* pass2() { return partial.p + MAXW * PART_LD; }
+    double* other() { return partial.p + 2 * MAXW * PART_LD; }
     ~GmresWork() {
         for (auto& kv : arnoldi) cudaGraphExecDestroy(kv.second);
         if (cap) cudaStreamDestroy(cap);
@@ -405,7 +519,7 @@ GmresWork* gmres_work(knp_problem* p, int restart) {
     g->n4 = 4 * p->n_nodes;
     g->V.alloc((restart + 1) * g->n4);
     g->Z.alloc((restart + 1) * g->n4);
-    g->partial.alloc(RED_BLOCKS * MAXW);
+    g->partial.alloc(3 * MAXW * PART_LD);   // first pass, second pass, everything else
     g->dots.alloc(DOTS_LEN);
     g->y.alloc(MAXV);
     g->cy.alloc(2 * MAXV);
@@ -421,9 +535,9 @@ void gmres_free(GmresWork* g) { delete g; }
 // squared norm of a device vector (through the multi-dot kernels)
 static double norm2_dev(GmresWork& g, const double* v, cudaStream_t st) {
     count_launch(2);
-    const int nb = red_grid((const void*)&k_mdot<0>);
-    k_mdot<0><<<nb, RED_THREADS, 0, st>>>(g.n4, nullptr, 0, v, g.partial.p);
-    k_reduce<<<1, 256, 0, st>>>(g.partial.p, nb, 1, g.dots.p);
+    const int nb = red_grid(g.n4);
+    k_mdot<0><<<nb, RED_THREADS, 0, st>>>(g.n4, nullptr, 0, v, g.other());
+    k_reduce<<<1, RED_THREADS, 0, st>>>(g.other(), nb, 1, g.dots.p);
     double s;
     KNP_CUDA(cudaMemcpyAsync(&s, g.dots.p, sizeof(double), cudaMemcpyDeviceToHost, st));
     KNP_CUDA(cudaStreamSynchronize(st));
@@ -435,21 +549,20 @@ static double norm2_dev(GmresWork& g, const double* v, cudaStream_t st) {
 static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, cudaStream_t st) {
     const int64_t n4 = g.n4;
     const int nv = j + 1;
-    int nb_red = RED_BLOCKS;
+    const int nb_red = red_grid(n4);
+    const unsigned nb_vec = vec_grid(n4);
     double* zj = g.Z.p + (int64_t)j * n4;
     double* w = g.V.p + (int64_t)(j + 1) * n4;
     op_apply(p, zj, w, p->sinv.p, nullptr, transpose, st);
     ProfScope ps(&p->prof, KC_ORTHO, st);
-    count_launch(5);
-#define KNP_ARGS n4, g.V.p, n4, w, g.partial.p
+    count_launch(3);
+#define KNP_ARGS n4, g.V.p, n4, w, g.pass1()
     KNP_LAUNCH_NV(nv, k_mdot);
 #undef KNP_ARGS
-    k_reduce<<<nv + 1, 256, 0, st>>>(g.partial.p, nb_red, nv + 1, g.dots.p);
-#define KNP_ARGS n4, g.V.p, n4, g.dots.p, w, g.partial.p
+#define KNP_ARGS n4, g.V.p, n4, g.pass1(), nb_red, g.dots.p, w, g.pass2()
     KNP_LAUNCH_NV(nv, k_orth_update_dot);
 #undef KNP_ARGS
-    k_reduce<<<nv + 1, 256, 0, st>>>(g.partial.p, nb_red, nv + 1, g.dots.p + MAXV);
-#define KNP_ARGS n4, g.V.p, n4, g.dots.p + MAXV, w, g.dots.p + 2 * MAXV + MAXW
+#define KNP_ARGS n4, g.V.p, n4, g.pass2(), nb_red, g.dots.p + SECOND_OFF, g.dots.p + MAXV, w, g.dots.p + 2 * MAXV + MAXW
     KNP_LAUNCH_NV(nv, k_orth_final);
 #undef KNP_ARGS
     KNP_CUDA(cudaGetLastError());
@@ -483,7 +596,7 @@ static void arnoldi_graph_launch(knp_problem* p, GmresWork& g, int j, bool trans
         it = g.arnoldi.emplace(key, ex).first;
     }
     KNP_CUDA(cudaGraphLaunch(it->second, p->stream));
-    count_launch(6);
+    count_launch(4);
 }
 
 knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stats& stats, double* x,
@@ -518,7 +631,8 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
         KNP_CUDA(cudaStreamSynchronize(st));
     }
     const double* wts = paper_test ? g.ones.p : p->swt.p;
-    int nb_red = RED_BLOCKS;   // grid of the last reduction kernel (KNP_LAUNCH_NV sets it)
+    const int nb_red = red_grid(n4);
+    const unsigned nb_vec = vec_grid(n4);
     // Arnoldi steps from CUDA graphs, unless a kernel class is being profiled (event pairs go
     // around single launches) or graphs are switched off for the V-cycle as well
     const bool use_graphs = p->amg->use_graphs && p->prof.active < 0;
@@ -532,15 +646,11 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
             return;
         }
         count_launch(2);
-        int nb = 0;
-        if (NG == 3) {
-            nb = red_grid((const void*)&k_mdot_split<0, 3>);
-            k_mdot_split<0, 3><<<nb, RED_THREADS, 0, st>>>(n4, nullptr, 0, x, p->swt.p, n4i, g.partial.p);
-        } else {
-            nb = red_grid((const void*)&k_mdot_split<0, 2>);
-            k_mdot_split<0, 2><<<nb, RED_THREADS, 0, st>>>(n4, nullptr, 0, x, p->swt.p, n4i, g.partial.p);
-        }
-        k_reduce<<<NG, 256, 0, st>>>(g.partial.p, nb, NG, g.dots.p + 2 * MAXV);
+        if (NG == 3)
+            k_group_norms<3><<<nb_red, RED_THREADS, 0, st>>>(n4, x, p->swt.p, n4i, g.other());
+        else
+            k_group_norms<2><<<nb_red, RED_THREADS, 0, st>>>(n4, x, p->swt.p, n4i, g.other());
+        k_reduce<<<1, RED_THREADS, 0, st>>>(g.other(), nb_red, NG, g.dots.p + 2 * MAXV);
         double xn2[3] = {0, 0, 0};
         KNP_CUDA(cudaMemcpyAsync(xn2, g.dots.p + 2 * MAXV, NG * sizeof(double), cudaMemcpyDeviceToHost, st));
         KNP_CUDA(cudaStreamSynchronize(st));
@@ -635,13 +745,13 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
                 // for every realistic step, so Z y is formed only in the first case
                 bool with_y = false;
                 for (int q = 0; q < NG; ++q) with_y |= tol[q] == 0.0;
-#define KNP_ARGS n4, g.Z.p, n4, g.cy.p, wts, n4i, g.partial.p, (int)with_y
+#define KNP_ARGS n4, g.Z.p, n4, g.cy.p, wts, n4i, g.other(), (int)with_y
                 if (NG == 3)
                     KNP_LAUNCH_NV(j + 1, k_combo_norms3);
                 else
                     KNP_LAUNCH_NV(j + 1, k_combo_norms2);
 #undef KNP_ARGS
-                k_reduce<<<2 * NG, 256, 0, st>>>(g.partial.p, nb_red, 2 * NG, g.dots.p + CHK_OFF);
+                k_reduce<<<1, RED_THREADS, 0, st>>>(g.other(), nb_red, 2 * NG, g.dots.p + CHK_OFF);
             }
             const int nv = j + 1;
             if (arnoldi && use_graphs) {
