@@ -5,12 +5,10 @@
 // mixed-precision form; the coarsest dense solve is FP64 in both).
 //
 // Layouts: a level operator with short rows (the finest, about 15 entries per row in 3D) or
-// with enough rows to fill the GPU one thread per row is sliced-ELL with one thread per row;
-// the other operators and the transfer operators are CSR processed by groups of 4 x S threads
-// per row, one thread per (field, entry slot): each thread does one multiply-add per entry and
-// the group reduces one value per field over its S slots (S a power of two chosen from the mean
-// row length), so that the short, wide coarse levels still fill the GPU without spending the
-// slow FP64 pipe on four-value reductions.
+// with enough rows to fill the GPU one thread per row is sliced-ELL; the other operators and the
+// restriction are CSR with 4 to 128 lanes per row; the prolongation is sliced-ELL over rows sorted by
+// length. A lane always works on all four fields of an entry, so that the sums over a row's lanes can be
+// a reduce-scatter and no lane of the slow FP64 pipe idles.
 //
 // Smoothing: Chebyshev steps on [lambda_max / ratio, 1.1 lambda_max] per field, `pre` of them
 // before the coarse-grid correction (the first from x = 0 costs no operator product) and
@@ -134,35 +132,55 @@ __device__ __forceinline__ void sell_row(int64_t r, int t, const int64_t* __rest
     }
 }
 
-// Field f of a CSR row product, by a group of 4 x S lanes (lane = 4 x slot + f): slot k takes
-// entries k, k + S, ... of the row, and the S partial sums of each field are combined by
-// shuffles (and, for S > 8, across the row's warps through shared memory); every lane of the
-// group gets its field's sum. Blocks are 128 threads. Every thread of the block must call this
-// (full-mask shuffles, and a block barrier for S > 8); rows r >= n pass active = false and
-// contribute nothing.
-template <class T, int S>
-__device__ __forceinline__ T csr_row_field(bool active, int64_t r, int slot, int f, const int64_t* __restrict__ ptr,
+// Field t of a CSR row product by L lanes (t < L; lanes t < 4 of the row get the sum of field t): lane t
+// takes entries t, t + L, ... with all four fields of each, CSR_BATCH<L> entries' loads in flight. Up to 32
+// lanes are consecutive lanes of a warp; 128 lanes are the block, whose warps combine through shared
+// memory. Blocks are 128 threads. Every thread of the block must call this (full-mask shuffles, and a
+// block barrier for L = 128); rows r >= n pass active = false and contribute nothing.
+// An FP64 instruction occupies the SM for 16 cycles whether 4 or 32 of its lanes do work. With all
+// fields of an entry in one lane a row of n entries takes 4 ceil(n / L) instructions of 32 / L rows and
+// 3 (L = 4) to 6 (L = 32) for the sums; one lane per field and entry slot took as many for a row's
+// products and log2(slots) sums per row of half as many rows (64^3 FP64, 25,578 rows of 60 entries:
+// Chebyshev step 26.6 -> 22.4 us; restriction to 235 rows of 600 entries 17.3 -> 8.3 us with a block
+// per row).
+template <int L>
+constexpr int CSR_BATCH = L == 4 ? 2 : 4;   // many rows: registers for more blocks instead
+template <class T, int L>
+__device__ __forceinline__ T csr_row_field(bool active, int64_t r, int t, const int64_t* __restrict__ ptr,
                                            const int32_t* __restrict__ col, const T* __restrict__ val,
                                            const T* __restrict__ x) {
-    static_assert(S >= 1 && S <= 32 && (S & (S - 1)) == 0, "slots: a power of two up to 32");
-    T acc = T(0);
+    static_assert(L == 4 || L == 8 || L == 16 || L == 32 || L == 128, "lanes per row");
+    constexpr int U = CSR_BATCH<L>;
+    T acc[4] = {T(0), T(0), T(0), T(0)}, out[1];
     if (active) {
         const int64_t t1 = ptr[r + 1];
-        for (int64_t t = ptr[r] + slot; t < t1; t += S) acc += val[4 * t + f] * x[4 * (int64_t)col[t] + f];
+        for (int64_t q = ptr[r] + t; q < t1; q += U * L) {
+            int32_t c[U];
+            V4<T> a[U], xv[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (q + u * L < t1) {
+                    c[u] = col[q + u * L];
+                    a[u] = V4<T>::load(val + 4 * (q + u * L));
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (q + u * L < t1) xv[u] = V4<T>::load(x + 4 * (int64_t)c[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (q + u * L < t1)
+                    for (int f = 0; f < 4; ++f) acc[f] += a[u].v[f] * xv[u].v[f];
+        }
     }
-    constexpr int SW = S < 8 ? S : 8;   // slots of the row inside one warp
-    for (int o = 2 * SW; o >= 4; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, 4 * SW);
-    if constexpr (S > 8) {
-        constexpr int NW = S / 8;   // warps per row
-        __shared__ T part[4][4];    // [warp of the block][field]
-        const int w = threadIdx.x >> 5;
-        if ((threadIdx.x & 31) < 4) part[w][threadIdx.x & 31] = acc;
+    lane_reduce4<T, (L < 32 ? L : 32)>(acc, t, out);
+    if constexpr (L == 128) {
+        __shared__ T part[4][4];   // [warp][field]
+        if ((threadIdx.x & 31) < 4) part[threadIdx.x >> 5][threadIdx.x & 3] = out[0];
         __syncthreads();
-        const int w0 = w - w % NW;
-        acc = T(0);
-        for (int k = 0; k < NW; ++k) acc += part[w0 + k][f];
+        const int f = threadIdx.x & 3;
+        out[0] = (part[0][f] + part[1][f]) + (part[2][f] + part[3][f]);
     }
-    return acc;
+    return out[0];
 }
 
 // The coarse correction's input at node i: t = s .* v - (A Z y)_i. Row i of A Z y: its same-region
@@ -244,20 +262,19 @@ __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __r
     xx.store(x_out + k);
 }
 
-template <class T, int S>
+template <class T, int L>
 __global__ void __launch_bounds__(128) k_cheb_csr(int64_t n, const int64_t* __restrict__ ptr,
                                                   const int32_t* __restrict__ col, const T* __restrict__ val,
                                                   const T* __restrict__ x_in, const T* __restrict__ b,
                                                   const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
                                                   T* __restrict__ x_out, int read_d, int write_d) {
-    int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
-    int64_t i = g / (4 * S);
-    int lane = (int)(g % (4 * S)), f = lane & 3;
-    T acc = csr_row_field<T, S>(i < n, i, lane >> 2, f, ptr, col, val, x_in);
-    if (lane < 4 && i < n) {
-        const int64_t k = 4 * i + f;
-        T dd = (T)pick4(c.c2, f) * dinv[k] * (b[k] - acc);
-        if (read_d) dd = (T)pick4(c.c1, f) * d[k] + dd;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
+    const int t = (int)(g % L);
+    const T acc = csr_row_field<T, L>(i < n, i, t, ptr, col, val, x_in);
+    if (t < 4 && i < n) {
+        const int64_t k = 4 * i + t;
+        T dd = (T)pick4(c.c2, t) * dinv[k] * (b[k] - acc);
+        if (read_d) dd = (T)pick4(c.c1, t) * d[k] + dd;
         if (write_d) d[k] = dd;
         x_out[k] = x_in[k] + dd;
     }
@@ -289,30 +306,77 @@ __global__ void __launch_bounds__(128) k_resid_sell(int64_t n, const int64_t* __
     out.store(y + k);
 }
 
-template <class T, int S>
+template <class T, int L>
 __global__ void __launch_bounds__(128) k_resid_csr(int64_t n, const int64_t* __restrict__ ptr,
                                                    const int32_t* __restrict__ col, const T* __restrict__ val,
                                                    const T* __restrict__ x, const T* __restrict__ b,
                                                    T* __restrict__ r) {
-    int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
-    int64_t i = g / (4 * S);
-    int lane = (int)(g % (4 * S)), f = lane & 3;
-    T acc = csr_row_field<T, S>(i < n, i, lane >> 2, f, ptr, col, val, x);
-    if (lane < 4 && i < n) r[4 * i + f] = b[4 * i + f] - acc;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
+    const int t = (int)(g % L);
+    const T acc = csr_row_field<T, L>(i < n, i, t, ptr, col, val, x);
+    if (t < 4 && i < n) r[4 * i + t] = b[4 * i + t] - acc;
 }
 
-// y[i] (+)= (M x)[i] for a CSR with four values per entry (restriction and prolongation)
-template <class T, int S>
+// y = M x for a CSR with four values per entry (restriction)
+template <class T, int L>
 __global__ void __launch_bounds__(128) k_csr4(int64_t n, const int64_t* __restrict__ ptr,
                                               const int32_t* __restrict__ col, const T* __restrict__ val,
-                                              const T* __restrict__ x, T* __restrict__ y, int accumulate) {
-    int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
-    int64_t i = g / (4 * S);
-    int lane = (int)(g % (4 * S)), f = lane & 3;
-    T acc = csr_row_field<T, S>(i < n, i, lane >> 2, f, ptr, col, val, x);
-    if (lane < 4 && i < n) {
-        const int64_t k = 4 * i + f;
-        y[k] = accumulate ? y[k] + acc : acc;
+                                              const T* __restrict__ x, T* __restrict__ y) {
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
+    const int t = (int)(g % L);
+    const T acc = csr_row_field<T, L>(i < n, i, t, ptr, col, val, x);
+    if (t < 4 && i < n) y[4 * i + t] = acc;
+}
+
+// x += P xc, P sliced ELL whose rows are sorted by length within windows (perm: sorted row -> row).
+// One thread per row, or four (one per field) where that leaves too few threads: P's rows are short
+// (about 6 entries), so splitting them over lanes would cost more in sums than it gains.
+template <class T, int L>
+__global__ void __launch_bounds__(128) k_prolong(int64_t n, const int64_t* __restrict__ sp,
+                                                 const int32_t* __restrict__ col, const T* __restrict__ val,
+                                                 const int32_t* __restrict__ perm, const T* __restrict__ xc,
+                                                 T* __restrict__ x) {
+    static_assert(L == 1 || L == 4, "threads per row");
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t q = g / L;
+    if (q >= n) return;
+    const int64_t s = q / SELL_C, base = sp[s] + q % SELL_C;
+    const int w = (int)((sp[s + 1] - sp[s]) / SELL_C);
+    const int64_t r = perm[q];
+    if constexpr (L == 1) {
+        V4<T> acc = V4<T>::load(x + 4 * r);
+        for (int k0 = 0; k0 < w; k0 += 2) {
+            V4<T> a[2], v[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (k0 + u < w) {
+                    const int64_t pos = base + (k0 + u) * SELL_C;
+                    a[u] = V4<T>::load(val + 4 * pos);
+                    v[u] = V4<T>::load(xc + 4 * (int64_t)col[pos]);
+                }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (k0 + u < w)
+                    for (int f = 0; f < 4; ++f) acc.v[f] += a[u].v[f] * v[u].v[f];
+        }
+        acc.store(x + 4 * r);
+    } else {
+        const int f = (int)(g % L);
+        T acc = x[4 * r + f];
+        for (int k0 = 0; k0 < w; k0 += 4) {
+            T a[4], v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < w) {
+                    const int64_t pos = base + (k0 + u) * SELL_C;
+                    a[u] = val[4 * pos + f];
+                    v[u] = xc[4 * (int64_t)col[pos] + f];
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < w) acc += a[u] * v[u];
+        }
+        x[4 * r + f] = acc;
     }
 }
 
@@ -358,12 +422,14 @@ std::vector<T> cast_vec(const std::vector<double>& v) {
     return std::vector<T>(v.begin(), v.end());
 }
 
-// entry slots per row, a power of two up to 32 (4 x S threads per row): doubled while the grid
-// stays within about two waves of 152 SMs x 2048 threads and each slot keeps at least two entries
-int pick_slots(int64_t rows, double mean_len) {
-    int sl = 1;
-    while (sl < 32 && (double)rows * 4 * (2 * sl) <= 622592.0 && 4 * sl <= mean_len) sl *= 2;
-    return sl;
+// Lanes per row of the CSR kernels: 4, more (up to 32) while the grid stays below LANE_THREADS and a
+// lane keeps two entries of a mean row; a block of 128 for few, very long rows (the restriction to the
+// coarsest level: 235 rows of 600 entries at 64^3).
+int csr_lanes(int64_t rows, double mean_len) {
+    if (mean_len >= 256.0 && 128 * rows <= 2 * LANE_THREADS) return 128;
+    int l = 4;
+    while (l < 32 && 2 * l * rows <= LANE_THREADS && 4 * l <= mean_len) l *= 2;
+    return l;
 }
 
 }  // namespace
@@ -389,14 +455,15 @@ void take_values(DArray<T>& out, DArray<double>& in, int64_t count, cudaStream_t
 
 template <class T>
 struct DevCsr4 {
-    int64_t n = 0;
-    int slots = 1;
+    int64_t n = 0, nnz = 0;
+    int lanes = 4;
     DArray<int64_t> ptr;
     DArray<int32_t> col;
     DArray<T> val;
     void upload(const HostCsr4& h, cudaStream_t st) {
         n = h.n_rows;
-        slots = pick_slots(n, n ? (double)h.nnz() / (double)n : 1.0);
+        nnz = h.nnz();
+        lanes = csr_lanes(n, n ? (double)nnz / (double)n : 1.0);
         ptr.upload(h.ptr, st);
         col.upload(h.col, st);
         val.upload(cast_vec<T>(h.val), st);
@@ -404,10 +471,82 @@ struct DevCsr4 {
     // takes over a device CSR built by the GPU setup (no copy through the host)
     void take(DevCsr4d& d, cudaStream_t st) {
         n = d.n_rows;
-        slots = pick_slots(n, n ? (double)d.nnz / (double)n : 1.0);
+        nnz = d.nnz;
+        lanes = csr_lanes(n, n ? (double)nnz / (double)n : 1.0);
         ptr = std::move(d.ptr);
         col = std::move(d.col);
         take_values(val, d.val, 4 * d.nnz, st);
+    }
+};
+
+// The prolongation as k_prolong reads it: sliced ELL over rows sorted by length, longest first, within
+// windows of SORT_WINDOW rows. Unsorted, a warp runs as long as its longest row (P's rows have 1 to
+// some 20 entries, about 6 on average), in FP64 instructions as in padding read; sorted over 256 rows the
+// padding is a few percent and a window's writes still fall into the same lines (finest level at 64^3
+// FP64 30.8 -> 22 us, at 128^3 FP32 115 -> 60 us).
+constexpr int SORT_WINDOW = 256;
+
+__global__ void __launch_bounds__(SORT_WINDOW) k_sort_rows(int64_t n, const int64_t* __restrict__ ptr,
+                                                           int32_t* __restrict__ perm) {
+    __shared__ int64_t len[SORT_WINDOW];
+    const int64_t r = blockIdx.x * (int64_t)SORT_WINDOW + threadIdx.x;
+    const int64_t mine = r < n ? ptr[r + 1] - ptr[r] : -1;
+    len[threadIdx.x] = mine;
+    __syncthreads();
+    int rank = 0;
+    for (int q = 0; q < SORT_WINDOW; ++q) rank += len[q] > mine || (len[q] == mine && q < (int)threadIdx.x);
+    if (r < n) perm[blockIdx.x * (int64_t)SORT_WINDOW + rank] = (int32_t)r;
+}
+
+// entries of each slice of sorted rows: its first row is its longest
+__global__ void k_sorted_widths(int64_t n, int64_t ns, const int64_t* __restrict__ ptr,
+                                const int32_t* __restrict__ perm, int64_t* __restrict__ w) {
+    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (s >= ns) return;
+    const int64_t r = perm[s * SELL_C];
+    w[s] = (ptr[r + 1] - ptr[r]) * SELL_C;
+}
+
+// CSR -> sorted sliced ELL; padding has zero values and repeats the row's last column (0 in an empty row)
+template <class T>
+__global__ void k_sorted_fill(int64_t n, int64_t ns, const int64_t* __restrict__ ptr, const int32_t* __restrict__ col,
+                              const T* __restrict__ val, const int32_t* __restrict__ perm,
+                              const int64_t* __restrict__ sp, int32_t* __restrict__ scol, T* __restrict__ sval) {
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= ns * SELL_C) return;
+    const int64_t s = q / SELL_C, w = (sp[s + 1] - sp[s]) / SELL_C;
+    const int64_t r = q < n ? perm[q] : -1;
+    const int64_t len = r >= 0 ? ptr[r + 1] - ptr[r] : 0;
+    for (int64_t k = 0; k < w; ++k) {
+        const int64_t pos = sp[s] + q % SELL_C + k * SELL_C;
+        scol[pos] = len > 0 ? col[ptr[r] + min(k, len - 1)] : 0;
+        for (int f = 0; f < 4; ++f) sval[4 * pos + f] = k < len ? val[4 * (ptr[r] + k) + f] : T(0);
+    }
+}
+
+template <class T>
+struct DevProlong {
+    int64_t n = 0;
+    DArray<int64_t> sp;
+    DArray<int32_t> col, perm;
+    DArray<T> val;
+    // builds the sorted form of P (whose CSR arrays can be released afterwards)
+    void build(const DevCsr4<T>& P, cudaStream_t st) {
+        n = P.n;
+        if (!n) return;
+        const int64_t ns = (n + SELL_C - 1) / SELL_C;
+        perm.alloc(n);
+        k_sort_rows<<<nblk(n, SORT_WINDOW), SORT_WINDOW, 0, st>>>(n, P.ptr.p, perm.p);
+        DArray<int64_t> w;
+        w.alloc(ns);
+        k_sorted_widths<<<nblk(ns, 256), 256, 0, st>>>(n, ns, P.ptr.p, perm.p, w.p);
+        sp.alloc(ns + 1);
+        const int64_t total = device_exclusive_scan(w.p, sp.p, ns, st);
+        col.alloc(std::max<int64_t>(total, 1));
+        val.alloc(std::max<int64_t>(4 * total, 1));
+        k_sorted_fill<T><<<nblk(ns * SELL_C, 128), 128, 0, st>>>(n, ns, P.ptr.p, P.col.p, P.val.p, perm.p, sp.p, col.p,
+                                                                 val.p);
+        KNP_CUDA(cudaStreamSynchronize(st));
     }
 };
 
@@ -424,7 +563,8 @@ struct DevLevel {
     DevCsr4<T> A;
     DArray<T> dinv;
     double lmax[4], lmin[4];
-    DevCsr4<T> P, R;
+    DevProlong<T> P;
+    DevCsr4<T> R;
     DArray<T> x, x2, b, r, d;
 };
 
@@ -545,7 +685,9 @@ static void upload_hierarchy(AmgDev<T>& D, const HostHierarchy& H, int degree, i
             L->lmin[f] = HL.lmin[f];
         }
         if (HL.P.n_rows) {
-            L->P.upload(HL.P, st);
+            DevCsr4<T> P;
+            P.upload(HL.P, st);
+            L->P.build(P, st);
             L->R.upload(HL.R, st);
         }
         level_vectors_and_coefs(D, *L, std::max(degree, pre), st);
@@ -631,7 +773,9 @@ static void take_hierarchy(AmgDev<T>& D, GpuHierarchy& H, int degree, int pre, c
             L->lmin[f] = G->lmin[f];
         }
         if (G->P.n_rows) {
-            L->P.take(G->P, st);
+            DevCsr4<T> P;
+            P.take(G->P, st);
+            L->P.build(P, st);
             L->R.take(G->R, st);
         }
         level_vectors_and_coefs(D, *L, std::max(degree, pre), st);
@@ -689,14 +833,14 @@ void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, in
     KNP_CUDA(cudaStreamSynchronize(p->stream));
 }
 
-#define KNP_SLOT_DISPATCH(slots, KERNEL, grid_rows, ...)                                                   \
-    switch (slots) {                                                                                       \
-        case 1: KERNEL<T, 1><<<nblk((grid_rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;             \
-        case 2: KERNEL<T, 2><<<nblk((grid_rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;             \
-        case 4: KERNEL<T, 4><<<nblk((grid_rows) * 16, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
-        case 8: KERNEL<T, 8><<<nblk((grid_rows) * 32, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
-        case 16: KERNEL<T, 16><<<nblk((grid_rows) * 64, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
-        default: KERNEL<T, 32><<<nblk((grid_rows) * 128, 128), 128, 0, st>>>(__VA_ARGS__); break;         \
+// CSR kernels with the matrix's lanes per row
+#define KNP_CSR_DISPATCH(lanes, KERNEL, rows, ...)                                                \
+    switch (lanes) {                                                                              \
+        case 4: KERNEL<T, 4><<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
+        case 8: KERNEL<T, 8><<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
+        case 16: KERNEL<T, 16><<<nblk((rows) * 16, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
+        case 32: KERNEL<T, 32><<<nblk((rows) * 32, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
+        default: KERNEL<T, 128><<<nblk((rows) * 128, 128), 128, 0, st>>>(__VA_ARGS__); break;     \
     }
 
 // sliced-ELL kernels with the level's lanes per row
@@ -717,7 +861,7 @@ static void launch_cheb(const DevLevel<T>& L, const T* x_in, const T* b, const C
         KNP_LANE_DISPATCH(L.lanes, k_cheb_sell, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x_in, b, L.dinv.p, c, d, x_out,
                           read_d, write_d);
     } else {
-        KNP_SLOT_DISPATCH(L.A.slots, k_cheb_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x_in, b, L.dinv.p, c, d,
+        KNP_CSR_DISPATCH(L.A.lanes, k_cheb_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x_in, b, L.dinv.p, c, d,
                          x_out, read_d, write_d);
     }
 }
@@ -728,7 +872,7 @@ static void launch_resid(const DevLevel<T>& L, const T* x, const T* b, T* r, cud
     if (L.sell) {
         KNP_LANE_DISPATCH(L.lanes, k_resid_sell, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x, b, r);
     } else {
-        KNP_SLOT_DISPATCH(L.A.slots, k_resid_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x, b, r);
+        KNP_CSR_DISPATCH(L.A.lanes, k_resid_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x, b, r);
     }
 }
 
@@ -745,10 +889,21 @@ static void residual(DevLevel<T>& L, Profiler* pr, bool fine, cudaStream_t st) {
     launch_resid(L, L.x.p, L.b.p, L.r.p, st);
 }
 
+// rc = R r
 template <class T>
-static void csr_apply(DevCsr4<T>& M, const T* x, T* y, int accumulate, cudaStream_t st) {
+static void restrict_to(const DevCsr4<T>& R, const T* r, T* rc, cudaStream_t st) {
     count_launch();
-    KNP_SLOT_DISPATCH(M.slots, k_csr4, M.n, M.n, M.ptr.p, M.col.p, M.val.p, x, y, accumulate);
+    KNP_CSR_DISPATCH(R.lanes, k_csr4, R.n, R.n, R.ptr.p, R.col.p, R.val.p, r, rc);
+}
+
+// x += P xc
+template <class T>
+static void prolong(const DevProlong<T>& P, const T* xc, T* x, cudaStream_t st) {
+    count_launch();
+    if (P.n >= LANE_THREADS)
+        k_prolong<T, 1><<<nblk(P.n, 128), 128, 0, st>>>(P.n, P.sp.p, P.col.p, P.val.p, P.perm.p, xc, x);
+    else
+        k_prolong<T, 4><<<nblk(4 * P.n, 128), 128, 0, st>>>(P.n, P.sp.p, P.col.p, P.val.p, P.perm.p, xc, x);
 }
 
 template <class T>
@@ -783,9 +938,9 @@ static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, co
     DevLevel<T>& C = *D.L[l + 1];
     smooth(L, D.coef[l], D.pre, true, v, s, df, pr, l == 0, st);
     residual(L, pr, l == 0, st);
-    csr_apply(L.R, L.r.p, C.b.p, 0, st);
+    restrict_to(L.R, L.r.p, C.b.p, st);
     vcycle_rec(D, l + 1, nullptr, nullptr, DeflFuse{}, pr, st);
-    csr_apply(L.P, C.x.p, L.x.p, 1, st);
+    prolong(L.P, C.x.p, L.x.p, st);
     smooth(L, D.coef[l], D.degree, false, nullptr, nullptr, DeflFuse{}, pr, l == 0, st);
 }
 
@@ -970,11 +1125,9 @@ static void na_vcycle_rec(AmgDev<T>& D, std::vector<NaWork<T>>& W, int l, const 
                                                      D.pre > 1);
     for (int k = 1; k < D.pre; ++k) na_cheb_step(L, w, cs[k], k, D.pre, st);
     launch_resid(L, w.x, w.b, w.r, st);
-    count_launch();
-    KNP_SLOT_DISPATCH(L.R.slots, k_csr4, C.n, C.n, L.R.ptr.p, L.R.col.p, L.R.val.p, w.r, wc.b, 0);
+    restrict_to(L.R, w.r, wc.b, st);
     na_vcycle_rec(D, W, l + 1, nullptr, nullptr, st);
-    count_launch();
-    KNP_SLOT_DISPATCH(L.P.slots, k_csr4, L.n, L.n, L.P.ptr.p, L.P.col.p, L.P.val.p, wc.x, w.x, 1);
+    prolong(L.P, wc.x, w.x, st);
     for (int k = 0; k < D.degree; ++k) na_cheb_step(L, w, cs[k], k, D.degree, st);
 }
 
