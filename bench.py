@@ -246,13 +246,13 @@ def _source_parts(path, spans):
 
 def kernel_source_hash(kind="cheb_fine"):
     """Hash of a reported kernel's source text, so that DRAM counters taken on an older version of
-    it are not reported: "cheb_fine" (sell_row, cheb_update, k_cheb_sell) or "spmv" (k_op_apply)."""
+    it are not reported: "cheb_fine" (sell_row, k_cheb_sell) or "spmv" (k_op_apply)."""
     if kind == "spmv":
         return _source_parts("spmv.cu", (("// w[c] = sum_k z_k tau_r^k x^k[c]",
                                           "// g^k = m + tau_r^k a per stored entry"),))
-    return _source_parts("vcycle.cu", (("// Row product of a sliced-ELL operator", "// Field f of a CSR row product"),
-                                       ("// Chebyshev update of one row",
-                                        "template <class T, int S>\n__global__ void __launch_bounds__(128) k_cheb_csr")))
+    return _source_parts("vcycle.cu", (("// Row product of a sliced-ELL operator", "// Field t of a CSR row product"),
+                                       ("// Chebyshev step: r = b - A x_in",
+                                        "template <class T, int L>\n__global__ void __launch_bounds__(128) k_cheb_csr")))
 
 
 def fp64_peak_tflops(torch):
@@ -276,12 +276,13 @@ def fp64_peak_tflops(torch):
 
 def dominant_kernel_work(prob, precision):
     """Algorithmic bytes and FLOPs of one finest-level Chebyshev step (the V-cycle's largest kernel). Bytes: the operator once
-    (column index + four values per stored entry) and six node vectors of four values (x gathered,
-    b, D^-1, d read, d written, x written). FLOPs: 4 FMAs per stored entry and 20 per row."""
+    (column index + four values per stored entry) and five node vectors of four values (x gathered,
+    b, D^-1, x written, and d, which the first of the two steps writes and the second reads). FLOPs: 4
+    FMAs per stored entry and 20 per row."""
     info = prob.amg_info()
     n, nnz = info["nodes"][0], info["nnz"][0]
     t = 8 if precision == "fp64" else 4
-    return nnz * (4 + 4 * t) + n * 4 * t * 6, 8.0 * nnz + 20.0 * n
+    return nnz * (4 + 4 * t) + n * 4 * t * 5, 8.0 * nnz + 20.0 * n
 
 
 def spmv_work(prob):
