@@ -19,19 +19,23 @@
 // Z^T A^T Z = E^T.
 //
 // Costs. A applied to a piecewise-constant potential is nonzero only through the membrane and
-// pin terms: per row, the sum of its same-region e^k coefficients times the constant of its own
-// region, plus its cross-region entries times the constants of their cells. Those row sums are
-// formed once per step (RS, three values per node), E is an arrowhead matrix (cells couple only
-// to the extracellular space) solved by its Schur complement on the device, and each application
-// adds a gather and a small solve; the right-hand-side pass and the update run inside the
-// V-cycle's first and last kernels (the transposed form and CG(P_0) keep them as separate passes,
-// about 0.2 KB per node).
-// Sums are taken in a fixed order (no atomics), so the result is reproducible bit for bit.
+// pin terms: the same-region row sums of e^k (and of a) vanish except at the active rows, the membrane
+// nodes and the pinned node with its neighbours, since every assembled diagonal is minus its row's sum.
+// So A Z y is formed at the active rows alone (a few percent of the nodes): their row sums times the
+// constant of their own region, plus their cross-region entries times the constants of their cells.
+// The row sums are formed once per step (RS, three values per active row), E is an arrowhead matrix
+// (cells couple only to the extracellular space) solved by its Schur complement on the device, and each
+// application adds a gather and a small solve; the right-hand-side pass and the update run inside the
+// V-cycle's first and last kernels (CG(P_0) keeps them as separate passes).
+// Sums are taken in a fixed order (no atomics), so the result is reproducible bit for bit. They are
+// split into chunks of GATHER_NODES nodes, also within a cell: one block per cell took 37 us per
+// application and 546 us per step for the one cell of the 64^3 workload.
 #include <algorithm>
 #include <map>
 #include <vector>
 
 #include "deflate.h"
+#include "deflate_input.h"
 #include "problem.h"
 #include "vcycle.h"
 
@@ -39,8 +43,9 @@ namespace knp {
 
 namespace {
 
-constexpr int DT = 256;          // threads of the deflation kernels
-constexpr int EXT_BLOCKS = 304;  // partial-sum blocks over the extracellular nodes
+constexpr int DT = 256;              // threads of the deflation kernels
+constexpr int GATHER_NODES = 1024;   // nodes per block of the gather
+constexpr int EXT_BLOCKS = 304;      // most partial sums over the extracellular nodes
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -54,24 +59,26 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return s;   // valid in thread 0
 }
 
-// RS[r][k] = sum of the same-region e^k values of row r over phi columns other than the pin;
-// RSa[r] the same sum of the static stiffness a (for the transposed operator's concentration rows)
-__global__ void k_defl_rowsums(int64_t n, int32_t pin, const int64_t* __restrict__ slice_ptr,
-                               const int32_t* __restrict__ col, const double* __restrict__ e, int64_t ne,
-                               const double* __restrict__ a, double* __restrict__ RS, double* __restrict__ RSa) {
-    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= n) return;
+// RS[q][k] = sum of the same-region e^k values of active row q over phi columns other than the pin;
+// RSa[q] the same sum of the static stiffness a (for the transposed operator's concentration rows)
+__global__ void k_defl_rowsums(int64_t na, int32_t pin, const int32_t* __restrict__ rows,
+                               const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ col,
+                               const double* __restrict__ e, int64_t ne, const double* __restrict__ a,
+                               double* __restrict__ RS, double* __restrict__ RSa) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= na) return;
+    const int64_t r = rows[i];
     const int64_t s = r / SELL_C, base = slice_ptr[s] + r % SELL_C;
-    const int64_t w = (slice_ptr[s + 1] - slice_ptr[s]) / SELL_C;
+    const int w = (int)((slice_ptr[s + 1] - slice_ptr[s]) / SELL_C);
     double acc[KI] = {0, 0, 0}, sa = 0.0;
-    for (int64_t k = 0; k < w; ++k) {
+    for (int k = 0; k < w; ++k) {
         const int64_t pos = base + k * SELL_C;
         if (col[pos] == pin) continue;
         for (int q = 0; q < KI; ++q) acc[q] += e[q * ne + pos];
         sa += a[pos];
     }
-    for (int q = 0; q < KI; ++q) RS[3 * r + q] = acc[q];
-    RSa[r] = sa;
+    for (int q = 0; q < KI; ++q) RS[3 * i + q] = acc[q];
+    RSa[i] = sa;
 }
 
 // group of the source row of every transposed cross entry (-1: the pinned node)
@@ -83,171 +90,139 @@ __global__ void k_defl_xtg(int64_t nx, int64_t N_i, int32_t pin, const int32_t* 
     xtg[t] = j == pin ? -1 : (j < N_i ? rgrp[j] : ext_group);
 }
 
-// Per cell group j (one block): E_jj, E_je and E_ej of E = Z^T A Z. Potential-row coefficient of a
-// stored entry: sum_k z_k e^k (same region) or sum_k z_k xe^k (cross region).
-__global__ void __launch_bounds__(DT) k_defl_E_cells(const int64_t* __restrict__ cptr, const int32_t* __restrict__ cnodes,
-                                                     const double* __restrict__ RS, const int32_t* __restrict__ xptr,
-                                                     const int32_t* __restrict__ xg, const int32_t* __restrict__ xtptr,
-                                                     const int32_t* __restrict__ xtrow, const int32_t* __restrict__ xtidx,
-                                                     const double* __restrict__ xe, int64_t n_cross, int32_t pin,
-                                                     double z0, double z1, double z2, int32_t ext_group,
-                                                     double* __restrict__ Ejj, double* __restrict__ Eje,
-                                                     double* __restrict__ Eej) {
+// Chunk b of a cell group's active rows (one block): its share of E_jj, E_je and E_ej of E = Z^T A Z.
+// Potential-row coefficient of a stored entry: sum_k z_k e^k (same region) or sum_k z_k xe^k (cross
+// region). Blocks from nchunks on: one chunk each of the extracellular active rows' share of E_ee.
+__global__ void __launch_bounds__(DT) k_defl_E(int nchunks, const int64_t* __restrict__ cbeg,
+                                               const int32_t* __restrict__ aidx, int64_t ext0, int64_t na,
+                                               const int32_t* __restrict__ rows, const double* __restrict__ RS,
+                                               const int32_t* __restrict__ xptr, const int32_t* __restrict__ xg,
+                                               const int32_t* __restrict__ xtptr, const int32_t* __restrict__ xtrow,
+                                               const int32_t* __restrict__ xtidx, const double* __restrict__ xe,
+                                               int64_t n_cross, int32_t pin, double z0, double z1, double z2,
+                                               int32_t ext_group, double* __restrict__ part) {
     __shared__ double sh[DT / 32];
-    const int j = blockIdx.x;
+    const int b = blockIdx.x;
     double djj = 0.0, dje = 0.0, dej = 0.0;
-    for (int64_t q = cptr[j] + threadIdx.x; q < cptr[j + 1]; q += blockDim.x) {
-        const int64_t r = cnodes[q];
-        djj += z0 * RS[3 * r] + z1 * RS[3 * r + 1] + z2 * RS[3 * r + 2];
-        for (int t = xptr[r]; t < xptr[r + 1]; ++t)
-            if (xg[t] == ext_group)
-                dje += z0 * xe[t] + z1 * xe[n_cross + t] + z2 * xe[2 * n_cross + t];
-        // column r of the cross part: rows of the extracellular space (the pinned one left out)
-        for (int t = xtptr[r]; t < xtptr[r + 1]; ++t) {
-            if (xtrow[t] == pin) continue;
-            const int64_t idx = xtidx[t];
-            dej += z0 * xe[idx] + z1 * xe[n_cross + idx] + z2 * xe[2 * n_cross + idx];
+    if (b < nchunks) {
+        const int64_t q = cbeg[b] + threadIdx.x;
+        if (q < cbeg[b + 1]) {
+            const int64_t i = aidx[q], r = rows[i];
+            djj = z0 * RS[3 * i] + z1 * RS[3 * i + 1] + z2 * RS[3 * i + 2];
+            for (int t = xptr[r]; t < xptr[r + 1]; ++t)
+                if (xg[t] == ext_group) dje += z0 * xe[t] + z1 * xe[n_cross + t] + z2 * xe[2 * n_cross + t];
+            // column r of the cross part: rows of the extracellular space (the pinned one left out)
+            for (int t = xtptr[r]; t < xtptr[r + 1]; ++t) {
+                if (xtrow[t] == pin) continue;
+                const int64_t idx = xtidx[t];
+                dej += z0 * xe[idx] + z1 * xe[n_cross + idx] + z2 * xe[2 * n_cross + idx];
+            }
         }
+    } else {
+        const int64_t i = ext0 + (b - nchunks) * (int64_t)DT + threadIdx.x;
+        if (i < na && rows[i] != pin) djj = z0 * RS[3 * i] + z1 * RS[3 * i + 1] + z2 * RS[3 * i + 2];
     }
     double a = block_sum(djj, sh);
-    if (threadIdx.x == 0) Ejj[j] = a;
+    if (threadIdx.x == 0) part[3 * b] = a;
     a = block_sum(dje, sh);
-    if (threadIdx.x == 0) Eje[j] = a;
+    if (threadIdx.x == 0) part[3 * b + 1] = a;
     a = block_sum(dej, sh);
-    if (threadIdx.x == 0) Eej[j] = a;
+    if (threadIdx.x == 0) part[3 * b + 2] = a;
 }
 
-// partial sums of E_ee over the extracellular rows (the pinned one left out)
-__global__ void __launch_bounds__(DT) k_defl_E_ext(int64_t N_i, int64_t n, int32_t pin, const double* __restrict__ RS,
-                                                   double z0, double z1, double z2, double* __restrict__ part) {
-    __shared__ double sh[DT / 32];
-    double acc = 0.0;
-    for (int64_t r = N_i + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-        if (r != pin) acc += z0 * RS[3 * r] + z1 * RS[3 * r + 1] + z2 * RS[3 * r + 2];
-    const double s = block_sum(acc, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// E_ee and the Schur complement S_e = E_ee - sum_j E_ej E_je / E_jj (one block)
-__global__ void __launch_bounds__(DT) k_defl_schur(int nc, int nparts, const double* __restrict__ part,
-                                                   const double* __restrict__ Ejj, const double* __restrict__ Eje,
-                                                   const double* __restrict__ Eej, double* __restrict__ Ee) {
+// 1 / E_jj, E_je, E_ej of each group from its chunks' shares; E_ee and one over the Schur complement
+// S_e = E_ee - sum_j E_ej E_je / E_jj (one block)
+__global__ void __launch_bounds__(DT) k_defl_schur(int nc, int nchunks, int next, const int32_t* __restrict__ cchunk,
+                                                   const double* __restrict__ part, double* __restrict__ iEjj,
+                                                   double* __restrict__ Eje, double* __restrict__ Eej,
+                                                   double* __restrict__ Ee) {
     __shared__ double sh[DT / 32];
     double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < nparts; q += blockDim.x) a += part[q];
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) b += Eej[j] * Eje[j] / Ejj[j];
+    for (int q = threadIdx.x; q < next; q += blockDim.x) a += part[3 * (int64_t)(nchunks + q)];
+    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
+        double jj = 0.0, je = 0.0, ej = 0.0;
+        for (int64_t q = cchunk[j]; q < cchunk[j + 1]; ++q) {
+            jj += part[3 * q];
+            je += part[3 * q + 1];
+            ej += part[3 * q + 2];
+        }
+        iEjj[j] = 1.0 / jj;
+        Eje[j] = je;
+        Eej[j] = ej;
+        b += ej * je / jj;
+    }
     const double eee = block_sum(a, sh);
     const double red = block_sum(b, sh);
     if (threadIdx.x == 0) {
         Ee[0] = eee;
-        Ee[1] = eee - red;
+        Ee[1] = 1.0 / (eee - red);
     }
 }
 
-// g = Z^T r with r = s .* v: blocks [0, nc) sum the potentials of one cell each, blocks
-// [nc, nc + EXT_BLOCKS) partial sums over the extracellular potentials (pin left out)
-__global__ void __launch_bounds__(DT) k_defl_gather(int nc, const int64_t* __restrict__ cptr,
+// Partial sums of g = Z^T r with r = s .* v: blocks [0, nchunks) take one chunk of a cell's nodes each,
+// the others shares of the extracellular potentials (pin left out)
+__global__ void __launch_bounds__(DT) k_defl_gather(int nchunks, const int64_t* __restrict__ cbeg,
                                                     const int32_t* __restrict__ cnodes, int64_t N_i, int64_t n,
                                                     int32_t pin, const double* __restrict__ v,
-                                                    const double* __restrict__ s, double* __restrict__ g,
-                                                    double* __restrict__ part) {
+                                                    const double* __restrict__ s, double* __restrict__ part) {
     __shared__ double sh[DT / 32];
     double acc = 0.0;
-    if ((int)blockIdx.x < nc) {
-        const int j = blockIdx.x;
-        for (int64_t q = cptr[j] + threadIdx.x; q < cptr[j + 1]; q += blockDim.x) {
+    if ((int)blockIdx.x < nchunks) {
+        const int64_t end = cbeg[blockIdx.x + 1];
+        for (int64_t q = cbeg[blockIdx.x] + threadIdx.x; q < end; q += DT) {
             const int64_t i = 4 * (int64_t)cnodes[q] + 3;
             acc += s[i] * v[i];
         }
-        const double t = block_sum(acc, sh);
-        if (threadIdx.x == 0) g[j] = t;
     } else {
-        const int b = blockIdx.x - nc;
-        for (int64_t r = N_i + b * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)EXT_BLOCKS * blockDim.x)
+        const int64_t stride = (int64_t)(gridDim.x - nchunks) * DT;
+        for (int64_t r = N_i + (blockIdx.x - nchunks) * (int64_t)DT + threadIdx.x; r < n; r += stride)
             if (r != pin) acc += s[4 * r + 3] * v[4 * r + 3];
-        const double t = block_sum(acc, sh);
-        if (threadIdx.x == 0) part[b] = t;
     }
+    const double t = block_sum(acc, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
 // y = E^{-1} g for the arrowhead E (one block): y_e = (g_e - sum_j E_ej g_j / E_jj) / S_e,
-// y_j = (g_j - E_je y_e) / E_jj; y[nc] = y_e
-__global__ void __launch_bounds__(DT) k_defl_solve(int nc, const double* __restrict__ part, const double* __restrict__ g,
-                                                   const double* __restrict__ Ejj, const double* __restrict__ Eje,
-                                                   const double* __restrict__ Eej, const double* __restrict__ Ee,
-                                                   double* __restrict__ y) {
+// y_j = (g_j - E_je y_e) / E_jj; y[nc] = y_e. The division by E_jj and S_e is a product with their
+// reciprocals, formed once per step (an FP64 division is a chain of some 20 instructions).
+__global__ void __launch_bounds__(DT) k_defl_solve(int nc, int nchunks, int next, const int32_t* __restrict__ cchunk,
+                                                   const double* __restrict__ part, const double* __restrict__ iEjj,
+                                                   const double* __restrict__ Eje, const double* __restrict__ Eej,
+                                                   const double* __restrict__ Ee, double* __restrict__ y) {
     __shared__ double sh[DT / 32];
     __shared__ double ye_s;
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < EXT_BLOCKS; q += blockDim.x) a += part[q];
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) b += Eej[j] * g[j] / Ejj[j];
-    const double ge = block_sum(a, sh);
-    const double red = block_sum(b, sh);
+    double a = 0.0;
+    for (int q = threadIdx.x; q < next; q += DT) a += part[nchunks + q];
+    // a thread per cell, or a warp where cells have many chunks: g_j (kept in y until the solve)
+    const bool wide = nchunks > 8 * nc;
+    const int lane = threadIdx.x & 31;
+    for (int j = wide ? threadIdx.x >> 5 : threadIdx.x; j < nc; j += wide ? DT / 32 : DT) {
+        double g = 0.0;
+        for (int q = cchunk[j] + (wide ? lane : 0); q < cchunk[j + 1]; q += wide ? 32 : 1) g += part[q];
+        if (wide)
+            for (int o = 16; o > 0; o >>= 1) g += __shfl_down_sync(0xffffffffu, g, o);
+        if (!wide || lane == 0) {
+            y[j] = g;
+            a -= Eej[j] * (g * iEjj[j]);
+        }
+    }
+    const double t = block_sum(a, sh);
     if (threadIdx.x == 0) {
-        ye_s = (ge - red) / Ee[1];
+        ye_s = t * Ee[1];
         y[nc] = ye_s;
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) y[j] = (g[j] - Eje[j] * ye_s) / Ejj[j];
+    for (int j = threadIdx.x; j < nc; j += DT) y[j] = (y[j] - Eje[j] * ye_s) * iEjj[j];
 }
 
-// t = s .* v - A Z y. Row r of A Z y: its same-region phi columns hold its own region's constant
-// (RS), its cross-region entries their cells' constants; the potential row is sum_k z_k of the
-// concentration rows' terms; the pinned potential row (the identity) gives 0.
-__global__ void k_defl_rhs(int64_t n, int64_t N_i, int32_t pin, const int32_t* __restrict__ rgrp,
-                           const double* __restrict__ RS, const int32_t* __restrict__ xptr,
-                           const int32_t* __restrict__ xg, const double* __restrict__ xe, int64_t n_cross, double z0,
-                           double z1, double z2, const double* __restrict__ y, int32_t ext_group,
-                           const double* __restrict__ v, const double* __restrict__ s, double* __restrict__ t) {
+// t = s .* v - A Z y (or - A^T Z y), for CG(P_0)
+__global__ void k_defl_rhs(int64_t n, const double* __restrict__ v, const double* __restrict__ s, DeflFuse df,
+                           double* __restrict__ t) {
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const double yr = y[r < N_i ? rgrp[r] : ext_group];
-    double ae[KI];
-    for (int q = 0; q < KI; ++q) ae[q] = RS[3 * r + q] * yr;
-    for (int u = xptr[r]; u < xptr[r + 1]; ++u) {
-        const int gq = xg[u];
-        if (gq < 0) continue;
-        const double yc = y[gq];
-        for (int q = 0; q < KI; ++q) ae[q] += xe[q * n_cross + u] * yc;
-    }
-    double out3 = z0 * ae[0] + z1 * ae[1] + z2 * ae[2];
-    if (r == pin) out3 = 0.0;
-    const int64_t b = 4 * r;
-    t[b] = s[b] * v[b] - ae[0];
-    t[b + 1] = s[b + 1] * v[b + 1] - ae[1];
-    t[b + 2] = s[b + 2] * v[b + 2] - ae[2];
-    t[b + 3] = s[b + 3] * v[b + 3] - out3;
-}
-
-// t = s .* v - A^T Z y (the transposed operator's node block, cf. the transposed product): the
-// concentration rows see tau_r^k z_k (sum of a over the row's phi columns) times the row's own
-// constant; the potential row sum_k z_k e^k times it plus, through the transposed cross-region
-// list, sum_k z_k xe^k times the source rows' constants; the pinned potential row gives 0.
-__global__ void k_defl_rhs_t(int64_t n, int64_t N_i, int32_t pin, const int32_t* __restrict__ rgrp,
-                             const double* __restrict__ RS, const double* __restrict__ RSa,
-                             const int32_t* __restrict__ xtptr, const int32_t* __restrict__ xtidx,
-                             const int32_t* __restrict__ xtg, const double* __restrict__ xe, int64_t n_cross,
-                             double z0, double z1, double z2, RegionCoef ri, RegionCoef re,
-                             const double* __restrict__ y, int32_t ext_group, const double* __restrict__ v,
-                             const double* __restrict__ s, double* __restrict__ t) {
-    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const bool in = r < N_i;
-    const RegionCoef& rc = in ? ri : re;
-    const double yr = y[in ? rgrp[r] : ext_group];
-    const double z[KI] = {z0, z1, z2};
-    double out[4];
-    for (int q = 0; q < KI; ++q) out[q] = rc.tau[q] * z[q] * RSa[r] * yr;
-    double o3 = (z0 * RS[3 * r] + z1 * RS[3 * r + 1] + z2 * RS[3 * r + 2]) * yr;
-    for (int u = xtptr[r]; u < xtptr[r + 1]; ++u) {
-        const int gq = xtg[u];
-        if (gq < 0) continue;
-        const int64_t idx = xtidx[u];
-        o3 += (z0 * xe[idx] + z1 * xe[n_cross + idx] + z2 * xe[2 * n_cross + idx]) * y[gq];
-    }
-    out[3] = r == pin ? 0.0 : o3;
-    const int64_t b = 4 * r;
-    for (int q = 0; q < 4; ++q) t[b + q] = s[b + q] * v[b + q] - out[q];
+    double o[4];
+    defl_input(r, v, s, df, o);
+    for (int q = 0; q < 4; ++q) t[4 * r + q] = o[q];
 }
 
 // z += Z y: the potential of every node of a group takes its group's constant
@@ -269,19 +244,40 @@ inline unsigned nbk(int64_t n, int t) { return (unsigned)std::max<int64_t>(1, (n
 
 struct Deflation {
     int nc = 0;                       // cell groups (cells with at least one intracellular node)
-    DArray<int64_t> cptr;             // group -> its intracellular nodes (increasing)
-    DArray<int32_t> cnodes;
+    int64_t na = 0, na_i = 0;         // active rows, and the intracellular ones (first) among them
+    int gchunks = 0, echunks = 0;     // chunks of the cells' nodes (gather) and active rows (E)
+    int gext = 0, eext = 0;           // blocks of the extracellular sums of the two
+    DArray<int64_t> gbeg, ebeg;       // chunk -> its first entry of cnodes / aidx
+    DArray<int32_t> gcell, ecell;     // group -> its first chunk
+    DArray<int32_t> cnodes;           // intracellular nodes by group (increasing)
+    DArray<int32_t> aidx;             // intracellular active rows by group, as indices into rows
+    DArray<int32_t> rows;             // active rows (increasing)
+    DArray<int32_t> act;              // node -> its index in rows, -1 if not active
     DArray<int32_t> rgrp;             // intracellular node -> its group
     DArray<int32_t> xg;               // cross entry -> group of its column (-1: the pinned node)
-    DArray<double> RS;                // [n][3] row sums of e^k over phi columns (per step)
-    DArray<double> RSa;               // [n] row sums of a over phi columns (the transposed operator)
+    DArray<double> RS;                // [na][3] row sums of e^k over phi columns (per step)
+    DArray<double> RSa;               // [na] row sums of a over phi columns (the transposed operator)
     DArray<int32_t> xtg;              // transposed cross entry -> group of its source row (-1: pin)
-    DArray<double> Ejj, Eje, Eej, Ee; // the arrowhead E (per step); Ee = {E_ee, Schur complement}
-    DArray<double> g, y, part, t, ones;
+    DArray<double> iEjj, Eje, Eej;    // the arrowhead E (per step): 1 / E_jj, E_je, E_ej
+    DArray<double> Ee;                // {E_ee, 1 / Schur complement}
+    DArray<double> y, gpart, epart;
+    DArray<double> t, ones;           // CG(P_0)'s separate passes, on first use
     int64_t built_for = -1;           // assembly whose operator E was formed from
 };
 
 void deflation_free(Deflation* d) { delete d; }
+
+// Splits the lists of each group (gptr: group -> first entry) into chunks of at most `most` entries
+static void make_chunks(const std::vector<int64_t>& gptr, int64_t most, std::vector<int64_t>& beg,
+                        std::vector<int32_t>& first) {
+    beg.clear();
+    first.assign(1, 0);
+    for (size_t j = 0; j + 1 < gptr.size(); ++j) {
+        for (int64_t q = gptr[j]; q < gptr[j + 1]; q += most) beg.push_back(q);
+        first.push_back((int32_t)beg.size());
+    }
+    beg.push_back(gptr.back());
+}
 
 static Deflation& deflation_setup(knp_problem* p) {
     if (p->defl) return *p->defl;
@@ -291,52 +287,82 @@ static Deflation& deflation_setup(knp_problem* p) {
     const knp_mesh& m = *p->mesh;
     const std::vector<int32_t>& cell = p->degree == 2 ? p2_nodes(m).node_cell_i : m.node_cell_i;
     KNP_REQUIRE((int64_t)cell.size() == p->N_i, KNP_ERR_STATE, "cell map does not match the intracellular nodes");
+    const int64_t n = p->n_nodes;
     std::map<int32_t, int> gid;
     for (int32_t c : cell) gid.emplace(c, 0);
     int k = 0;
     for (auto& kv : gid) kv.second = k++;
     d->nc = k;
     std::vector<int32_t> rg(std::max<int64_t>(p->N_i, 1), 0);
-    std::vector<int64_t> cptr(d->nc + 1, 0);
-    for (int64_t r = 0; r < p->N_i; ++r) {
-        rg[r] = gid[cell[r]];
-        cptr[rg[r] + 1]++;
-    }
-    for (int j = 0; j < d->nc; ++j) cptr[j + 1] += cptr[j];
-    std::vector<int32_t> cn(std::max<int64_t>(p->N_i, 1));
+    for (int64_t r = 0; r < p->N_i; ++r) rg[r] = gid[cell[r]];
+    // active rows: membrane nodes (they have cross-region entries) and the rows with the pin's column,
+    // which by the pattern's symmetry are the columns of the pin's row
+    std::vector<uint8_t> on(n, 0);
+    for (int64_t r = 0; r < n; ++r) on[r] = p->h_xptr[r + 1] > p->h_xptr[r];
     {
-        std::vector<int64_t> fill(cptr.begin(), cptr.end() - 1);
-        for (int64_t r = 0; r < p->N_i; ++r) cn[fill[rg[r]]++] = (int32_t)r;
+        const SellPattern& S = p->sell;
+        const int64_t s = p->pin / SELL_C;
+        for (int64_t q = S.h_slice_ptr[s] + p->pin % SELL_C; q < S.h_slice_ptr[s + 1]; q += SELL_C) on[S.h_col[q]] = 1;
     }
+    std::vector<int32_t> rows, act(n, -1);
+    for (int64_t r = 0; r < n; ++r)
+        if (on[r]) {
+            act[r] = (int32_t)rows.size();
+            rows.push_back((int32_t)r);
+            d->na_i += r < p->N_i;
+        }
+    d->na = (int64_t)rows.size();
+    // entries [0, count) of a list (list[q]: intracellular node of entry q) by group, stably
+    auto by_group = [&](int64_t count, auto node_of, std::vector<int64_t>& gptr, std::vector<int32_t>& out) {
+        gptr.assign(d->nc + 1, 0);
+        for (int64_t q = 0; q < count; ++q) gptr[rg[node_of(q)] + 1]++;
+        for (int j = 0; j < d->nc; ++j) gptr[j + 1] += gptr[j];
+        out.assign(std::max<int64_t>(count, 1), 0);
+        std::vector<int64_t> fill(gptr.begin(), gptr.end() - 1);
+        for (int64_t q = 0; q < count; ++q) out[fill[rg[node_of(q)]]++] = (int32_t)q;
+    };
+    std::vector<int64_t> gptr, beg;
+    std::vector<int32_t> list, first;
+    by_group(p->N_i, [](int64_t q) { return q; }, gptr, list);
+    make_chunks(gptr, GATHER_NODES, beg, first);
+    d->gchunks = (int)beg.size() - 1;
+    d->gext = (int)std::min<int64_t>(EXT_BLOCKS, std::max<int64_t>(1, (p->N_e + GATHER_NODES - 1) / GATHER_NODES));
+    d->cnodes.upload(list, st);
+    d->gbeg.upload(beg, st);
+    d->gcell.upload(first, st);
+    by_group(d->na_i, [&](int64_t q) { return (int64_t)rows[q]; }, gptr, list);
+    make_chunks(gptr, DT, beg, first);
+    d->echunks = (int)beg.size() - 1;
+    d->eext = (int)std::max<int64_t>(1, (d->na - d->na_i + DT - 1) / DT);
+    d->aidx.upload(list, st);
+    d->ebeg.upload(beg, st);
+    d->ecell.upload(first, st);
     const int32_t ext = d->nc;
     std::vector<int32_t> xg(std::max<size_t>(p->h_xcol.size(), 1), -1);
     for (size_t t = 0; t < p->h_xcol.size(); ++t) {
         const int32_t c = p->h_xcol[t];
         xg[t] = c == p->pin ? -1 : (c < p->N_i ? rg[c] : ext);
     }
-    d->cptr.upload(cptr, st);
-    d->cnodes.upload(cn, st);
+    d->rows.upload(rows, st);
+    d->act.upload(act, st);
     d->rgrp.upload(rg, st);
     d->xg.upload(xg, st);
-    const int64_t n = p->n_nodes;
-    d->RS.alloc(3 * n);
-    d->RSa.alloc(n);
+    d->RS.alloc(3 * d->na);
+    d->RSa.alloc(d->na);
     const int64_t nx = (int64_t)p->h_xcol.size();
     d->xtg.alloc(std::max<int64_t>(nx, 1));
     if (nx) {
         k_defl_xtg<<<nbk(nx, 256), 256, 0, st>>>(nx, p->N_i, p->pin, p->xtrow.p, d->rgrp.p, ext, d->xtg.p);
         count_launch();
     }
-    for (DArray<double>* a : {&d->Ejj, &d->Eje, &d->Eej}) a->alloc(std::max(d->nc, 1));
+    for (DArray<double>* a : {&d->iEjj, &d->Eje, &d->Eej}) a->alloc(std::max(d->nc, 1));
     d->Ee.alloc(2);
-    d->g.alloc(std::max(d->nc, 1));
     d->y.alloc(d->nc + 1);
-    d->part.alloc(EXT_BLOCKS);
-    d->t.alloc(4 * n);
-    d->ones.alloc(4 * n);
-    k_fill_ones<<<nbk(4 * n, 256), 256, 0, st>>>(4 * n, d->ones.p);
-    count_launch();
+    d->gpart.alloc(d->gchunks + d->gext);
+    d->epart.alloc(3 * (d->echunks + d->eext));
     KNP_CUDA(cudaGetLastError());
+    // the host tables above go out of scope here
+    KNP_CUDA(cudaStreamSynchronize(st));
     return *d;
 }
 
@@ -344,58 +370,63 @@ void deflation_prepare(knp_problem* p) {
     Deflation& d = deflation_setup(p);
     if (d.built_for == p->assembly_id) return;
     cudaStream_t st = p->stream;
-    const int64_t n = p->n_nodes, nx = (int64_t)p->h_xcol.size();
+    const int64_t nx = (int64_t)p->h_xcol.size();
     const double* z = p->sp.z;
-    count_launch(4);
-    k_defl_rowsums<<<nbk(n, 128), 128, 0, st>>>(n, p->pin, p->sell.slice_ptr.p, p->sell.col.p, p->sell_e.p,
-                                                 p->sell.n_entries, p->sell_a.p, d.RS.p, d.RSa.p);
-    if (d.nc)
-        k_defl_E_cells<<<d.nc, DT, 0, st>>>(d.cptr.p, d.cnodes.p, d.RS.p, p->xptr.p, d.xg.p, p->xtptr.p, p->xtrow.p,
-                                            p->xtidx.p, p->xe.p, nx, p->pin, z[0], z[1], z[2], d.nc, d.Ejj.p,
-                                            d.Eje.p, d.Eej.p);
-    k_defl_E_ext<<<EXT_BLOCKS, DT, 0, st>>>(p->N_i, n, p->pin, d.RS.p, z[0], z[1], z[2], d.part.p);
-    k_defl_schur<<<1, DT, 0, st>>>(d.nc, EXT_BLOCKS, d.part.p, d.Ejj.p, d.Eje.p, d.Eej.p, d.Ee.p);
+    count_launch(3);
+    k_defl_rowsums<<<nbk(d.na, 64), 64, 0, st>>>(d.na, p->pin, d.rows.p, p->sell.slice_ptr.p, p->sell.col.p,
+                                                 p->sell_e.p, p->sell.n_entries, p->sell_a.p, d.RS.p, d.RSa.p);
+    k_defl_E<<<d.echunks + d.eext, DT, 0, st>>>(d.echunks, d.ebeg.p, d.aidx.p, d.na_i, d.na, d.rows.p, d.RS.p,
+                                                p->xptr.p, d.xg.p, p->xtptr.p, p->xtrow.p, p->xtidx.p, p->xe.p, nx,
+                                                p->pin, z[0], z[1], z[2], d.nc, d.epart.p);
+    k_defl_schur<<<1, DT, 0, st>>>(d.nc, d.echunks, d.eext, d.ecell.p, d.epart.p, d.iEjj.p, d.Eje.p, d.Eej.p, d.Ee.p);
     KNP_CUDA(cudaGetLastError());
     d.built_for = p->assembly_id;
 }
 
-void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose) {
+void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose,
+                            double* w) {
     Deflation& d = *p->defl;
     cudaStream_t st = p->stream;
-    const int64_t n = p->n_nodes, nx = (int64_t)p->h_xcol.size();
-    const double* zc = p->sp.z;
+    const int64_t n = p->n_nodes;
     count_launch(2);
-    k_defl_gather<<<d.nc + EXT_BLOCKS, DT, 0, st>>>(d.nc, d.cptr.p, d.cnodes.p, p->N_i, n, p->pin, v, s, d.g.p,
-                                                    d.part.p);
+    k_defl_gather<<<d.gchunks + d.gext, DT, 0, st>>>(d.gchunks, d.gbeg.p, d.cnodes.p, p->N_i, n, p->pin, v, s,
+                                                     d.gpart.p);
     // Z^T A^T Z = E^T: the same Schur complement, E_je and E_ej exchanged
-    k_defl_solve<<<1, DT, 0, st>>>(d.nc, d.part.p, d.g.p, d.Ejj.p, transpose ? d.Eej.p : d.Eje.p,
-                                   transpose ? d.Eje.p : d.Eej.p, d.Ee.p, d.y.p);
-    if (!transpose && p->amg->inner_cg_max_it == 0) {
+    k_defl_solve<<<1, DT, 0, st>>>(d.nc, d.gchunks, d.gext, d.gcell.p, d.gpart.p, d.iEjj.p,
+                                   transpose ? d.Eej.p : d.Eje.p, transpose ? d.Eje.p : d.Eej.p, d.Ee.p, d.y.p);
+    KNP_CUDA(cudaGetLastError());
+    DeflFuse df;
+    df.rgrp = d.rgrp.p;
+    df.act = d.act.p;
+    df.RS = d.RS.p;
+    df.RSa = d.RSa.p;
+    df.xptr = transpose ? p->xtptr.p : p->xptr.p;
+    df.xg = transpose ? d.xtg.p : d.xg.p;
+    df.xidx = transpose ? p->xtidx.p : nullptr;
+    df.xe = p->xe.p;
+    df.y = d.y.p;
+    df.n_cross = (int64_t)p->h_xcol.size();
+    df.N_i = p->N_i;
+    df.pin = p->pin;
+    df.ext_group = d.nc;
+    df.transpose = transpose;
+    for (int q = 0; q < 3; ++q) {
+        df.z[q] = p->sp.z[q];
+        for (int r = 0; r < 2; ++r) df.ztau[r][q] = p->sp.z[q] * p->sp.reg[r].tau[q];
+    }
+    if (p->amg->inner_cg_max_it == 0) {
         // one V-cycle: its first kernel forms s .* v - A Z y and its output kernel adds Z y
-        DeflFuse df;
-        df.rgrp = d.rgrp.p;
-        df.RS = d.RS.p;
-        df.xptr = p->xptr.p;
-        df.xg = d.xg.p;
-        df.xe = p->xe.p;
-        df.y = d.y.p;
-        df.n_cross = nx;
-        df.N_i = p->N_i;
-        df.pin = p->pin;
-        df.ext_group = d.nc;
-        for (int q = 0; q < 3; ++q) df.z[q] = zc[q];
-        KNP_CUDA(cudaGetLastError());
-        vcycle_apply(p, v, s, z, &df);
+        vcycle_apply(p, v, s, z, &df, w);
         return;
     }
+    if (!d.t.p) {
+        d.t.alloc(4 * n);
+        d.ones.alloc(4 * n);
+        k_fill_ones<<<nbk(4 * n, 256), 256, 0, st>>>(4 * n, d.ones.p);
+        count_launch();
+    }
     count_launch();
-    if (transpose)
-        k_defl_rhs_t<<<nbk(n, 128), 128, 0, st>>>(n, p->N_i, p->pin, d.rgrp.p, d.RS.p, d.RSa.p, p->xtptr.p,
-                                                  p->xtidx.p, d.xtg.p, p->xe.p, nx, zc[0], zc[1], zc[2], p->sp.reg[0],
-                                                  p->sp.reg[1], d.y.p, d.nc, v, s, d.t.p);
-    else
-        k_defl_rhs<<<nbk(n, 128), 128, 0, st>>>(n, p->N_i, p->pin, d.rgrp.p, d.RS.p, p->xptr.p, d.xg.p, p->xe.p, nx,
-                                                zc[0], zc[1], zc[2], d.y.p, d.nc, v, s, d.t.p);
+    k_defl_rhs<<<nbk(n, 128), 128, 0, st>>>(n, v, s, df, d.t.p);
     precond_apply(p, d.t.p, d.ones.p, z);
     count_launch();
     k_defl_add<<<nbk(n, 256), 256, 0, st>>>(n, p->N_i, p->pin, d.rgrp.p, d.y.p, d.nc, z);

@@ -8,6 +8,7 @@ namespace knp {
 void deflation_prepare(knp_problem* p);
 // z = P_0^{-1} (r - A Z y) + Z y with r = s .* v, y = E^{-1} Z^T r (after deflation_prepare); with
 // transpose, A^T and E^T in their places (P_0 is symmetric)
-void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose = false);
+void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose = false,
+                            double* w = nullptr);
 void deflation_free(Deflation* d);
 }  // namespace knp

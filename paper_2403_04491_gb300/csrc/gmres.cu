@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <chrono>
 #include <map>
+#include <tuple>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -495,8 +496,8 @@ struct GmresWork {
     double* hh = nullptr;           // pinned copy of dots, DOTS_LEN
     cudaEvent_t ev_dots = nullptr;  // recorded after the copy of dots to hh
     // the Arnoldi step of basis index j (SpMV, the three orthogonalisation passes with their
-    // reductions, the copy of the dots to hh) as a CUDA graph per (j, transposed)
-    std::map<std::pair<int, bool>, cudaGraphExec_t> arnoldi;
+    // reductions, the copy of the dots to hh) as a CUDA graph per (j, transposed, w formed by the V-cycle)
+    std::map<std::tuple<int, bool, bool>, cudaGraphExec_t> arnoldi;
     cudaStream_t cap = nullptr;     // capture stream (the problem's stream may be the legacy one)
     // partial sums: of an Arnoldi step's two passes, each read by the kernel after it, and the others'
     double* pass1() { return partial.p; }
@@ -546,14 +547,14 @@ static double norm2_dev(GmresWork& g, const double* v, cudaStream_t st) {
 
 // w = S^-1 A z_j into V_{j+1}, orthogonalised against V_0..V_j (CGS2, second pass skipped on the
 // device when it has nothing to remove) and normalised; the dots of both passes land in g.dots
-static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, cudaStream_t st) {
+static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready, cudaStream_t st) {
     const int64_t n4 = g.n4;
     const int nv = j + 1;
     const int nb_red = red_grid(n4);
     const unsigned nb_vec = vec_grid(n4);
     double* zj = g.Z.p + (int64_t)j * n4;
     double* w = g.V.p + (int64_t)(j + 1) * n4;
-    op_apply(p, zj, w, p->sinv.p, nullptr, transpose, st);
+    op_apply(p, zj, w, p->sinv.p, nullptr, transpose, st, w_ready);
     ProfScope ps(&p->prof, KC_ORTHO, st);
     count_launch(3);
 #define KNP_ARGS n4, g.V.p, n4, w, g.pass1()
@@ -570,15 +571,15 @@ static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose,
 
 // The Arnoldi step j followed by the copy of the dots to the pinned g.hh, replayed from a CUDA
 // graph captured at first use (about ten launches become one).
-static void arnoldi_graph_launch(knp_problem* p, GmresWork& g, int j, bool transpose) {
-    auto key = std::make_pair(j, transpose);
+static void arnoldi_graph_launch(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready) {
+    auto key = std::make_tuple(j, transpose, w_ready);
     auto it = g.arnoldi.find(key);
     if (it == g.arnoldi.end()) {
         if (!g.cap) KNP_CUDA(cudaStreamCreateWithFlags(&g.cap, cudaStreamNonBlocking));
         const int64_t before = g_launches.load();
         KNP_CUDA(cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal));
         try {
-            arnoldi_kernels(p, g, j, transpose, g.cap);
+            arnoldi_kernels(p, g, j, transpose, w_ready, g.cap);
             KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, g.cap));
         } catch (...) {
             cudaGraph_t tmp = nullptr;
@@ -618,11 +619,15 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
     const int64_t n4i = 4 * p->N_i;
     const bool defl = o.deflate != 0;
     if (defl) deflation_prepare(p);
+    // the forward product of the preconditioner's result reads its w, which the V-cycle can form; the
+    // Arnoldi step of z_j always follows its preconditioning directly
+    const bool w_ready = !transpose && op_reads_w(p) && vcycle_forms_w(p);
+    double* const wz = w_ready ? p->op_w.p : nullptr;
     auto precond = [&](const double* v, const double* s, double* z) {
         if (defl)
-            deflated_precond_apply(p, v, s, z, transpose);
+            deflated_precond_apply(p, v, s, z, transpose, wz);
         else
-            precond_apply(p, v, s, z);
+            precond_apply(p, v, s, z, wz);
     };
     if (paper_test && !g.ones.p) {
         g.ones.alloc(n4);
@@ -755,9 +760,9 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
             }
             const int nv = j + 1;
             if (arnoldi && use_graphs) {
-                arnoldi_graph_launch(p, g, j, transpose);   // includes the copy of the dots
+                arnoldi_graph_launch(p, g, j, transpose, w_ready);   // includes the copy of the dots
             } else {
-                if (arnoldi) arnoldi_kernels(p, g, j, transpose, st);
+                if (arnoldi) arnoldi_kernels(p, g, j, transpose, w_ready, st);
                 KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, st));
             }
             KNP_CUDA(cudaEventRecord(g.ev_dots, st));

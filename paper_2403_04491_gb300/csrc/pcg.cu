@@ -204,12 +204,12 @@ void pcg_apply(knp_problem* p, const double* v, const double* s, double* z) {
 
 }  // namespace
 
-void precond_apply(knp_problem* p, const double* v, const double* s, double* z) {
+void precond_apply(knp_problem* p, const double* v, const double* s, double* z, double* w) {
     KNP_REQUIRE(p->amg, KNP_ERR_STATE, "knp_amg_setup has not been called");
     if (p->amg->inner_cg_max_it > 0)
         pcg_apply(p, v, s, z);
     else
-        vcycle_apply(p, v, s, z);
+        vcycle_apply(p, v, s, z, nullptr, w);
 }
 
 }  // namespace knp

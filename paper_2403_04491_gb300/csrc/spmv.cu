@@ -11,7 +11,8 @@
 // GB300 issues FP64 at 1/64 of its FP32 rate, so the forward product is bound by FP64 FMAs, not
 // by bytes. It therefore reads the static per-ion sums g^k = m + tau_r^k a (folded once at
 // problem creation) and, for the potential row, a per-node w = sum_k z_k tau_r^k x^k made by a
-// small pass over the nodes first:
+// small pass over the nodes first (or by
+// the V-cycle's last kernel, when x is its result):
 //     c^k row:  sum g^k x^k + sum e^k phi,     phi row:  sum a w + sum_k z_k (sum e^k phi),
 // seven FMAs per stored entry (g^k x^k, e^k phi, a w) for 60 bytes, where m, a with the
 // per-row tau take nine for 44 bytes. The transposed product keeps the m, a form.
@@ -253,8 +254,14 @@ __global__ void __launch_bounds__(128) k_op_apply_t(OpArgs A, const double* __re
 
 }  // namespace
 
+static int op_lanes(const knp_problem* p) {
+    return row_lanes(p->n_nodes, (double)p->sell.n_entries / (double)std::max<int64_t>(p->n_nodes, 1));
+}
+
+bool op_reads_w(const knp_problem* p) { return op_lanes(p) == 1; }
+
 void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale, const double* b, bool transpose,
-              cudaStream_t st) {
+              cudaStream_t st, bool w_ready) {
     if (st == kProblemStream) st = p->stream;
     OpArgs A;
     A.n = p->n_nodes;
@@ -278,7 +285,7 @@ void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale
     for (int r = 0; r < 2; ++r)
         for (int k = 0; k < KI; ++k) A.tau[r][k] = p->sp.reg[r].tau[k];
     for (int k = 0; k < KI; ++k) A.z[k] = p->sp.z[k];
-    const int lanes = row_lanes(A.n, (double)A.n_entries / (double)std::max<int64_t>(A.n, 1));
+    const int lanes = op_lanes(p);
     const unsigned blocks = (unsigned)((A.n * lanes + 127) / 128);
     ProfScope ps(&p->prof, KC_SPMV, st);
     count_launch();
@@ -290,8 +297,10 @@ void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale
         else
             k_op_apply_t<8><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
     } else if (lanes == 1) {
-        count_launch();
-        k_op_w<<<(unsigned)((A.n + 255) / 256), 256, 0, st>>>(A, x, p->op_w.p);
+        if (!w_ready) {
+            count_launch();
+            k_op_w<<<(unsigned)((A.n + 255) / 256), 256, 0, st>>>(A, x, p->op_w.p);
+        }
         k_op_apply<1><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
     } else if (lanes == 4) {
         k_op_apply<4><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);

@@ -22,6 +22,7 @@
 
 #include "amg.h"
 #include "amg_gpu.h"
+#include "deflate_input.h"
 #include "lanes.h"
 #include "problem.h"
 #include "vcycle.h"
@@ -183,27 +184,6 @@ __device__ __forceinline__ T csr_row_field(bool active, int64_t r, int t, const 
     return out[0];
 }
 
-// The coarse correction's input at node i: t = s .* v - (A Z y)_i. Row i of A Z y: its same-region
-// phi columns hold its own group's constant (the row sums RS), its cross-region entries their
-// groups' constants; the potential row is sum_k z_k of the concentration rows' terms, and the
-// pinned potential row (the identity) gives 0.
-__device__ __forceinline__ void defl_input(int64_t i, const double* __restrict__ v, const double* __restrict__ s,
-                                           const DeflFuse& df, double t[4]) {
-    const double yr = df.y[i < df.N_i ? df.rgrp[i] : df.ext_group];
-    double ae[3];
-    for (int q = 0; q < 3; ++q) ae[q] = df.RS[3 * i + q] * yr;
-    for (int u = df.xptr[i]; u < df.xptr[i + 1]; ++u) {
-        const int gq = df.xg[u];
-        if (gq < 0) continue;
-        const double yc = df.y[gq];
-        for (int q = 0; q < 3; ++q) ae[q] += df.xe[q * df.n_cross + u] * yc;
-    }
-    double out3 = df.z[0] * ae[0] + df.z[1] * ae[1] + df.z[2] * ae[2];
-    if (i == df.pin) out3 = 0.0;
-    for (int q = 0; q < 3; ++q) t[q] = s[4 * i + q] * v[4 * i + q] - ae[q];
-    t[3] = s[4 * i + 3] * v[4 * i + 3] - out3;
-}
-
 // first Chebyshev step from x = 0: d = c2 D^-1 b, x = d (d stored if a second step reads it). On the finest level b = s .* v (double
 // input), or s .* v - A Z y inside the coarse correction (df.y set).
 template <class T>
@@ -230,14 +210,46 @@ __global__ void k_cheb_first(int64_t n, const double* __restrict__ v, const doub
     dd.store(x + 4 * i);
 }
 
+// Where the finest level's last smoothing step puts the V-cycle's result: z = x in FP64, every
+// potential but the pinned one raised by its group's constant of the coarse correction (y set), and the
+// operator product's w = sum_k z_k tau_r^k z^k (w set; needs all fields in one thread). Done there it
+// saves a pass that reads x and one that reads z, and their launches.
+struct VcycleOut {
+    double* z = nullptr;
+    double* w = nullptr;
+    const double* y = nullptr;
+    const int32_t* rgrp = nullptr;
+    int64_t N_i = 0;
+    int32_t pin = -1, ext_group = 0;
+    double ztau[2][3] = {};
+};
+
+// fields f0 .. f0 + F of node i
+template <class T, int F>
+__device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0, const VN<T, F>& x) {
+    VN<double, F> z;
+    for (int f = 0; f < F; ++f) z.v[f] = (double)x.v[f];
+    const bool in = i < o.N_i;
+    if (o.y && f0 + F == 4 && i != o.pin) z.v[F - 1] += o.y[in ? o.rgrp[i] : o.ext_group];
+    z.store(o.z + 4 * i + f0);
+    if constexpr (F == 4) {
+        if (o.w) {
+            const double z0 = in ? o.ztau[0][0] : o.ztau[1][0], z1 = in ? o.ztau[0][1] : o.ztau[1][1],
+                         z2 = in ? o.ztau[0][2] : o.ztau[1][2];
+            o.w[i] = z0 * z.v[0] + z1 * z.v[1] + z2 * z.v[2];
+        }
+    }
+}
+
 // Chebyshev step: r = b - A x_in; d = c1 d + c2 D^-1 r; x_out = x_in + d. The first step of a sweep
-// (c1 = 0) does not read d, the last one does not store it.
-template <class T, int L>
+// (c1 = 0) does not read d, the last one does not store it; with OUT it is the V-cycle's last and writes
+// its result instead of x_out.
+template <class T, int L, bool OUT>
 __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __restrict__ sp,
                                                    const int32_t* __restrict__ col, const T* __restrict__ val,
                                                    const T* __restrict__ x_in, const T* __restrict__ b,
                                                    const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
-                                                   T* __restrict__ x_out, int read_d, int write_d) {
+                                                   T* __restrict__ x_out, int read_d, int write_d, VcycleOut out) {
     constexpr int F = LANE_FIELDS<L>;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t i = g / L;
@@ -259,15 +271,18 @@ __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __r
     }
     for (int f = 0; f < F; ++f) xx.v[f] += dd.v[f];
     if (write_d) dd.store(d + k);
-    xx.store(x_out + k);
+    if constexpr (OUT)
+        store_out<T, F>(out, i, f0, xx);
+    else
+        xx.store(x_out + k);
 }
 
-template <class T, int L>
+template <class T, int L, bool OUT>
 __global__ void __launch_bounds__(128) k_cheb_csr(int64_t n, const int64_t* __restrict__ ptr,
                                                   const int32_t* __restrict__ col, const T* __restrict__ val,
                                                   const T* __restrict__ x_in, const T* __restrict__ b,
                                                   const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
-                                                  T* __restrict__ x_out, int read_d, int write_d) {
+                                                  T* __restrict__ x_out, int read_d, int write_d, VcycleOut out) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
     const int t = (int)(g % L);
     const T acc = csr_row_field<T, L>(i < n, i, t, ptr, col, val, x_in);
@@ -276,7 +291,11 @@ __global__ void __launch_bounds__(128) k_cheb_csr(int64_t n, const int64_t* __re
         T dd = (T)pick4(c.c2, t) * dinv[k] * (b[k] - acc);
         if (read_d) dd = (T)pick4(c.c1, t) * d[k] + dd;
         if (write_d) d[k] = dd;
-        x_out[k] = x_in[k] + dd;
+        const T x = x_in[k] + dd;
+        if constexpr (OUT)
+            store_out<T, 1>(out, i, t, VN<T, 1>{{x}});
+        else
+            x_out[k] = x;
     }
 }
 
@@ -401,18 +420,11 @@ __global__ void k_to_double(int64_t n4, const T* __restrict__ x, double* __restr
     if (i < n4) z[i] = (double)x[i];
 }
 
-// z = x + Z y: the V-cycle's output in FP64, every potential but the pinned one raised by its
-// group's constant of the coarse correction
+// the V-cycle's result from x (a single-level hierarchy)
 template <class T>
-__global__ void k_out_defl(int64_t n, const T* __restrict__ x, double* __restrict__ z, DeflFuse df) {
-    int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const V4<T> xx = V4<T>::load(x + 4 * r);
-    double o3 = (double)xx.v[3];
-    if (r != df.pin) o3 += df.y[r < df.N_i ? df.rgrp[r] : df.ext_group];
-    double2* zp = reinterpret_cast<double2*>(z + 4 * r);
-    zp[0] = make_double2((double)xx.v[0], (double)xx.v[1]);
-    zp[1] = make_double2((double)xx.v[2], o3);
+__global__ void k_out(int64_t n, const T* __restrict__ x, VcycleOut out) {
+    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (r < n) store_out<T, 4>(out, r, 0, VN<T, 4>::load(x + 4 * r));
 }
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -836,33 +848,38 @@ void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, in
 // CSR kernels with the matrix's lanes per row
 #define KNP_CSR_DISPATCH(lanes, KERNEL, rows, ...)                                                \
     switch (lanes) {                                                                              \
-        case 4: KERNEL<T, 4><<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
-        case 8: KERNEL<T, 8><<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
-        case 16: KERNEL<T, 16><<<nblk((rows) * 16, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
-        case 32: KERNEL<T, 32><<<nblk((rows) * 32, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
-        default: KERNEL<T, 128><<<nblk((rows) * 128, 128), 128, 0, st>>>(__VA_ARGS__); break;     \
+        case 4: KERNEL(4)<<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
+        case 8: KERNEL(8)<<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
+        case 16: KERNEL(16)<<<nblk((rows) * 16, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
+        case 32: KERNEL(32)<<<nblk((rows) * 32, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
+        default: KERNEL(128)<<<nblk((rows) * 128, 128), 128, 0, st>>>(__VA_ARGS__); break;     \
     }
 
 // sliced-ELL kernels with the level's lanes per row
 #define KNP_LANE_DISPATCH(lanes, KERNEL, rows, ...)                                               \
     switch (lanes) {                                                                              \
-        case 1: KERNEL<T, 1><<<nblk(rows, 128), 128, 0, st>>>(__VA_ARGS__); break;                \
-        case 4: KERNEL<T, 4><<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
-        default: KERNEL<T, 8><<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;         \
+        case 1: KERNEL(1)<<<nblk(rows, 128), 128, 0, st>>>(__VA_ARGS__); break;                   \
+        case 4: KERNEL(4)<<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;             \
+        default: KERNEL(8)<<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
     }
+#define KNP_K_CHEB_SELL(L) k_cheb_sell<T, L, OUT>
+#define KNP_K_CHEB_CSR(L) k_cheb_csr<T, L, OUT>
+#define KNP_K_RESID_SELL(L) k_resid_sell<T, L>
+#define KNP_K_RESID_CSR(L) k_resid_csr<T, L>
+#define KNP_K_CSR4(L) k_csr4<T, L>
 
-// Chebyshev step k of a sweep of `steps` steps
-template <class T>
+// Chebyshev step k of a sweep of `steps` steps; OUT: into `out` instead of x_out
+template <class T, bool OUT = false>
 static void launch_cheb(const DevLevel<T>& L, const T* x_in, const T* b, const Coef4& c, T* d, T* x_out, int k,
-                        int steps, cudaStream_t st) {
+                        int steps, cudaStream_t st, const VcycleOut& out = VcycleOut{}) {
     count_launch();
     const int read_d = k > 0, write_d = k + 1 < steps;
     if (L.sell) {
-        KNP_LANE_DISPATCH(L.lanes, k_cheb_sell, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x_in, b, L.dinv.p, c, d, x_out,
-                          read_d, write_d);
+        KNP_LANE_DISPATCH(L.lanes, KNP_K_CHEB_SELL, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x_in, b, L.dinv.p, c, d, x_out,
+                          read_d, write_d, out);
     } else {
-        KNP_CSR_DISPATCH(L.A.lanes, k_cheb_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x_in, b, L.dinv.p, c, d,
-                         x_out, read_d, write_d);
+        KNP_CSR_DISPATCH(L.A.lanes, KNP_K_CHEB_CSR, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x_in, b, L.dinv.p, c, d,
+                         x_out, read_d, write_d, out);
     }
 }
 
@@ -870,9 +887,9 @@ template <class T>
 static void launch_resid(const DevLevel<T>& L, const T* x, const T* b, T* r, cudaStream_t st) {
     count_launch();
     if (L.sell) {
-        KNP_LANE_DISPATCH(L.lanes, k_resid_sell, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x, b, r);
+        KNP_LANE_DISPATCH(L.lanes, KNP_K_RESID_SELL, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x, b, r);
     } else {
-        KNP_CSR_DISPATCH(L.A.lanes, k_resid_csr, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x, b, r);
+        KNP_CSR_DISPATCH(L.A.lanes, KNP_K_RESID_CSR, L.n, L.n, L.A.ptr.p, L.A.col.p, L.A.val.p, x, b, r);
     }
 }
 
@@ -881,6 +898,14 @@ static void cheb_step(DevLevel<T>& L, const Coef4& c, int k, int steps, Profiler
     ProfScope ps(fine ? pr : nullptr, KC_CHEB_FINE, st);
     launch_cheb(L, L.x.p, L.b.p, c, L.d.p, L.x2.p, k, steps, st);
     std::swap(L.x.p, L.x2.p);
+}
+
+// the sweep's last step, whose result is the V-cycle's
+template <class T>
+static void cheb_step_out(DevLevel<T>& L, const Coef4& c, int k, int steps, const VcycleOut& out, Profiler* pr,
+                          cudaStream_t st) {
+    ProfScope ps(pr, KC_CHEB_FINE, st);
+    launch_cheb<T, true>(L, L.x.p, L.b.p, c, L.d.p, nullptr, k, steps, st, out);
 }
 
 template <class T>
@@ -893,7 +918,7 @@ static void residual(DevLevel<T>& L, Profiler* pr, bool fine, cudaStream_t st) {
 template <class T>
 static void restrict_to(const DevCsr4<T>& R, const T* r, T* rc, cudaStream_t st) {
     count_launch();
-    KNP_CSR_DISPATCH(R.lanes, k_csr4, R.n, R.n, R.ptr.p, R.col.p, R.val.p, r, rc);
+    KNP_CSR_DISPATCH(R.lanes, KNP_K_CSR4, R.n, R.n, R.ptr.p, R.col.p, R.val.p, r, rc);
 }
 
 // x += P xc
@@ -921,7 +946,7 @@ static void smooth(DevLevel<T>& L, const std::vector<Coef4>& cs, int degree, boo
 
 template <class T>
 static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, const DeflFuse& df, Profiler* pr,
-                       cudaStream_t st) {
+                       cudaStream_t st, const VcycleOut& out) {
     DevLevel<T>& L = *D.L[l];
     const int last = (int)D.L.size() - 1;
     if (l == last) {
@@ -939,31 +964,54 @@ static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, co
     smooth(L, D.coef[l], D.pre, true, v, s, df, pr, l == 0, st);
     residual(L, pr, l == 0, st);
     restrict_to(L.R, L.r.p, C.b.p, st);
-    vcycle_rec(D, l + 1, nullptr, nullptr, DeflFuse{}, pr, st);
+    vcycle_rec(D, l + 1, nullptr, nullptr, DeflFuse{}, pr, st, out);
     prolong(L.P, C.x.p, L.x.p, st);
-    smooth(L, D.coef[l], D.degree, false, nullptr, nullptr, DeflFuse{}, pr, l == 0, st);
+    if (l > 0) {
+        smooth(L, D.coef[l], D.degree, false, nullptr, nullptr, DeflFuse{}, pr, false, st);
+    } else {
+        for (int k = 0; k + 1 < D.degree; ++k) cheb_step(L, D.coef[l][k], k, D.degree, pr, true, st);
+        cheb_step_out(L, D.coef[l][D.degree - 1], D.degree - 1, D.degree, out, pr, st);
+    }
 }
 
-static void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse& df,
-                          cudaStream_t st) {
-    if (p->amg->h32) {
-        auto& D = *static_cast<AmgDev<float>*>(p->amg->h32);
-        vcycle_rec(D, 0, v, s, df, &p->prof, st);
+template <class T>
+static void vcycle_typed(knp_problem* p, AmgDev<T>& D, const double* v, const double* s, double* z,
+                         const DeflFuse& df, double* w, cudaStream_t st) {
+    VcycleOut out;
+    out.z = z;
+    out.w = w;
+    out.y = df.y;
+    out.rgrp = df.rgrp;
+    out.N_i = p->N_i;
+    out.pin = df.pin;
+    out.ext_group = df.ext_group;
+    for (int r = 0; r < 2; ++r)
+        for (int q = 0; q < 3; ++q) out.ztau[r][q] = p->sp.z[q] * p->sp.reg[r].tau[q];
+    vcycle_rec(D, 0, v, s, df, &p->prof, st, out);
+    if (D.L.size() == 1) {
+        // no smoothing on a single level: the coarse solution is the result
         count_launch();
-        if (df.y)
-            k_out_defl<float><<<nblk(D.L[0]->n, 256), 256, 0, st>>>(D.L[0]->n, D.L[0]->x.p, z, df);
-        else
-            k_to_double<float><<<nblk(4 * D.L[0]->n, 256), 256, 0, st>>>(4 * D.L[0]->n, D.L[0]->x.p, z);
-    } else {
-        auto& D = *static_cast<AmgDev<double>*>(p->amg->h64);
-        vcycle_rec(D, 0, v, s, df, &p->prof, st);
-        if (df.y) {
-            count_launch();
-            k_out_defl<double><<<nblk(D.L[0]->n, 256), 256, 0, st>>>(D.L[0]->n, D.L[0]->x.p, z, df);
-        } else {
-            KNP_CUDA(cudaMemcpyAsync(z, D.L[0]->x.p, 4 * D.L[0]->n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-        }
+        k_out<T><<<nblk(D.L[0]->n, 256), 256, 0, st>>>(D.L[0]->n, D.L[0]->x.p, out);
     }
+}
+
+static void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse& df, double* w,
+                          cudaStream_t st) {
+    if (p->amg->h32)
+        vcycle_typed(p, *static_cast<AmgDev<float>*>(p->amg->h32), v, s, z, df, w, st);
+    else
+        vcycle_typed(p, *static_cast<AmgDev<double>*>(p->amg->h64), v, s, z, df, w, st);
+}
+
+template <class T>
+static bool forms_w(const AmgDev<T>& D) {
+    return D.L.size() > 1 && D.L[0]->sell && D.L[0]->lanes == 1;
+}
+
+bool vcycle_forms_w(const knp_problem* p) {
+    if (!p->amg || p->amg->inner_cg_max_it > 0) return false;
+    return p->amg->h32 ? forms_w(*static_cast<AmgDev<float>*>(p->amg->h32))
+                       : forms_w(*static_cast<AmgDev<double>*>(p->amg->h64));
 }
 
 // z = V-cycle(P_0)(s .* v); v, s, z are [n][4] doubles on the device. The V-cycle is a fixed
@@ -980,29 +1028,29 @@ void p0_apply(knp_problem* p, const double* x, double* y) {
     KNP_CUDA(cudaGetLastError());
 }
 
-void vcycle_apply(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse* dfp) {
+void vcycle_apply(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse* dfp, double* w) {
     KNP_REQUIRE(p->amg, KNP_ERR_STATE, "knp_amg_setup has not been called");
     AmgHierarchy& H = *p->amg;
     cudaStream_t st = p->stream;
     const DeflFuse df = dfp ? *dfp : DeflFuse{};
     if (!H.use_graphs || p->prof.active >= 0) {
         ProfScope ps(&p->prof, KC_VCYCLE, st);
-        vcycle_launch(p, v, s, z, df, st);
+        vcycle_launch(p, v, s, z, df, w, st);
         KNP_CUDA(cudaGetLastError());
         return;
     }
     if (!H.gstream) {
         KNP_CUDA(cudaStreamCreateWithFlags(&H.gstream, cudaStreamNonBlocking));
     }
-    // the correction's arrays are fixed per problem, so its y pointer identifies them
-    auto key = std::make_tuple(v, s, z, df.y);
+    // the correction's arrays are fixed per problem, so its y pointer and direction identify them
+    auto key = std::make_tuple(v, s, z, df.y, (int)df.transpose, w);
     auto it = H.graphs.find(key);
     if (it == H.graphs.end()) {
         VcycleGraph g;
         int64_t before = g_launches.load();
         KNP_CUDA(cudaStreamBeginCapture(H.gstream, cudaStreamCaptureModeThreadLocal));
         try {
-            vcycle_launch(p, v, s, z, df, H.gstream);
+            vcycle_launch(p, v, s, z, df, w, H.gstream);
         } catch (...) {
             cudaGraph_t tmp;
             cudaStreamEndCapture(H.gstream, &tmp);
