@@ -251,8 +251,8 @@ def kernel_source_hash(kind="cheb_fine"):
         return _source_parts("spmv.cu", (("// w[c] = sum_k z_k tau_r^k x^k[c]",
                                           "// g^k = m + tau_r^k a per stored entry"),))
     return _source_parts("vcycle.cu", (("// Row product of a sliced-ELL operator", "// Field t of a CSR row product"),
-                                       ("// Chebyshev step: r = b - A x_in",
-                                        "template <class T, int L>\n__global__ void __launch_bounds__(128) k_cheb_csr")))
+                                       ("// Where the finest level's last smoothing step puts",
+                                        "template <class T, int L, bool OUT>\n__global__ void __launch_bounds__(128) k_cheb_csr")))
 
 
 def fp64_peak_tflops(torch):
