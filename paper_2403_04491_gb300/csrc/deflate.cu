@@ -21,9 +21,9 @@
 // Costs. A applied to a piecewise-constant potential is nonzero only through the membrane and
 // pin terms: the same-region row sums of e^k (and of a) vanish except at the active rows, the membrane
 // nodes and the pinned node with its neighbours, since every assembled diagonal is minus its row's sum.
-// So A Z y is formed at the active rows alone (a few percent of the nodes): their row sums times the
-// constant of their own region, plus their cross-region entries times the constants of their cells.
-// The row sums are formed once per step (RS, three values per active row), E is an arrowhead matrix
+// So A Z y is nonzero at the active rows alone (a few percent of the nodes), and there it is a fixed
+// combination of two constants, the node's own group's and the one on the membrane's other side; the
+// eight coefficients of an active row are formed once per step. E is an arrowhead matrix
 // (cells couple only to the extracellular space) solved by its Schur complement on the device, and each
 // application adds a gather and a small solve; the right-hand-side pass and the update run inside the
 // V-cycle's first and last kernels (CG(P_0) keeps them as separate passes).
@@ -59,68 +59,81 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return s;   // valid in thread 0
 }
 
-// RS[q][k] = sum of the same-region e^k values of active row q over phi columns other than the pin;
-// RSa[q] the same sum of the static stiffness a (for the transposed operator's concentration rows)
-__global__ void k_defl_rowsums(int64_t na, int32_t pin, const int32_t* __restrict__ rows,
-                               const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ col,
-                               const double* __restrict__ e, int64_t ne, const double* __restrict__ a,
-                               double* __restrict__ RS, double* __restrict__ RSa) {
+// Coefficients of active row i, formed once per step: (A Z y)_f = C[f] y_own + C[4 + f] y_cross for its
+// four fields f, and (A^T Z y)_f likewise with CT. A Z y: the row's same-region phi columns other than
+// the pin hold its own group's constant (sums of e^k), its cross-region entries that of the one group on
+// the membrane's other side (a membrane node touches one cell only, so all its entries share it; xgrp);
+// the potential row is sum_k z_k of the concentration rows' terms. A^T Z y: tau_r^k z_k times the row
+// sum of a on the concentrations, sum_k z_k e^k and, through the transposed list, sum_k z_k xe^k on the
+// potential. The pinned potential row (the identity) gives 0.
+__global__ void k_defl_coefs(int64_t na, int64_t N_i, int32_t pin, const int32_t* __restrict__ rows,
+                             const int64_t* __restrict__ slice_ptr, const int32_t* __restrict__ col,
+                             const double* __restrict__ e, int64_t ne, const double* __restrict__ a,
+                             const int32_t* __restrict__ xptr, const int32_t* __restrict__ xcol,
+                             const int32_t* __restrict__ xtptr, const int32_t* __restrict__ xtrow,
+                             const int32_t* __restrict__ xtidx, const double* __restrict__ xe, int64_t n_cross,
+                             double z0, double z1, double z2, RegionCoef ri, RegionCoef re, double* __restrict__ C,
+                             double* __restrict__ CT) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= na) return;
     const int64_t r = rows[i];
     const int64_t s = r / SELL_C, base = slice_ptr[s] + r % SELL_C;
     const int w = (int)((slice_ptr[s + 1] - slice_ptr[s]) / SELL_C);
-    double acc[KI] = {0, 0, 0}, sa = 0.0;
+    const double z[KI] = {z0, z1, z2};
+    double own[KI] = {0, 0, 0}, cross[KI] = {0, 0, 0}, sa = 0.0, ct = 0.0;
     for (int k = 0; k < w; ++k) {
         const int64_t pos = base + k * SELL_C;
         if (col[pos] == pin) continue;
-        for (int q = 0; q < KI; ++q) acc[q] += e[q * ne + pos];
+        for (int q = 0; q < KI; ++q) own[q] += e[q * ne + pos];
         sa += a[pos];
     }
-    for (int q = 0; q < KI; ++q) RS[3 * i + q] = acc[q];
-    RSa[i] = sa;
+    for (int t = xptr[r]; t < xptr[r + 1]; ++t) {
+        if (xcol[t] == pin) continue;
+        for (int q = 0; q < KI; ++q) cross[q] += xe[q * n_cross + t];
+    }
+    for (int t = xtptr[r]; t < xtptr[r + 1]; ++t) {
+        if (xtrow[t] == pin) continue;
+        const int64_t idx = xtidx[t];
+        for (int q = 0; q < KI; ++q) ct += z[q] * xe[q * n_cross + idx];
+    }
+    const bool in = r < N_i, free = r != pin;
+    double* c = C + 8 * i;
+    double* t = CT + 8 * i;
+    double po = 0.0, pc = 0.0;
+    for (int q = 0; q < KI; ++q) {
+        c[q] = own[q];
+        c[4 + q] = cross[q];
+        po += z[q] * own[q];
+        pc += z[q] * cross[q];
+        t[q] = (in ? ri.tau[q] : re.tau[q]) * z[q] * sa;
+        t[4 + q] = 0.0;
+    }
+    c[3] = t[3] = free ? po : 0.0;
+    c[7] = free ? pc : 0.0;
+    t[7] = free ? ct : 0.0;
 }
 
-// group of the source row of every transposed cross entry (-1: the pinned node)
-__global__ void k_defl_xtg(int64_t nx, int64_t N_i, int32_t pin, const int32_t* __restrict__ xtrow,
-                           const int32_t* __restrict__ rgrp, int32_t ext_group, int32_t* __restrict__ xtg) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nx) return;
-    const int32_t j = xtrow[t];
-    xtg[t] = j == pin ? -1 : (j < N_i ? rgrp[j] : ext_group);
-}
-
-// Chunk b of a cell group's active rows (one block): its share of E_jj, E_je and E_ej of E = Z^T A Z.
-// Potential-row coefficient of a stored entry: sum_k z_k e^k (same region) or sum_k z_k xe^k (cross
-// region). Blocks from nchunks on: one chunk each of the extracellular active rows' share of E_ee.
+// Chunk b of a cell group's active rows (one block): its share of E_jj, E_je and E_ej of E = Z^T A Z,
+// the sums of the potential rows' coefficients of A Z and (for E_ej) of A^T Z. Blocks from nchunks on:
+// one chunk each of the extracellular active rows' share of E_ee.
 __global__ void __launch_bounds__(DT) k_defl_E(int nchunks, const int64_t* __restrict__ cbeg,
                                                const int32_t* __restrict__ aidx, int64_t ext0, int64_t na,
-                                               const int32_t* __restrict__ rows, const double* __restrict__ RS,
-                                               const int32_t* __restrict__ xptr, const int32_t* __restrict__ xg,
-                                               const int32_t* __restrict__ xtptr, const int32_t* __restrict__ xtrow,
-                                               const int32_t* __restrict__ xtidx, const double* __restrict__ xe,
-                                               int64_t n_cross, int32_t pin, double z0, double z1, double z2,
-                                               int32_t ext_group, double* __restrict__ part) {
+                                               const double* __restrict__ C, const double* __restrict__ CT,
+                                               double* __restrict__ part) {
     __shared__ double sh[DT / 32];
     const int b = blockIdx.x;
     double djj = 0.0, dje = 0.0, dej = 0.0;
     if (b < nchunks) {
         const int64_t q = cbeg[b] + threadIdx.x;
         if (q < cbeg[b + 1]) {
-            const int64_t i = aidx[q], r = rows[i];
-            djj = z0 * RS[3 * i] + z1 * RS[3 * i + 1] + z2 * RS[3 * i + 2];
-            for (int t = xptr[r]; t < xptr[r + 1]; ++t)
-                if (xg[t] == ext_group) dje += z0 * xe[t] + z1 * xe[n_cross + t] + z2 * xe[2 * n_cross + t];
-            // column r of the cross part: rows of the extracellular space (the pinned one left out)
-            for (int t = xtptr[r]; t < xtptr[r + 1]; ++t) {
-                if (xtrow[t] == pin) continue;
-                const int64_t idx = xtidx[t];
-                dej += z0 * xe[idx] + z1 * xe[n_cross + idx] + z2 * xe[2 * n_cross + idx];
-            }
+            const int64_t i = aidx[q];
+            djj = C[8 * i + 3];
+            dje = C[8 * i + 7];
+            dej = CT[8 * i + 7];
         }
     } else {
         const int64_t i = ext0 + (b - nchunks) * (int64_t)DT + threadIdx.x;
-        if (i < na && rows[i] != pin) djj = z0 * RS[3 * i] + z1 * RS[3 * i + 1] + z2 * RS[3 * i + 2];
+        if (i < na) djj = C[8 * i + 3];
     }
     double a = block_sum(djj, sh);
     if (threadIdx.x == 0) part[3 * b] = a;
@@ -254,10 +267,8 @@ struct Deflation {
     DArray<int32_t> rows;             // active rows (increasing)
     DArray<int32_t> act;              // node -> its index in rows, -1 if not active
     DArray<int32_t> rgrp;             // intracellular node -> its group
-    DArray<int32_t> xg;               // cross entry -> group of its column (-1: the pinned node)
-    DArray<double> RS;                // [na][3] row sums of e^k over phi columns (per step)
-    DArray<double> RSa;               // [na] row sums of a over phi columns (the transposed operator)
-    DArray<int32_t> xtg;              // transposed cross entry -> group of its source row (-1: pin)
+    DArray<int32_t> xgrp;             // active row -> group on the membrane's other side
+    DArray<double> C, CT;             // [na][8] coefficients of A Z y and A^T Z y (per step)
     DArray<double> iEjj, Eje, Eej;    // the arrowhead E (per step): 1 / E_jj, E_je, E_ej
     DArray<double> Ee;                // {E_ee, 1 / Schur complement}
     DArray<double> y, gpart, epart;
@@ -338,23 +349,24 @@ static Deflation& deflation_setup(knp_problem* p) {
     d->ebeg.upload(beg, st);
     d->ecell.upload(first, st);
     const int32_t ext = d->nc;
-    std::vector<int32_t> xg(std::max<size_t>(p->h_xcol.size(), 1), -1);
-    for (size_t t = 0; t < p->h_xcol.size(); ++t) {
-        const int32_t c = p->h_xcol[t];
-        xg[t] = c == p->pin ? -1 : (c < p->N_i ? rg[c] : ext);
+    std::vector<int32_t> xgrp(d->na, 0);   // rows without a usable cross entry have zero coefficients
+    for (int64_t i = 0; i < d->na; ++i) {
+        int32_t group = -1;
+        for (int32_t t = p->h_xptr[rows[i]]; t < p->h_xptr[rows[i] + 1]; ++t) {
+            const int32_t c = p->h_xcol[t];
+            if (c == p->pin) continue;
+            const int32_t gc = c < p->N_i ? rg[c] : ext;
+            KNP_REQUIRE(group < 0 || group == gc, KNP_ERR_INVALID_MESH, "a membrane node touches two cells");
+            group = gc;
+        }
+        if (group >= 0) xgrp[i] = group;
     }
     d->rows.upload(rows, st);
     d->act.upload(act, st);
     d->rgrp.upload(rg, st);
-    d->xg.upload(xg, st);
-    d->RS.alloc(3 * d->na);
-    d->RSa.alloc(d->na);
-    const int64_t nx = (int64_t)p->h_xcol.size();
-    d->xtg.alloc(std::max<int64_t>(nx, 1));
-    if (nx) {
-        k_defl_xtg<<<nbk(nx, 256), 256, 0, st>>>(nx, p->N_i, p->pin, p->xtrow.p, d->rgrp.p, ext, d->xtg.p);
-        count_launch();
-    }
+    d->xgrp.upload(xgrp, st);
+    d->C.alloc(8 * d->na);
+    d->CT.alloc(8 * d->na);
     for (DArray<double>* a : {&d->iEjj, &d->Eje, &d->Eej}) a->alloc(std::max(d->nc, 1));
     d->Ee.alloc(2);
     d->y.alloc(d->nc + 1);
@@ -373,11 +385,11 @@ void deflation_prepare(knp_problem* p) {
     const int64_t nx = (int64_t)p->h_xcol.size();
     const double* z = p->sp.z;
     count_launch(3);
-    k_defl_rowsums<<<nbk(d.na, 64), 64, 0, st>>>(d.na, p->pin, d.rows.p, p->sell.slice_ptr.p, p->sell.col.p,
-                                                 p->sell_e.p, p->sell.n_entries, p->sell_a.p, d.RS.p, d.RSa.p);
-    k_defl_E<<<d.echunks + d.eext, DT, 0, st>>>(d.echunks, d.ebeg.p, d.aidx.p, d.na_i, d.na, d.rows.p, d.RS.p,
-                                                p->xptr.p, d.xg.p, p->xtptr.p, p->xtrow.p, p->xtidx.p, p->xe.p, nx,
-                                                p->pin, z[0], z[1], z[2], d.nc, d.epart.p);
+    k_defl_coefs<<<nbk(d.na, 64), 64, 0, st>>>(d.na, p->N_i, p->pin, d.rows.p, p->sell.slice_ptr.p, p->sell.col.p,
+                                               p->sell_e.p, p->sell.n_entries, p->sell_a.p, p->xptr.p, p->xcol.p,
+                                               p->xtptr.p, p->xtrow.p, p->xtidx.p, p->xe.p, nx, z[0], z[1], z[2],
+                                               p->sp.reg[0], p->sp.reg[1], d.C.p, d.CT.p);
+    k_defl_E<<<d.echunks + d.eext, DT, 0, st>>>(d.echunks, d.ebeg.p, d.aidx.p, d.na_i, d.na, d.C.p, d.CT.p, d.epart.p);
     k_defl_schur<<<1, DT, 0, st>>>(d.nc, d.echunks, d.eext, d.ecell.p, d.epart.p, d.iEjj.p, d.Eje.p, d.Eej.p, d.Ee.p);
     KNP_CUDA(cudaGetLastError());
     d.built_for = p->assembly_id;
@@ -398,22 +410,13 @@ void deflated_precond_apply(knp_problem* p, const double* v, const double* s, do
     DeflFuse df;
     df.rgrp = d.rgrp.p;
     df.act = d.act.p;
-    df.RS = d.RS.p;
-    df.RSa = d.RSa.p;
-    df.xptr = transpose ? p->xtptr.p : p->xptr.p;
-    df.xg = transpose ? d.xtg.p : d.xg.p;
-    df.xidx = transpose ? p->xtidx.p : nullptr;
-    df.xe = p->xe.p;
+    df.C = transpose ? d.CT.p : d.C.p;
+    df.xgrp = d.xgrp.p;
     df.y = d.y.p;
-    df.n_cross = (int64_t)p->h_xcol.size();
     df.N_i = p->N_i;
     df.pin = p->pin;
     df.ext_group = d.nc;
     df.transpose = transpose;
-    for (int q = 0; q < 3; ++q) {
-        df.z[q] = p->sp.z[q];
-        for (int r = 0; r < 2; ++r) df.ztau[r][q] = p->sp.z[q] * p->sp.reg[r].tau[q];
-    }
     if (p->amg->inner_cg_max_it == 0) {
         // one V-cycle: its first kernel forms s .* v - A Z y and its output kernel adds Z y
         vcycle_apply(p, v, s, z, &df, w);

@@ -15,18 +15,12 @@ namespace knp {
 struct DeflFuse {
     const int32_t* rgrp = nullptr;   // intracellular node -> its cell group
     const int32_t* act = nullptr;    // node -> active row, -1 where A Z y is zero
-    const double* RS = nullptr;      // [active rows][3] row sums of e^k over phi columns
-    const double* RSa = nullptr;     // [active rows] row sums of a over phi columns
-    const int32_t* xptr = nullptr;   // cross-region entries of each row (of A^T: transposed list)
-    const int32_t* xg = nullptr;     // cross entry -> group of its column (-1: the pinned node)
-    const int32_t* xidx = nullptr;   // transposed: entry -> index of its value
-    const double* xe = nullptr;      // [3][n_cross] cross-region values
+    const double* C = nullptr;       // [active rows][8] coefficients of A Z y (or A^T Z y)
+    const int32_t* xgrp = nullptr;   // active row -> group on the membrane's other side
     const double* y = nullptr;       // [groups + 1] the coarse solution, extracellular group last
-    int64_t n_cross = 0, N_i = 0;
+    int64_t N_i = 0;
     int32_t pin = -1, ext_group = 0;
     int32_t transpose = 0;           // A^T Z y in place of A Z y
-    double z[3] = {0, 0, 0};         // valences
-    double ztau[2][3] = {};          // z_k tau_r^k
 };
 
 // One captured V-cycle: a CUDA graph instantiated for a given (input, scale, output) triple.
