@@ -176,9 +176,10 @@ __global__ void __launch_bounds__(DT) k_defl_schur(int nc, int nchunks, int next
 // the others shares of the extracellular potentials (pin left out)
 __global__ void __launch_bounds__(DT) k_defl_gather(int nchunks, const int64_t* __restrict__ cbeg,
                                                     const int32_t* __restrict__ cnodes, int64_t N_i, int64_t n,
-                                                    int32_t pin, const double* __restrict__ v,
+                                                    int32_t pin, const double* v,
                                                     const double* __restrict__ s, double* __restrict__ part) {
     __shared__ double sh[DT / 32];
+    chain_wait();
     double acc = 0.0;
     if ((int)blockIdx.x < nchunks) {
         const int64_t end = cbeg[blockIdx.x + 1];
@@ -199,11 +200,12 @@ __global__ void __launch_bounds__(DT) k_defl_gather(int nchunks, const int64_t* 
 // y_j = (g_j - E_je y_e) / E_jj; y[nc] = y_e. The division by E_jj and S_e is a product with their
 // reciprocals, formed once per step (an FP64 division is a chain of some 20 instructions).
 __global__ void __launch_bounds__(DT) k_defl_solve(int nc, int nchunks, int next, const int32_t* __restrict__ cchunk,
-                                                   const double* __restrict__ part, const double* __restrict__ iEjj,
-                                                   const double* __restrict__ Eje, const double* __restrict__ Eej,
-                                                   const double* __restrict__ Ee, double* __restrict__ y) {
+                                                   const double* part, const double* iEjj,
+                                                   const double* Eje, const double* Eej, const double* Ee,
+                                                   double* y) {
     __shared__ double sh[DT / 32];
     __shared__ double ye_s;
+    chain_wait();
     double a = 0.0;
     for (int q = threadIdx.x; q < next; q += DT) a += part[nchunks + q];
     // a thread per cell, or a warp where cells have many chunks: g_j (kept in y until the solve)

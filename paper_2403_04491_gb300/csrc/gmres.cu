@@ -118,7 +118,7 @@ __device__ __forceinline__ void block_reduce_store(const double (&acc)[NT], doub
 
 // out[k] = sum over blocks of partial[k * PART_LD + b], k < nt, by one block of RED_THREADS: each
 // warp takes four sums at a time. Every block of a kernel gets the same bits. out is shared memory.
-__device__ __forceinline__ void sum_partials(const double* __restrict__ partial, int nblocks, int nt, double* out) {
+__device__ __forceinline__ void sum_partials(const double* partial, int nblocks, int nt, double* out) {
     const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
     for (int k0 = 4 * wid; k0 < nt; k0 += 4 * (RED_THREADS / 32)) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -134,7 +134,7 @@ __device__ __forceinline__ void sum_partials(const double* __restrict__ partial,
 }
 
 // Two neighbouring elements of a vector; vectors are 4 n doubles, 16-byte aligned
-__device__ __forceinline__ double2 ld2(const double* __restrict__ p, int64_t i2) {
+__device__ __forceinline__ double2 ld2(const double* p, int64_t i2) {
     return reinterpret_cast<const double2*>(p)[i2];
 }
 __device__ __forceinline__ void st2(double* __restrict__ p, int64_t i2, double2 v) {
@@ -147,8 +147,9 @@ constexpr int PAIRS = NV <= 3 ? 4 : NV <= 7 ? 2 : 1;
 
 // partial sums of <V_k, w> for k < NV, and of <w, w> at k = NV
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS, 1) k_mdot(int64_t n4, const double* __restrict__ V, int64_t ldv,
-                                                         const double* __restrict__ w, double* __restrict__ partial) {
+__global__ void __launch_bounds__(RED_THREADS, 1) k_mdot(int64_t n4, const double* V, int64_t ldv,
+                                                         const double* w, double* __restrict__ partial) {
+    chain_wait();
     constexpr int E = PAIRS<NV>;
     double acc[NV + 1];
 #pragma unroll
@@ -284,14 +285,14 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_combo_norms(int64_t n4, cons
 // 85-99% of the steps, and FP64 issue (not bandwidth) bounds these kernels on GB300.
 constexpr double REORTH_KEEP = 1e-4;
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, const double* __restrict__ V,
-                                                                    int64_t ldv, const double* __restrict__ pdots,
-                                                                    int nblocks, double* __restrict__ dots,
-                                                                    double* __restrict__ w,
+__global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, const double* V,
+                                                                    int64_t ldv, const double* pdots,
+                                                                    int nblocks, double* __restrict__ dots, double* w,
                                                                     double* __restrict__ partial) {
     constexpr int E = PAIRS<NV>;
     __shared__ double h[NV + 1];
     __shared__ int second_s;
+    chain_wait();
     sum_partials(pdots, nblocks, NV + 1, h);
     if (threadIdx.x == 0) {
         double hh = 0.0;
@@ -366,14 +367,15 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, 
 // Block 0 stores h2 to dots2.
 constexpr double ORTH_SKIP = 1e-10;
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const double* __restrict__ V, int64_t ldv,
-                                                            const double* __restrict__ pdots, int nblocks,
-                                                            const double* __restrict__ second,
-                                                            double* __restrict__ dots2, double* __restrict__ w,
+__global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const double* V, int64_t ldv,
+                                                            const double* pdots, int nblocks,
+                                                            const double* second,
+                                                            double* __restrict__ dots2, double* w,
                                                             double* __restrict__ flag) {
     __shared__ double h2[NV + 1];
     __shared__ double inv_s;
     __shared__ int skip_s;
+    chain_wait();
     if (second[0] != 0.0) {
         sum_partials(pdots, nblocks, NV + 1, h2);
     } else {
@@ -460,11 +462,11 @@ unsigned vec_grid(int64_t n4) {
     X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16) X(17) X(18) X(19) \
     X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30) X(31)
 
-#define KNP_NV_CASE_k_mdot(N) case N: k_mdot<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_mdot(N) case N: launch(k_mdot<N>, nb_red, RED_THREADS, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_combo_norms2(N) case N: k_combo_norms<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 #define KNP_NV_CASE_k_combo_norms3(N) case N: k_combo_norms<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_orth_update_dot(N) case N: k_orth_update_dot<N><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_orth_final(N) case N: k_orth_final<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_update_dot(N) case N: launch(k_orth_update_dot<N>, nb_red, RED_THREADS, q, KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec, RED_THREADS, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_update_x(N) case N: k_update_x<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 // Launch KERNEL<nv> with the caller's grid (nb_red or nb_vec) for a runtime nv in [0, 31]
 #define KNP_LAUNCH_NV(nv, KERNEL)                                                                    \
@@ -547,15 +549,15 @@ static double norm2_dev(GmresWork& g, const double* v, cudaStream_t st) {
 
 // w = S^-1 A z_j into V_{j+1}, orthogonalised against V_0..V_j (CGS2, second pass skipped on the
 // device when it has nothing to remove) and normalised; the dots of both passes land in g.dots
-static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready, cudaStream_t st) {
+static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready, const Queue& q) {
     const int64_t n4 = g.n4;
     const int nv = j + 1;
     const int nb_red = red_grid(n4);
     const unsigned nb_vec = vec_grid(n4);
     double* zj = g.Z.p + (int64_t)j * n4;
     double* w = g.V.p + (int64_t)(j + 1) * n4;
-    op_apply(p, zj, w, p->sinv.p, nullptr, transpose, st, w_ready);
-    ProfScope ps(&p->prof, KC_ORTHO, st);
+    op_apply(p, zj, w, p->sinv.p, nullptr, transpose, q, w_ready);
+    ProfScope ps(&p->prof, KC_ORTHO, q.st);
     count_launch(3);
 #define KNP_ARGS n4, g.V.p, n4, w, g.pass1()
     KNP_LAUNCH_NV(nv, k_mdot);
@@ -579,7 +581,7 @@ static void arnoldi_graph_launch(knp_problem* p, GmresWork& g, int j, bool trans
         const int64_t before = g_launches.load();
         KNP_CUDA(cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal));
         try {
-            arnoldi_kernels(p, g, j, transpose, w_ready, g.cap);
+            arnoldi_kernels(p, g, j, transpose, w_ready, Queue(g.cap, true));
             KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, g.cap));
         } catch (...) {
             cudaGraph_t tmp = nullptr;

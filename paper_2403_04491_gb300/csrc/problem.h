@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "common.h"
+#include "launch.h"
 #include "profile.h"
 
 namespace knp {
@@ -202,9 +203,9 @@ void adjoint_get(knp_problem* P, bool device, double* dLdu0, double* dLdw0, doub
 // y = A x (unscaled), or with row scaling / residual; see spmv.cu
 // stands for "the problem's own stream" in stream arguments
 inline const cudaStream_t kProblemStream = reinterpret_cast<cudaStream_t>(~uintptr_t(0));
-// (on `st`, or on the problem's stream when st is the default argument); w_ready: p->op_w holds x's w
+// (on `q`, or on the problem's stream when q is the default argument); w_ready: p->op_w holds x's w
 void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale, const double* b,
-              bool transpose = false, cudaStream_t st = kProblemStream, bool w_ready = false);
+              bool transpose = false, Queue q = kProblemStream, bool w_ready = false);
 // whether the forward product reads p->op_w (one thread per row)
 bool op_reads_w(const knp_problem* p);
 // the static per-ion values of the forward product (after the pattern and m, a are on the device)

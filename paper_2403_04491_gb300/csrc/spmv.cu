@@ -24,6 +24,7 @@
 #include <algorithm>
 
 #include "lanes.h"
+#include "launch.h"
 #include "problem.h"
 
 namespace knp {
@@ -52,7 +53,8 @@ struct OpArgs {
 };
 
 // w[c] = sum_k z_k tau_r^k x^k[c], r the region of node c
-__global__ void k_op_w(OpArgs A, const double* __restrict__ x, double* __restrict__ w) {
+__global__ void k_op_w(OpArgs A, const double* x, double* __restrict__ w) {
+    chain_wait();
     int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (c >= A.n) return;
     const int reg = c < A.N_i ? 0 : 1;
@@ -64,7 +66,7 @@ __global__ void k_op_w(OpArgs A, const double* __restrict__ x, double* __restric
 // y = rowscale .* (b - A x)  (b, rowscale optional) on the fields of row r that a lane holds in out
 template <int F>
 __device__ __forceinline__ void op_store(int64_t k, const double* out, double* __restrict__ y,
-                                         const double* __restrict__ rowscale, const double* __restrict__ b) {
+                                         const double* __restrict__ rowscale, const double* b) {
     double o[F];
 #pragma unroll
     for (int f = 0; f < F; ++f) {
@@ -89,8 +91,8 @@ __device__ __forceinline__ void op_store(int64_t k, const double* out, double* _
 template <int L>
 constexpr int OP_BATCH = L == 1 ? 1 : 3;
 template <int L>
-__global__ void __launch_bounds__(128) k_op_apply(OpArgs A, const double* __restrict__ x, double* __restrict__ y,
-                                                  const double* __restrict__ rowscale, const double* __restrict__ b) {
+__global__ void __launch_bounds__(128) k_op_apply(OpArgs A, const double* x, double* __restrict__ y,
+                                                  const double* __restrict__ rowscale, const double* b) {
     constexpr int F = LANE_FIELDS<L>, U = OP_BATCH<L>;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t r = gid / L;
@@ -108,6 +110,7 @@ __global__ void __launch_bounds__(128) k_op_apply(OpArgs A, const double* __rest
     int32_t c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = t + u * L < w ? cp[(t + u * L) * SELL_C] : 0;
+    chain_wait();
     for (int k = t; k < w; k += U * L) {
         double2 x01[U], x23[U];
         double gv[U][KI], ev[U][KI], av[U], wv[U];
@@ -183,9 +186,8 @@ __global__ void k_fold_g(int64_t n, int64_t N_i, int64_t ne, const int64_t* __re
 //     c^k row:  (m + tau^k a) x^k_j + z_k tau^k a x^phi_j,   phi row:  sum_k e^k (x^k_j + z_k x^phi_j)
 // with m, a, e symmetric on same-region entries; the cross-region part uses the transposed list.
 template <int L>
-__global__ void __launch_bounds__(128) k_op_apply_t(OpArgs A, const double* __restrict__ x, double* __restrict__ y,
-                                                    const double* __restrict__ rowscale,
-                                                    const double* __restrict__ b) {
+__global__ void __launch_bounds__(128) k_op_apply_t(OpArgs A, const double* x, double* __restrict__ y,
+                                                    const double* __restrict__ rowscale, const double* b) {
     constexpr int F = LANE_FIELDS<L>, U = OP_BATCH<L>;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t r = gid / L;
@@ -203,6 +205,7 @@ __global__ void __launch_bounds__(128) k_op_apply_t(OpArgs A, const double* __re
     int32_t c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = t + u * L < w ? cp[(t + u * L) * SELL_C] : 0;
+    chain_wait();
     for (int k = t; k < w; k += U * L) {
         double2 x01[U], x23[U];
         double ev[U][KI], mv[U], av[U];
@@ -261,8 +264,8 @@ static int op_lanes(const knp_problem* p) {
 bool op_reads_w(const knp_problem* p) { return op_lanes(p) == 1; }
 
 void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale, const double* b, bool transpose,
-              cudaStream_t st, bool w_ready) {
-    if (st == kProblemStream) st = p->stream;
+              Queue q, bool w_ready) {
+    if (q.st == kProblemStream) q.st = p->stream;
     OpArgs A;
     A.n = p->n_nodes;
     A.N_i = p->N_i;
@@ -287,25 +290,25 @@ void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale
     for (int k = 0; k < KI; ++k) A.z[k] = p->sp.z[k];
     const int lanes = op_lanes(p);
     const unsigned blocks = (unsigned)((A.n * lanes + 127) / 128);
-    ProfScope ps(&p->prof, KC_SPMV, st);
+    ProfScope ps(&p->prof, KC_SPMV, q.st);
     count_launch();
     if (transpose) {
         if (lanes == 1)
-            k_op_apply_t<1><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+            launch(k_op_apply_t<1>, blocks, 128, q, A, x, y, rowscale, b);
         else if (lanes == 4)
-            k_op_apply_t<4><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+            launch(k_op_apply_t<4>, blocks, 128, q, A, x, y, rowscale, b);
         else
-            k_op_apply_t<8><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+            launch(k_op_apply_t<8>, blocks, 128, q, A, x, y, rowscale, b);
     } else if (lanes == 1) {
         if (!w_ready) {
             count_launch();
-            k_op_w<<<(unsigned)((A.n + 255) / 256), 256, 0, st>>>(A, x, p->op_w.p);
+            launch(k_op_w, (A.n + 255) / 256, 256, q, A, x, p->op_w.p);
         }
-        k_op_apply<1><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+        launch(k_op_apply<1>, blocks, 128, q, A, x, y, rowscale, b);
     } else if (lanes == 4) {
-        k_op_apply<4><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+        launch(k_op_apply<4>, blocks, 128, q, A, x, y, rowscale, b);
     } else {
-        k_op_apply<8><<<blocks, 128, 0, st>>>(A, x, y, rowscale, b);
+        launch(k_op_apply<8>, blocks, 128, q, A, x, y, rowscale, b);
     }
     KNP_CUDA(cudaGetLastError());
 }

@@ -24,6 +24,7 @@
 #include "amg_gpu.h"
 #include "deflate_input.h"
 #include "lanes.h"
+#include "launch.h"
 #include "problem.h"
 #include "vcycle.h"
 
@@ -100,7 +101,7 @@ struct VN {
 template <class T, int L>
 __device__ __forceinline__ void sell_row(int64_t r, int t, const int64_t* __restrict__ sp,
                                          const int32_t* __restrict__ col, const T* __restrict__ val,
-                                         const T* __restrict__ x, T acc[4]) {
+                                         const T* x, T acc[4]) {
     const int64_t s = r / SELL_C;
     const int64_t base = sp[s] + r % SELL_C;
     const int w = (int)((sp[s + 1] - sp[s]) / SELL_C);
@@ -111,6 +112,7 @@ __device__ __forceinline__ void sell_row(int64_t r, int t, const int64_t* __rest
     int32_t c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = t + u * L < w ? cp[(t + u * L) * SELL_C] : 0;
+    chain_wait();
     for (int k = t; k < w; k += U * L) {
         V4<T> a[U], xv[U];
 #pragma unroll
@@ -149,24 +151,26 @@ constexpr int CSR_BATCH = L == 4 ? 2 : 4;   // many rows: registers for more blo
 template <class T, int L>
 __device__ __forceinline__ T csr_row_field(bool active, int64_t r, int t, const int64_t* __restrict__ ptr,
                                            const int32_t* __restrict__ col, const T* __restrict__ val,
-                                           const T* __restrict__ x) {
+                                           const T* x) {
     static_assert(L == 4 || L == 8 || L == 16 || L == 32 || L == 128, "lanes per row");
     constexpr int U = CSR_BATCH<L>;
     T acc[4] = {T(0), T(0), T(0), T(0)}, out[1];
+    const int64_t t0 = active ? ptr[r] + t : 0, t1 = active ? ptr[r + 1] : 0;
+    int32_t c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = t0 + u * L < t1 ? col[t0 + u * L] : 0;
+    chain_wait();
     if (active) {
-        const int64_t t1 = ptr[r + 1];
-        for (int64_t q = ptr[r] + t; q < t1; q += U * L) {
-            int32_t c[U];
+        for (int64_t q = t0; q < t1; q += U * L) {
             V4<T> a[U], xv[U];
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (q + u * L < t1) {
-                    c[u] = col[q + u * L];
                     a[u] = V4<T>::load(val + 4 * (q + u * L));
+                    xv[u] = V4<T>::load(x + 4 * (int64_t)c[u]);
                 }
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (q + u * L < t1) xv[u] = V4<T>::load(x + 4 * (int64_t)c[u]);
+            for (int u = 0; u < U; ++u) c[u] = q + (U + u) * L < t1 ? col[q + (U + u) * L] : 0;
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (q + u * L < t1)
@@ -187,11 +191,13 @@ __device__ __forceinline__ T csr_row_field(bool active, int64_t r, int t, const 
 // first Chebyshev step from x = 0: d = c2 D^-1 b, x = d (d stored if a second step reads it). On the finest level b = s .* v (double
 // input), or s .* v - A Z y inside the coarse correction (df.y set).
 template <class T>
-__global__ void k_cheb_first(int64_t n, const double* __restrict__ v, const double* __restrict__ s, T* __restrict__ b,
+__global__ void k_cheb_first(int64_t n, const double* v, const double* __restrict__ s, T* b,
                              const T* __restrict__ dinv, Coef4 c, T* __restrict__ x, T* __restrict__ d, DeflFuse df,
                              int write_d) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
+    V4<T> di = V4<T>::load(dinv + 4 * i), dd;
+    chain_wait();
     V4<T> bb;
     if (v && df.y) {
         double t[4];
@@ -204,7 +210,6 @@ __global__ void k_cheb_first(int64_t n, const double* __restrict__ v, const doub
     } else {
         bb = V4<T>::load(b + 4 * i);
     }
-    V4<T> di = V4<T>::load(dinv + 4 * i), dd;
     for (int f = 0; f < 4; ++f) dd.v[f] = (T)c.c2[f] * di.v[f] * bb.v[f];
     if (write_d) dd.store(d + 4 * i);
     dd.store(x + 4 * i);
@@ -247,8 +252,8 @@ __device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0,
 template <class T, int L, bool OUT>
 __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __restrict__ sp,
                                                    const int32_t* __restrict__ col, const T* __restrict__ val,
-                                                   const T* __restrict__ x_in, const T* __restrict__ b,
-                                                   const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
+                                                   const T* x_in, const T* b,
+                                                   const T* __restrict__ dinv, Coef4 c, T* d,
                                                    T* __restrict__ x_out, int read_d, int write_d, VcycleOut out) {
     constexpr int F = LANE_FIELDS<L>;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -280,8 +285,8 @@ __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __r
 template <class T, int L, bool OUT>
 __global__ void __launch_bounds__(128) k_cheb_csr(int64_t n, const int64_t* __restrict__ ptr,
                                                   const int32_t* __restrict__ col, const T* __restrict__ val,
-                                                  const T* __restrict__ x_in, const T* __restrict__ b,
-                                                  const T* __restrict__ dinv, Coef4 c, T* __restrict__ d,
+                                                  const T* x_in, const T* b,
+                                                  const T* __restrict__ dinv, Coef4 c, T* d,
                                                   T* __restrict__ x_out, int read_d, int write_d, VcycleOut out) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
     const int t = (int)(g % L);
@@ -303,8 +308,7 @@ __global__ void __launch_bounds__(128) k_cheb_csr(int64_t n, const int64_t* __re
 template <class T, int L>
 __global__ void __launch_bounds__(128) k_resid_sell(int64_t n, const int64_t* __restrict__ sp,
                                                     const int32_t* __restrict__ col, const T* __restrict__ val,
-                                                    const T* __restrict__ x, const T* __restrict__ b,
-                                                    T* __restrict__ y) {
+                                                    const T* x, const T* b, T* __restrict__ y) {
     constexpr int F = LANE_FIELDS<L>;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t i = g / L;
@@ -328,8 +332,7 @@ __global__ void __launch_bounds__(128) k_resid_sell(int64_t n, const int64_t* __
 template <class T, int L>
 __global__ void __launch_bounds__(128) k_resid_csr(int64_t n, const int64_t* __restrict__ ptr,
                                                    const int32_t* __restrict__ col, const T* __restrict__ val,
-                                                   const T* __restrict__ x, const T* __restrict__ b,
-                                                   T* __restrict__ r) {
+                                                   const T* x, const T* b, T* __restrict__ r) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
     const int t = (int)(g % L);
     const T acc = csr_row_field<T, L>(i < n, i, t, ptr, col, val, x);
@@ -340,7 +343,7 @@ __global__ void __launch_bounds__(128) k_resid_csr(int64_t n, const int64_t* __r
 template <class T, int L>
 __global__ void __launch_bounds__(128) k_csr4(int64_t n, const int64_t* __restrict__ ptr,
                                               const int32_t* __restrict__ col, const T* __restrict__ val,
-                                              const T* __restrict__ x, T* __restrict__ y) {
+                                              const T* x, T* __restrict__ y) {
     const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x), i = g / L;
     const int t = (int)(g % L);
     const T acc = csr_row_field<T, L>(i < n, i, t, ptr, col, val, x);
@@ -353,8 +356,7 @@ __global__ void __launch_bounds__(128) k_csr4(int64_t n, const int64_t* __restri
 template <class T, int L>
 __global__ void __launch_bounds__(128) k_prolong(int64_t n, const int64_t* __restrict__ sp,
                                                  const int32_t* __restrict__ col, const T* __restrict__ val,
-                                                 const int32_t* __restrict__ perm, const T* __restrict__ xc,
-                                                 T* __restrict__ x) {
+                                                 const int32_t* __restrict__ perm, const T* xc, T* x) {
     static_assert(L == 1 || L == 4, "threads per row");
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t q = g / L;
@@ -362,19 +364,25 @@ __global__ void __launch_bounds__(128) k_prolong(int64_t n, const int64_t* __res
     const int64_t s = q / SELL_C, base = sp[s] + q % SELL_C;
     const int w = (int)((sp[s + 1] - sp[s]) / SELL_C);
     const int64_t r = perm[q];
+    constexpr int U = L == 1 ? 2 : 4;
+    int32_t c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = u < w ? col[base + u * SELL_C] : 0;
+    chain_wait();
     if constexpr (L == 1) {
         V4<T> acc = V4<T>::load(x + 4 * r);
-        for (int k0 = 0; k0 < w; k0 += 2) {
-            V4<T> a[2], v[2];
+        for (int k0 = 0; k0 < w; k0 += U) {
+            V4<T> a[U], v[U];
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+            for (int u = 0; u < U; ++u)
                 if (k0 + u < w) {
-                    const int64_t pos = base + (k0 + u) * SELL_C;
-                    a[u] = V4<T>::load(val + 4 * pos);
-                    v[u] = V4<T>::load(xc + 4 * (int64_t)col[pos]);
+                    a[u] = V4<T>::load(val + 4 * (base + (k0 + u) * SELL_C));
+                    v[u] = V4<T>::load(xc + 4 * (int64_t)c[u]);
                 }
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+            for (int u = 0; u < U; ++u) c[u] = k0 + U + u < w ? col[base + (k0 + U + u) * SELL_C] : 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
                 if (k0 + u < w)
                     for (int f = 0; f < 4; ++f) acc.v[f] += a[u].v[f] * v[u].v[f];
         }
@@ -382,17 +390,18 @@ __global__ void __launch_bounds__(128) k_prolong(int64_t n, const int64_t* __res
     } else {
         const int f = (int)(g % L);
         T acc = x[4 * r + f];
-        for (int k0 = 0; k0 < w; k0 += 4) {
-            T a[4], v[4];
+        for (int k0 = 0; k0 < w; k0 += U) {
+            T a[U], v[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < U; ++u)
                 if (k0 + u < w) {
-                    const int64_t pos = base + (k0 + u) * SELL_C;
-                    a[u] = val[4 * pos + f];
-                    v[u] = xc[4 * (int64_t)col[pos] + f];
+                    a[u] = val[4 * (base + (k0 + u) * SELL_C) + f];
+                    v[u] = xc[4 * (int64_t)c[u] + f];
                 }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < U; ++u) c[u] = k0 + U + u < w ? col[base + (k0 + U + u) * SELL_C] : 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
                 if (k0 + u < w) acc += a[u] * v[u];
         }
         x[4 * r + f] = acc;
@@ -401,7 +410,8 @@ __global__ void __launch_bounds__(128) k_prolong(int64_t n, const int64_t* __res
 
 // x_f = Ainv_f b_f on the coarsest level, FP64; one warp per (field, row)
 template <class T>
-__global__ void k_coarse(int64_t nc, const double* __restrict__ inv, const T* __restrict__ b, T* __restrict__ x) {
+__global__ void k_coarse(int64_t nc, const double* __restrict__ inv, const T* b, T* __restrict__ x) {
+    chain_wait();
     int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
     int lane = threadIdx.x % 32;
     if (wid >= 4 * nc) return;
@@ -422,7 +432,8 @@ __global__ void k_to_double(int64_t n4, const T* __restrict__ x, double* __restr
 
 // the V-cycle's result from x (a single-level hierarchy)
 template <class T>
-__global__ void k_out(int64_t n, const T* __restrict__ x, VcycleOut out) {
+__global__ void k_out(int64_t n, const T* x, VcycleOut out) {
+    chain_wait();
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r < n) store_out<T, 4>(out, r, 0, VN<T, 4>::load(x + 4 * r));
 }
@@ -848,19 +859,19 @@ void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, in
 // CSR kernels with the matrix's lanes per row
 #define KNP_CSR_DISPATCH(lanes, KERNEL, rows, ...)                                                \
     switch (lanes) {                                                                              \
-        case 4: KERNEL(4)<<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
-        case 8: KERNEL(8)<<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;          \
-        case 16: KERNEL(16)<<<nblk((rows) * 16, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
-        case 32: KERNEL(32)<<<nblk((rows) * 32, 128), 128, 0, st>>>(__VA_ARGS__); break;       \
-        default: KERNEL(128)<<<nblk((rows) * 128, 128), 128, 0, st>>>(__VA_ARGS__); break;     \
+        case 4: launch(KERNEL(4), nblk((rows) * 4, 128), 128, q, __VA_ARGS__); break;             \
+        case 8: launch(KERNEL(8), nblk((rows) * 8, 128), 128, q, __VA_ARGS__); break;             \
+        case 16: launch(KERNEL(16), nblk((rows) * 16, 128), 128, q, __VA_ARGS__); break;          \
+        case 32: launch(KERNEL(32), nblk((rows) * 32, 128), 128, q, __VA_ARGS__); break;          \
+        default: launch(KERNEL(128), nblk((rows) * 128, 128), 128, q, __VA_ARGS__); break;        \
     }
 
 // sliced-ELL kernels with the level's lanes per row
 #define KNP_LANE_DISPATCH(lanes, KERNEL, rows, ...)                                               \
     switch (lanes) {                                                                              \
-        case 1: KERNEL(1)<<<nblk(rows, 128), 128, 0, st>>>(__VA_ARGS__); break;                   \
-        case 4: KERNEL(4)<<<nblk((rows) * 4, 128), 128, 0, st>>>(__VA_ARGS__); break;             \
-        default: KERNEL(8)<<<nblk((rows) * 8, 128), 128, 0, st>>>(__VA_ARGS__); break;            \
+        case 1: launch(KERNEL(1), nblk(rows, 128), 128, q, __VA_ARGS__); break;                   \
+        case 4: launch(KERNEL(4), nblk((rows) * 4, 128), 128, q, __VA_ARGS__); break;             \
+        default: launch(KERNEL(8), nblk((rows) * 8, 128), 128, q, __VA_ARGS__); break;            \
     }
 #define KNP_K_CHEB_SELL(L) k_cheb_sell<T, L, OUT>
 #define KNP_K_CHEB_CSR(L) k_cheb_csr<T, L, OUT>
@@ -871,7 +882,7 @@ void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, in
 // Chebyshev step k of a sweep of `steps` steps; OUT: into `out` instead of x_out
 template <class T, bool OUT = false>
 static void launch_cheb(const DevLevel<T>& L, const T* x_in, const T* b, const Coef4& c, T* d, T* x_out, int k,
-                        int steps, cudaStream_t st, const VcycleOut& out = VcycleOut{}) {
+                        int steps, const Queue& q, const VcycleOut& out = VcycleOut{}) {
     count_launch();
     const int read_d = k > 0, write_d = k + 1 < steps;
     if (L.sell) {
@@ -884,7 +895,7 @@ static void launch_cheb(const DevLevel<T>& L, const T* x_in, const T* b, const C
 }
 
 template <class T>
-static void launch_resid(const DevLevel<T>& L, const T* x, const T* b, T* r, cudaStream_t st) {
+static void launch_resid(const DevLevel<T>& L, const T* x, const T* b, T* r, const Queue& q) {
     count_launch();
     if (L.sell) {
         KNP_LANE_DISPATCH(L.lanes, KNP_K_RESID_SELL, L.n, L.n, L.sp.p, L.scol.p, L.sval.p, x, b, r);
@@ -894,59 +905,59 @@ static void launch_resid(const DevLevel<T>& L, const T* x, const T* b, T* r, cud
 }
 
 template <class T>
-static void cheb_step(DevLevel<T>& L, const Coef4& c, int k, int steps, Profiler* pr, bool fine, cudaStream_t st) {
-    ProfScope ps(fine ? pr : nullptr, KC_CHEB_FINE, st);
-    launch_cheb(L, L.x.p, L.b.p, c, L.d.p, L.x2.p, k, steps, st);
+static void cheb_step(DevLevel<T>& L, const Coef4& c, int k, int steps, Profiler* pr, bool fine, const Queue& q) {
+    ProfScope ps(fine ? pr : nullptr, KC_CHEB_FINE, q.st);
+    launch_cheb(L, L.x.p, L.b.p, c, L.d.p, L.x2.p, k, steps, q);
     std::swap(L.x.p, L.x2.p);
 }
 
 // the sweep's last step, whose result is the V-cycle's
 template <class T>
 static void cheb_step_out(DevLevel<T>& L, const Coef4& c, int k, int steps, const VcycleOut& out, Profiler* pr,
-                          cudaStream_t st) {
-    ProfScope ps(pr, KC_CHEB_FINE, st);
-    launch_cheb<T, true>(L, L.x.p, L.b.p, c, L.d.p, nullptr, k, steps, st, out);
+                          const Queue& q) {
+    ProfScope ps(pr, KC_CHEB_FINE, q.st);
+    launch_cheb<T, true>(L, L.x.p, L.b.p, c, L.d.p, nullptr, k, steps, q, out);
 }
 
 template <class T>
-static void residual(DevLevel<T>& L, Profiler* pr, bool fine, cudaStream_t st) {
-    ProfScope ps(fine ? pr : nullptr, KC_RESID_FINE, st);
-    launch_resid(L, L.x.p, L.b.p, L.r.p, st);
+static void residual(DevLevel<T>& L, Profiler* pr, bool fine, const Queue& q) {
+    ProfScope ps(fine ? pr : nullptr, KC_RESID_FINE, q.st);
+    launch_resid(L, L.x.p, L.b.p, L.r.p, q);
 }
 
 // rc = R r
 template <class T>
-static void restrict_to(const DevCsr4<T>& R, const T* r, T* rc, cudaStream_t st) {
+static void restrict_to(const DevCsr4<T>& R, const T* r, T* rc, const Queue& q) {
     count_launch();
     KNP_CSR_DISPATCH(R.lanes, KNP_K_CSR4, R.n, R.n, R.ptr.p, R.col.p, R.val.p, r, rc);
 }
 
 // x += P xc
 template <class T>
-static void prolong(const DevProlong<T>& P, const T* xc, T* x, cudaStream_t st) {
+static void prolong(const DevProlong<T>& P, const T* xc, T* x, const Queue& q) {
     count_launch();
     if (P.n >= LANE_THREADS)
-        k_prolong<T, 1><<<nblk(P.n, 128), 128, 0, st>>>(P.n, P.sp.p, P.col.p, P.val.p, P.perm.p, xc, x);
+        launch(k_prolong<T, 1>, nblk(P.n, 128), 128, q, P.n, P.sp.p, P.col.p, P.val.p, P.perm.p, xc, x);
     else
-        k_prolong<T, 4><<<nblk(4 * P.n, 128), 128, 0, st>>>(P.n, P.sp.p, P.col.p, P.val.p, P.perm.p, xc, x);
+        launch(k_prolong<T, 4>, nblk(4 * P.n, 128), 128, q, P.n, P.sp.p, P.col.p, P.val.p, P.perm.p, xc, x);
 }
 
 template <class T>
 static void smooth(DevLevel<T>& L, const std::vector<Coef4>& cs, int degree, bool zero_start, const double* v,
-                   const double* s, const DeflFuse& df, Profiler* pr, bool fine, cudaStream_t st) {
+                   const double* s, const DeflFuse& df, Profiler* pr, bool fine, const Queue& q) {
     int k0 = 0;
     if (zero_start) {
         count_launch();
-        k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, L.b.p, L.dinv.p, cs[0], L.x.p, L.d.p, df,
+        launch(k_cheb_first<T>, nblk(L.n, 256), 256, q, L.n, v, s, L.b.p, L.dinv.p, cs[0], L.x.p, L.d.p, df,
                                                          degree > 1);
         k0 = 1;
     }
-    for (int k = k0; k < degree; ++k) cheb_step(L, cs[k], k, degree, pr, fine, st);
+    for (int k = k0; k < degree; ++k) cheb_step(L, cs[k], k, degree, pr, fine, q);
 }
 
 template <class T>
 static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, const DeflFuse& df, Profiler* pr,
-                       cudaStream_t st, const VcycleOut& out) {
+                       const Queue& q, const VcycleOut& out) {
     DevLevel<T>& L = *D.L[l];
     const int last = (int)D.L.size() - 1;
     if (l == last) {
@@ -954,29 +965,29 @@ static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, co
             // single-level hierarchy: build b from the scaled input first
             Coef4 c0{};
             count_launch();
-            k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, L.b.p, L.dinv.p, c0, L.x.p, L.d.p, df, 0);
+            launch(k_cheb_first<T>, nblk(L.n, 256), 256, q, L.n, v, s, L.b.p, L.dinv.p, c0, L.x.p, L.d.p, df, 0);
         }
         count_launch();
-        k_coarse<T><<<nblk(4 * D.nc * 32, 256), 256, 0, st>>>(D.nc, D.cinv.p, L.b.p, L.x.p);
+        launch(k_coarse<T>, nblk(4 * D.nc * 32, 256), 256, q, D.nc, D.cinv.p, L.b.p, L.x.p);
         return;
     }
     DevLevel<T>& C = *D.L[l + 1];
-    smooth(L, D.coef[l], D.pre, true, v, s, df, pr, l == 0, st);
-    residual(L, pr, l == 0, st);
-    restrict_to(L.R, L.r.p, C.b.p, st);
-    vcycle_rec(D, l + 1, nullptr, nullptr, DeflFuse{}, pr, st, out);
-    prolong(L.P, C.x.p, L.x.p, st);
+    smooth(L, D.coef[l], D.pre, true, v, s, df, pr, l == 0, q);
+    residual(L, pr, l == 0, q);
+    restrict_to(L.R, L.r.p, C.b.p, q);
+    vcycle_rec(D, l + 1, nullptr, nullptr, DeflFuse{}, pr, q, out);
+    prolong(L.P, C.x.p, L.x.p, q);
     if (l > 0) {
-        smooth(L, D.coef[l], D.degree, false, nullptr, nullptr, DeflFuse{}, pr, false, st);
+        smooth(L, D.coef[l], D.degree, false, nullptr, nullptr, DeflFuse{}, pr, false, q);
     } else {
-        for (int k = 0; k + 1 < D.degree; ++k) cheb_step(L, D.coef[l][k], k, D.degree, pr, true, st);
-        cheb_step_out(L, D.coef[l][D.degree - 1], D.degree - 1, D.degree, out, pr, st);
+        for (int k = 0; k + 1 < D.degree; ++k) cheb_step(L, D.coef[l][k], k, D.degree, pr, true, q);
+        cheb_step_out(L, D.coef[l][D.degree - 1], D.degree - 1, D.degree, out, pr, q);
     }
 }
 
 template <class T>
 static void vcycle_typed(knp_problem* p, AmgDev<T>& D, const double* v, const double* s, double* z,
-                         const DeflFuse& df, double* w, cudaStream_t st) {
+                         const DeflFuse& df, double* w, const Queue& q) {
     VcycleOut out;
     out.z = z;
     out.w = w;
@@ -987,20 +998,20 @@ static void vcycle_typed(knp_problem* p, AmgDev<T>& D, const double* v, const do
     out.ext_group = df.ext_group;
     for (int r = 0; r < 2; ++r)
         for (int q = 0; q < 3; ++q) out.ztau[r][q] = p->sp.z[q] * p->sp.reg[r].tau[q];
-    vcycle_rec(D, 0, v, s, df, &p->prof, st, out);
+    vcycle_rec(D, 0, v, s, df, &p->prof, q, out);
     if (D.L.size() == 1) {
         // no smoothing on a single level: the coarse solution is the result
         count_launch();
-        k_out<T><<<nblk(D.L[0]->n, 256), 256, 0, st>>>(D.L[0]->n, D.L[0]->x.p, out);
+        launch(k_out<T>, nblk(D.L[0]->n, 256), 256, q, D.L[0]->n, D.L[0]->x.p, out);
     }
 }
 
 static void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse& df, double* w,
-                          cudaStream_t st) {
+                          const Queue& q) {
     if (p->amg->h32)
-        vcycle_typed(p, *static_cast<AmgDev<float>*>(p->amg->h32), v, s, z, df, w, st);
+        vcycle_typed(p, *static_cast<AmgDev<float>*>(p->amg->h32), v, s, z, df, w, q);
     else
-        vcycle_typed(p, *static_cast<AmgDev<double>*>(p->amg->h64), v, s, z, df, w, st);
+        vcycle_typed(p, *static_cast<AmgDev<double>*>(p->amg->h64), v, s, z, df, w, q);
 }
 
 template <class T>
@@ -1050,7 +1061,7 @@ void vcycle_apply(knp_problem* p, const double* v, const double* s, double* z, c
         int64_t before = g_launches.load();
         KNP_CUDA(cudaStreamBeginCapture(H.gstream, cudaStreamCaptureModeThreadLocal));
         try {
-            vcycle_launch(p, v, s, z, df, w, H.gstream);
+            vcycle_launch(p, v, s, z, df, w, Queue(H.gstream, true));
         } catch (...) {
             cudaGraph_t tmp;
             cudaStreamEndCapture(H.gstream, &tmp);
