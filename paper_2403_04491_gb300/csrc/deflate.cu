@@ -397,18 +397,15 @@ void deflation_prepare(knp_problem* p) {
     d.built_for = p->assembly_id;
 }
 
-void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose,
-                            double* w) {
+// y = E^{-1} Z^T (s .* v), and what forms s .* v - A Z y and adds Z y
+static DeflFuse coarse_solution(knp_problem* p, const double* v, const double* s, bool transpose, const Queue& q) {
     Deflation& d = *p->defl;
-    cudaStream_t st = p->stream;
-    const int64_t n = p->n_nodes;
     count_launch(2);
-    k_defl_gather<<<d.gchunks + d.gext, DT, 0, st>>>(d.gchunks, d.gbeg.p, d.cnodes.p, p->N_i, n, p->pin, v, s,
-                                                     d.gpart.p);
+    launch(k_defl_gather, d.gchunks + d.gext, DT, q, d.gchunks, d.gbeg.p, d.cnodes.p, p->N_i, p->n_nodes, p->pin, v, s,
+           d.gpart.p);
     // Z^T A^T Z = E^T: the same Schur complement, E_je and E_ej exchanged
-    k_defl_solve<<<1, DT, 0, st>>>(d.nc, d.gchunks, d.gext, d.gcell.p, d.gpart.p, d.iEjj.p,
-                                   transpose ? d.Eej.p : d.Eje.p, transpose ? d.Eje.p : d.Eej.p, d.Ee.p, d.y.p);
-    KNP_CUDA(cudaGetLastError());
+    launch(k_defl_solve, 1, DT, q, d.nc, d.gchunks, d.gext, d.gcell.p, d.gpart.p, d.iEjj.p,
+           transpose ? d.Eej.p : d.Eje.p, transpose ? d.Eje.p : d.Eej.p, d.Ee.p, d.y.p);
     DeflFuse df;
     df.rgrp = d.rgrp.p;
     df.act = d.act.p;
@@ -419,6 +416,21 @@ void deflated_precond_apply(knp_problem* p, const double* v, const double* s, do
     df.pin = p->pin;
     df.ext_group = d.nc;
     df.transpose = transpose;
+    return df;
+}
+
+void deflated_vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, bool transpose, double* w,
+                            const Queue& q) {
+    const DeflFuse df = coarse_solution(p, v, s, transpose, q);
+    vcycle_launch(p, v, s, z, df, w, q);
+}
+
+void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose,
+                            double* w) {
+    Deflation& d = *p->defl;
+    cudaStream_t st = p->stream;
+    const int64_t n = p->n_nodes;
+    const DeflFuse df = coarse_solution(p, v, s, transpose, st);
     if (p->amg->inner_cg_max_it == 0) {
         // one V-cycle: its first kernel forms s .* v - A Z y and its output kernel adds Z y
         vcycle_apply(p, v, s, z, &df, w);

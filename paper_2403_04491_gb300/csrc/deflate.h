@@ -10,5 +10,8 @@ void deflation_prepare(knp_problem* p);
 // transpose, A^T and E^T in their places (P_0 is symmetric)
 void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose = false,
                             double* w = nullptr);
+// the same with one V-cycle as P_0^{-1}, its kernels launched one by one into q (which may be capturing)
+void deflated_vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, bool transpose, double* w,
+                            const Queue& q);
 void deflation_free(Deflation* d);
 }  // namespace knp

@@ -47,7 +47,8 @@ constexpr int PART_LD = RED_BLOCKS + 8;   // partial[k * PART_LD + b]: block b's
 // device scalars: [0, MAXV) first-pass dots, [MAXV, 2 MAXV) second-pass dots, [2 MAXV, 2 MAXV +
 // MAXW) reference norms, 2 MAXV + MAXW the skip flag, then the six stopping-test norms, then the
 // second-pass flag of the Arnoldi step
-constexpr int CHK_OFF = 2 * MAXV + MAXW + 1;
+constexpr int SKIP_OFF = 2 * MAXV + MAXW;
+constexpr int CHK_OFF = SKIP_OFF + 1;
 constexpr int SECOND_OFF = CHK_OFF + 6;
 constexpr int DOTS_LEN = SECOND_OFF + 1;
 constexpr int CHECK_EVERY = 8;         // steps between exact evaluations of the stopping test, at most
@@ -363,20 +364,20 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, 
 // v_{j+1} = (w' - sum_k h2[k] V_k) / eta with eta^2 = <w',w'> - |h2|^2 (in place), h2 the sums of the
 // second pass's partial dots (pdots; only <w', w'> without a second pass). When the second
 // Gram-Schmidt pass found nothing to remove (|h2| <= ORTH_SKIP * |w'|), the subtraction is skipped,
-// V is not read, eta = |w'|, and flag[0] = 1 tells the host to keep h1 alone in the Hessenberg column.
-// Block 0 stores h2 to dots2.
+// V is not read, eta = |w'|, and the host keeps h1 alone in the Hessenberg column (skip flag).
+// The last block sends the step's scalars to the host (host: pinned memory, laid out as dots, then the
+// arrival flag) while the others work: a copy node took its place in the chain before the next V-cycle.
 constexpr double ORTH_SKIP = 1e-10;
 template <int NV>
 __global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const double* V, int64_t ldv,
-                                                            const double* pdots, int nblocks,
-                                                            const double* second,
-                                                            double* __restrict__ dots2, double* w,
-                                                            double* __restrict__ flag) {
+                                                            const double* pdots, int nblocks, const double* dots,
+                                                            double* w, double* host) {
     __shared__ double h2[NV + 1];
     __shared__ double inv_s;
     __shared__ int skip_s;
     chain_wait();
-    if (second[0] != 0.0) {
+    const bool second = dots[SECOND_OFF] != 0.0;
+    if (second) {
         sum_partials(pdots, nblocks, NV + 1, h2);
     } else {
         if ((int)threadIdx.x < NV) h2[threadIdx.x] = 0.0;
@@ -385,19 +386,26 @@ __global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const do
     if (threadIdx.x == 0) {
         const double s2 = h2[NV];
         double hh = 0.0;
-        if (second[0] != 0.0)
+        if (second)
             for (int k = 0; k < NV; ++k) hh += h2[k] * h2[k];
         const bool skip = hh <= ORTH_SKIP * ORTH_SKIP * s2;
         const double e2 = skip ? s2 : s2 - hh;
         inv_s = e2 > 0 ? rsqrt(e2) : 0.0;
         skip_s = skip;
-        if (blockIdx.x == 0) flag[0] = skip ? 1.0 : 0.0;
     }
-    if (blockIdx.x == 0 && threadIdx.x <= NV) dots2[threadIdx.x] = h2[threadIdx.x];
     __syncthreads();
     const double inv_eta = inv_s;
     const bool skip = skip_s != 0;
-    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
+    if (blockIdx.x == gridDim.x - 1) {
+        volatile double* out = host;
+        for (int k = threadIdx.x; k < DOTS_LEN; k += RED_THREADS)
+            out[k] = k >= MAXV && k <= MAXV + NV ? h2[k - MAXV] : k == SKIP_OFF ? (skip ? 1.0 : 0.0) : dots[k];
+        __threadfence_system();
+        __syncthreads();
+        if (threadIdx.x == 0) *reinterpret_cast<volatile uint64_t*>(host + DOTS_LEN) = 1;
+        return;
+    }
+    const int64_t n2 = n4 / 2, stride = (int64_t)(gridDim.x - 1) * RED_THREADS;
     const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
     if (skip) {
         for (int64_t i = i0; i < n2; i += 2 * stride) {
@@ -466,7 +474,7 @@ unsigned vec_grid(int64_t n4) {
 #define KNP_NV_CASE_k_combo_norms2(N) case N: k_combo_norms<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 #define KNP_NV_CASE_k_combo_norms3(N) case N: k_combo_norms<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 #define KNP_NV_CASE_k_orth_update_dot(N) case N: launch(k_orth_update_dot<N>, nb_red, RED_THREADS, q, KNP_ARGS); break;
-#define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec, RED_THREADS, q, KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec + 1, RED_THREADS, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_update_x(N) case N: k_update_x<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 // Launch KERNEL<nv> with the caller's grid (nb_red or nb_vec) for a runtime nv in [0, 31]
 #define KNP_LAUNCH_NV(nv, KERNEL)                                                                    \
@@ -495,21 +503,32 @@ struct GmresWork {
     int64_t n4 = 0;
     DArray<double> V, Z, partial, dots, y, cy, tmp;
     DArray<double> ones;            // unit weights (the paper's unscaled stopping test), on first use
-    double* hh = nullptr;           // pinned copy of dots, DOTS_LEN
-    cudaEvent_t ev_dots = nullptr;  // recorded after the copy of dots to hh
-    // the Arnoldi step of basis index j (SpMV, the three orthogonalisation passes with their
-    // reductions, the copy of the dots to hh) as a CUDA graph per (j, transposed, w formed by the V-cycle)
-    std::map<std::tuple<int, bool, bool>, cudaGraphExec_t> arnoldi;
+    double* hh = nullptr;           // pinned: the step's scalars as the device sends them (DOTS_LEN), arrival flag
+    uint64_t* flag() { return reinterpret_cast<uint64_t*>(hh + DOTS_LEN); }
+    // An iteration as a CUDA graph per (basis index j, transposed, w formed by the V-cycle, tail): the
+    // Arnoldi step (operator product, the three orthogonalisation passes) and, with a tail, the
+    // preconditioning of its result. The tail's kernels belong to the hierarchy that the graphs were
+    // captured with.
+    enum Tail { NO_TAIL, VCYCLE, DEFLATED_VCYCLE };
+    struct Graph {
+        cudaGraphExec_t exec = nullptr;
+        int launches = 0;
+    };
+    std::map<std::tuple<int, bool, bool, int>, Graph> graphs;
+    uint64_t graphs_amg = 0;        // AmgHierarchy::id of that hierarchy
     cudaStream_t cap = nullptr;     // capture stream (the problem's stream may be the legacy one)
+    void drop_graphs() {
+        for (auto& kv : graphs) cudaGraphExecDestroy(kv.second.exec);
+        graphs.clear();
+    }
     // partial sums: of an Arnoldi step's two passes, each read by the kernel after it, and the others'
     double* pass1() { return partial.p; }
     double* pass2() { return partial.p + MAXW * PART_LD; }
     double* other() { return partial.p + 2 * MAXW * PART_LD; }
     ~GmresWork() {
-        for (auto& kv : arnoldi) cudaGraphExecDestroy(kv.second);
+        drop_graphs();
         if (cap) cudaStreamDestroy(cap);
         if (hh) cudaFreeHost(hh);
-        if (ev_dots) cudaEventDestroy(ev_dots);
     }
 };
 
@@ -527,8 +546,7 @@ GmresWork* gmres_work(knp_problem* p, int restart) {
     g->y.alloc(MAXV);
     g->cy.alloc(2 * MAXV);
     g->tmp.alloc(g->n4);
-    KNP_CUDA(cudaMallocHost(&g->hh, DOTS_LEN * sizeof(double)));
-    KNP_CUDA(cudaEventCreateWithFlags(&g->ev_dots, cudaEventDisableTiming));
+    KNP_CUDA(cudaMallocHost(&g->hh, DOTS_LEN * sizeof(double) + sizeof(uint64_t)));
     p->gw = g;
     return g;
 }
@@ -565,24 +583,35 @@ static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose,
 #define KNP_ARGS n4, g.V.p, n4, g.pass1(), nb_red, g.dots.p, w, g.pass2()
     KNP_LAUNCH_NV(nv, k_orth_update_dot);
 #undef KNP_ARGS
-#define KNP_ARGS n4, g.V.p, n4, g.pass2(), nb_red, g.dots.p + SECOND_OFF, g.dots.p + MAXV, w, g.dots.p + 2 * MAXV + MAXW
+#define KNP_ARGS n4, g.V.p, n4, g.pass2(), nb_red, g.dots.p, w, g.hh
     KNP_LAUNCH_NV(nv, k_orth_final);
 #undef KNP_ARGS
     KNP_CUDA(cudaGetLastError());
 }
 
-// The Arnoldi step j followed by the copy of the dots to the pinned g.hh, replayed from a CUDA
-// graph captured at first use (about ten launches become one).
-static void arnoldi_graph_launch(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready) {
-    auto key = std::make_tuple(j, transpose, w_ready);
-    auto it = g.arnoldi.find(key);
-    if (it == g.arnoldi.end()) {
+// The iteration's graph (GmresWork::graphs), captured at first use; tail launches the kernels that
+// precondition v_{j+1} into the queue it is given. One launch replaces some 20, the kernels' prologues
+// overlap (launch.h), and the host has the step's scalars while the V-cycle runs. Graphs of the Arnoldi
+// step (ending in a copy node) and the V-cycle with the coarse correction's two kernels between them left
+// four gaps per iteration: three steps of the 2D problem with 4,612 unknowns took 3.73 ms, now 3.03; two
+// of 64^3 27.0 and 26.1.
+template <class TailFn>
+static void iteration_graph_launch(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready,
+                                   GmresWork::Tail kind, TailFn&& tail) {
+    if (g.graphs_amg != p->amg->id) {
+        g.drop_graphs();
+        g.graphs_amg = p->amg->id;
+    }
+    auto key = std::make_tuple(j, transpose, w_ready, (int)kind);
+    auto it = g.graphs.find(key);
+    if (it == g.graphs.end()) {
         if (!g.cap) KNP_CUDA(cudaStreamCreateWithFlags(&g.cap, cudaStreamNonBlocking));
         const int64_t before = g_launches.load();
+        const Queue q(g.cap, true);
         KNP_CUDA(cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal));
         try {
-            arnoldi_kernels(p, g, j, transpose, w_ready, Queue(g.cap, true));
-            KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, g.cap));
+            arnoldi_kernels(p, g, j, transpose, w_ready, q);
+            if (kind != GmresWork::NO_TAIL) tail(q);
         } catch (...) {
             cudaGraph_t tmp = nullptr;
             cudaStreamEndCapture(g.cap, &tmp);
@@ -591,15 +620,28 @@ static void arnoldi_graph_launch(knp_problem* p, GmresWork& g, int j, bool trans
         }
         cudaGraph_t graph = nullptr;
         KNP_CUDA(cudaStreamEndCapture(g.cap, &graph));
-        g_launches.fetch_sub(g_launches.load() - before);
-        cudaGraphExec_t ex = nullptr;
-        cudaError_t e = cudaGraphInstantiate(&ex, graph, 0);
+        GmresWork::Graph ng;
+        ng.launches = (int)(g_launches.load() - before);
+        g_launches.fetch_sub(ng.launches);
+        cudaError_t e = cudaGraphInstantiate(&ng.exec, graph, 0);
         cudaGraphDestroy(graph);
         KNP_CUDA(e);
-        it = g.arnoldi.emplace(key, ex).first;
+        it = g.graphs.emplace(key, ng).first;
     }
-    KNP_CUDA(cudaGraphLaunch(it->second, p->stream));
-    count_launch(4);
+    KNP_CUDA(cudaGraphLaunch(it->second.exec, p->stream));
+    count_launch(it->second.launches);
+}
+
+// Waits until the device has sent the scalars of the Arnoldi step launched last. A failed launch or
+// kernel ends the wait with its error.
+static void wait_scalars(GmresWork& g, cudaStream_t st) {
+    for (int64_t k = 1; !__atomic_load_n(g.flag(), __ATOMIC_ACQUIRE); ++k) {
+        if (k % 4096) continue;
+        const cudaError_t e = cudaStreamQuery(st);
+        if (e == cudaErrorNotReady) continue;
+        KNP_CUDA(e);
+        KNP_REQUIRE(__atomic_load_n(g.flag(), __ATOMIC_ACQUIRE), KNP_ERR_CUDA, "an Arnoldi step's scalars were not sent");
+    }
 }
 
 knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stats& stats, double* x,
@@ -640,9 +682,19 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
     const double* wts = paper_test ? g.ones.p : p->swt.p;
     const int nb_red = red_grid(n4);
     const unsigned nb_vec = vec_grid(n4);
-    // Arnoldi steps from CUDA graphs, unless a kernel class is being profiled (event pairs go
-    // around single launches) or graphs are switched off for the V-cycle as well
+    // iterations from CUDA graphs, unless a kernel class is being profiled (event pairs go
+    // around single launches) or graphs are switched off for the V-cycle as well; CG(P_0) waits for the
+    // host in every application and stays outside
     const bool use_graphs = p->amg->use_graphs && p->prof.active < 0;
+    const GmresWork::Tail tail_kind = p->amg->inner_cg_max_it > 0 ? GmresWork::NO_TAIL
+                                      : defl                      ? GmresWork::DEFLATED_VCYCLE
+                                                                  : GmresWork::VCYCLE;
+    auto tail = [&](double* v, double* z, const Queue& q) {
+        if (defl)
+            deflated_vcycle_launch(p, v, p->svec.p, z, transpose, wz, q);
+        else
+            vcycle_launch(p, v, p->svec.p, z, DeflFuse{}, wz, q);
+    };
     // reference norms of the stopping test, per group: ||S x|| of the iterate a cycle starts from
     // (the initial guess, then each restart's), taken together with the cycle's correction
     double tol[3] = {0, 0, 0};
@@ -761,20 +813,23 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
                 k_reduce<<<1, RED_THREADS, 0, st>>>(g.other(), nb_red, 2 * NG, g.dots.p + CHK_OFF);
             }
             const int nv = j + 1;
-            if (arnoldi && use_graphs) {
-                arnoldi_graph_launch(p, g, j, transpose, w_ready);   // includes the copy of the dots
-            } else {
-                if (arnoldi) arnoldi_kernels(p, g, j, transpose, w_ready, st);
-                KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, st));
-            }
-            KNP_CUDA(cudaEventRecord(g.ev_dots, st));
             if (arnoldi) {
-                // v_{j+1} is already normalised on the device: queue its V-cycle before the host
-                // waits for this step's dots, so the GPU works while the host does the Givens step
-                precond(g.V.p + (int64_t)(j + 1) * n4, p->svec.p, g.Z.p + (int64_t)(j + 1) * n4);
+                // v_{j+1} is normalised on the device: its preconditioning is queued before the host
+                // waits for this step's scalars, so the GPU works while the host does the Givens step
+                double *v1 = g.V.p + (int64_t)(j + 1) * n4, *z1 = g.Z.p + (int64_t)(j + 1) * n4;
+                __atomic_store_n(g.flag(), 0, __ATOMIC_RELEASE);
+                if (use_graphs)
+                    iteration_graph_launch(p, g, j, transpose, w_ready, tail_kind,
+                                           [&](const Queue& q) { tail(v1, z1, q); });
+                else
+                    arnoldi_kernels(p, g, j, transpose, w_ready, st);
+                if (!use_graphs || tail_kind == GmresWork::NO_TAIL) precond(v1, p->svec.p, z1);
                 vc_queued = true;
+                wait_scalars(g, st);
+            } else {
+                KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, st));
+                KNP_CUDA(cudaStreamSynchronize(st));
             }
-            KNP_CUDA(cudaEventSynchronize(g.ev_dots));
             KNP_CUDA(cudaGetLastError());
             if (check) {
                 bool ok = true;
@@ -816,7 +871,7 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
                 break;
             }
             // second pass skipped on the device (flag): the column is h1 and eta = |w'|
-            const bool skipped = g.hh[2 * MAXV + MAXW] != 0.0;
+            const bool skipped = g.hh[SKIP_OFF] != 0.0;
             if (monitor) {
                 // first Gram-Schmidt pass: |w'|^2 / |w|^2 = 1 - sum h1^2 / |w|^2
                 double h1 = 0.0;

@@ -14,6 +14,7 @@
 // before the coarse-grid correction (the first from x = 0 costs no operator product) and
 // `degree` after; one before and two after by default, which makes the V-cycle non-symmetric
 // (FGMRES takes any preconditioner; CG(P_0) is given as many steps before as after).
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <map>
@@ -601,6 +602,10 @@ struct AmgDev {
     std::vector<std::vector<Coef4>> coef;   // per level: coefficients of each Chebyshev step
 };
 
+static std::atomic<uint64_t> g_hierarchies{0};
+
+AmgHierarchy::AmgHierarchy() : id(++g_hierarchies) {}
+
 AmgHierarchy::~AmgHierarchy() {
     for (auto& kv : graphs)
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
@@ -1006,8 +1011,8 @@ static void vcycle_typed(knp_problem* p, AmgDev<T>& D, const double* v, const do
     }
 }
 
-static void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse& df, double* w,
-                          const Queue& q) {
+void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse& df, double* w,
+                   const Queue& q) {
     if (p->amg->h32)
         vcycle_typed(p, *static_cast<AmgDev<float>*>(p->amg->h32), v, s, z, df, w, q);
     else

@@ -4,6 +4,7 @@
 #include <vector>
 
 #include "amg.h"
+#include "launch.h"
 
 struct knp_problem;
 
@@ -30,6 +31,7 @@ struct VcycleGraph {
 };
 
 struct AmgHierarchy {
+    const uint64_t id;   // another for every hierarchy: captured graphs name it, not its address
     int precision = 0;
     int levels = 0;
     std::vector<int64_t> nodes, nnz;
@@ -48,6 +50,7 @@ struct AmgHierarchy {
     int setup_on_gpu = 0;
     int64_t long_rows_p = 0, long_rows_rap = 0;
     double setup_ms = 0.0;
+    AmgHierarchy();
     ~AmgHierarchy();
 };
 
@@ -61,6 +64,9 @@ void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, in
 // operator product's w of z.
 void vcycle_apply(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse* df = nullptr,
                   double* w = nullptr);
+// the same with its kernels launched one by one into q (which may be capturing)
+void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse& df, double* w,
+                   const Queue& q);
 // whether z = P_0^{-1} (s .* v) is one V-cycle whose last kernel can form w
 bool vcycle_forms_w(const knp_problem* p);
 // y = P_0 x with the finest level of the FP64 hierarchy; x, y [n][4] doubles on the device
