@@ -98,7 +98,9 @@ struct VN {
 // Row product of a sliced-ELL operator by L lanes: lane t adds entries t, t + L, ... The loads of
 // U entries (and the columns of the next batch) are issued together, so that a lane waits
 // for memory once or twice per batch instead of twice per entry; the order of the sums is that of
-// the entries.
+// the entries. One thread per row: four entries in FP32, which memory bounds (two steps of the 125-cell
+// 128^3 workload 228 -> 220 ms, most of it on the first coarse level's rows of 58 entries), one in FP64,
+// which the FP64 pipe bounds (two entries cost registers and 1% at 64^3).
 template <class T, int L>
 __device__ __forceinline__ void sell_row(int64_t r, int t, const int64_t* __restrict__ sp,
                                          const int32_t* __restrict__ col, const T* __restrict__ val,
@@ -106,7 +108,7 @@ __device__ __forceinline__ void sell_row(int64_t r, int t, const int64_t* __rest
     const int64_t s = r / SELL_C;
     const int64_t base = sp[s] + r % SELL_C;
     const int w = (int)((sp[s + 1] - sp[s]) / SELL_C);
-    constexpr int U = L == 1 ? 1 : 4;
+    constexpr int U = L == 1 && sizeof(T) == 8 ? 1 : 4;
     const int32_t* cp = col + base;
     const T* vp = val + 4 * base;
     acc[0] = acc[1] = acc[2] = acc[3] = T(0);
