@@ -43,21 +43,8 @@ namespace knp {
 
 namespace {
 
-constexpr int DT = 256;              // threads of the deflation kernels
 constexpr int GATHER_NODES = 1024;   // nodes per block of the gather
 constexpr int EXT_BLOCKS = 304;      // most partial sums over the extracellular nodes
-
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-    return s;   // valid in thread 0
-}
 
 // Coefficients of active row i, formed once per step: (A Z y)_f = C[f] y_own + C[4 + f] y_cross for its
 // four fields f, and (A^T Z y)_f likewise with CT. A Z y: the row's same-region phi columns other than
@@ -172,62 +159,18 @@ __global__ void __launch_bounds__(DT) k_defl_schur(int nc, int nchunks, int next
     }
 }
 
-// Partial sums of g = Z^T r with r = s .* v: blocks [0, nchunks) take one chunk of a cell's nodes each,
-// the others shares of the extracellular potentials (pin left out)
-__global__ void __launch_bounds__(DT) k_defl_gather(int nchunks, const int64_t* __restrict__ cbeg,
-                                                    const int32_t* __restrict__ cnodes, int64_t N_i, int64_t n,
-                                                    int32_t pin, const double* v,
-                                                    const double* __restrict__ s, double* __restrict__ part) {
+// partial sums of g = Z^T r with r = s .* v
+__global__ void __launch_bounds__(DT) k_defl_gather(GatherArgs a, const double* v, const double* __restrict__ s) {
     __shared__ double sh[DT / 32];
     chain_wait();
-    double acc = 0.0;
-    if ((int)blockIdx.x < nchunks) {
-        const int64_t end = cbeg[blockIdx.x + 1];
-        for (int64_t q = cbeg[blockIdx.x] + threadIdx.x; q < end; q += DT) {
-            const int64_t i = 4 * (int64_t)cnodes[q] + 3;
-            acc += s[i] * v[i];
-        }
-    } else {
-        const int64_t stride = (int64_t)(gridDim.x - nchunks) * DT;
-        for (int64_t r = N_i + (blockIdx.x - nchunks) * (int64_t)DT + threadIdx.x; r < n; r += stride)
-            if (r != pin) acc += s[4 * r + 3] * v[4 * r + 3];
-    }
-    const double t = block_sum(acc, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
+    const double t = block_sum(gather_share(a, blockIdx.x, [&](int64_t k) { return s[k] * v[k]; }), sh);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = t;
 }
 
-// y = E^{-1} g for the arrowhead E (one block): y_e = (g_e - sum_j E_ej g_j / E_jj) / S_e,
-// y_j = (g_j - E_je y_e) / E_jj; y[nc] = y_e. The division by E_jj and S_e is a product with their
-// reciprocals, formed once per step (an FP64 division is a chain of some 20 instructions).
-__global__ void __launch_bounds__(DT) k_defl_solve(int nc, int nchunks, int next, const int32_t* __restrict__ cchunk,
-                                                   const double* part, const double* iEjj,
-                                                   const double* Eje, const double* Eej, const double* Ee,
-                                                   double* y) {
-    __shared__ double sh[DT / 32];
-    __shared__ double ye_s;
+// y = E^{-1} g (one block)
+__global__ void __launch_bounds__(DT) k_defl_solve(CoarseSolve e, double* y) {
     chain_wait();
-    double a = 0.0;
-    for (int q = threadIdx.x; q < next; q += DT) a += part[nchunks + q];
-    // a thread per cell, or a warp where cells have many chunks: g_j (kept in y until the solve)
-    const bool wide = nchunks > 8 * nc;
-    const int lane = threadIdx.x & 31;
-    for (int j = wide ? threadIdx.x >> 5 : threadIdx.x; j < nc; j += wide ? DT / 32 : DT) {
-        double g = 0.0;
-        for (int q = cchunk[j] + (wide ? lane : 0); q < cchunk[j + 1]; q += wide ? 32 : 1) g += part[q];
-        if (wide)
-            for (int o = 16; o > 0; o >>= 1) g += __shfl_down_sync(0xffffffffu, g, o);
-        if (!wide || lane == 0) {
-            y[j] = g;
-            a -= Eej[j] * (g * iEjj[j]);
-        }
-    }
-    const double t = block_sum(a, sh);
-    if (threadIdx.x == 0) {
-        ye_s = t * Ee[1];
-        y[nc] = ye_s;
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < nc; j += DT) y[j] = (y[j] - Eje[j] * ye_s) * iEjj[j];
+    coarse_solve(e, y);
 }
 
 // t = s .* v - A Z y (or - A^T Z y), for CG(P_0)
@@ -236,7 +179,7 @@ __global__ void k_defl_rhs(int64_t n, const double* __restrict__ v, const double
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= n) return;
     double o[4];
-    defl_input(r, v, s, df, o);
+    defl_input(r, v, s, df, df.y, o);
     for (int q = 0; q < 4; ++q) t[4 * r + q] = o[q];
 }
 
@@ -397,15 +340,40 @@ void deflation_prepare(knp_problem* p) {
     d.built_for = p->assembly_id;
 }
 
-// y = E^{-1} Z^T (s .* v), and what forms s .* v - A Z y and adds Z y
-static DeflFuse coarse_solution(knp_problem* p, const double* v, const double* s, bool transpose, const Queue& q) {
+// The solve is a block's work of 2 us in a kernel of its own of 4. The V-cycle's first kernel does it in
+// every block instead where that is less: its grid at most two blocks per SM, the sums few.
+constexpr int SOLVE_ROWS = 152 * 512, SOLVE_SUMS = 512;
+
+// Most blocks of a gather that runs beside the normalisation: two per SM. With more (some 470 at 75^3) the
+// scalars that each of them forms and the second vector that the normalisation then needs cost what the
+// launch saves (0.4% of a pass).
+constexpr int GATHER_BESIDE = 2 * 152;
+
+bool deflation_gather_beside(const knp_problem* p) { return p->defl->gchunks + p->defl->gext <= GATHER_BESIDE; }
+
+GatherArgs deflation_gather(const knp_problem* p) {
+    const Deflation& d = *p->defl;
+    GatherArgs a;
+    a.nchunks = d.gchunks;
+    a.next = d.gext;
+    a.cbeg = d.gbeg.p;
+    a.cnodes = d.cnodes.p;
+    a.N_i = p->N_i;
+    a.n = p->n_nodes;
+    a.pin = p->pin;
+    a.part = d.gpart.p;
+    return a;
+}
+
+// y = E^{-1} Z^T (s .* v), and what forms s .* v - A Z y and adds Z y. gathered: Z^T (s .* v) is formed
+// already; in_vcycle: y may be left to the V-cycle's first kernel
+static DeflFuse coarse_solution(knp_problem* p, const double* v, const double* s, bool transpose, const Queue& q,
+                                bool gathered, bool in_vcycle) {
     Deflation& d = *p->defl;
-    count_launch(2);
-    launch(k_defl_gather, d.gchunks + d.gext, DT, q, d.gchunks, d.gbeg.p, d.cnodes.p, p->N_i, p->n_nodes, p->pin, v, s,
-           d.gpart.p);
-    // Z^T A^T Z = E^T: the same Schur complement, E_je and E_ej exchanged
-    launch(k_defl_solve, 1, DT, q, d.nc, d.gchunks, d.gext, d.gcell.p, d.gpart.p, d.iEjj.p,
-           transpose ? d.Eej.p : d.Eje.p, transpose ? d.Eje.p : d.Eej.p, d.Ee.p, d.y.p);
+    if (!gathered) {
+        count_launch();
+        launch(k_defl_gather, d.gchunks + d.gext, DT, q, deflation_gather(p), v, s);
+    }
     DeflFuse df;
     df.rgrp = d.rgrp.p;
     df.act = d.act.p;
@@ -416,13 +384,27 @@ static DeflFuse coarse_solution(knp_problem* p, const double* v, const double* s
     df.pin = p->pin;
     df.ext_group = d.nc;
     df.transpose = transpose;
+    df.e.nc = d.nc;
+    df.e.nchunks = d.gchunks;
+    df.e.next = d.gext;
+    df.e.cchunk = d.gcell.p;
+    df.e.part = d.gpart.p;
+    df.e.iEjj = d.iEjj.p;
+    // Z^T A^T Z = E^T: the same Schur complement, E_je and E_ej exchanged
+    df.e.Eje = transpose ? d.Eej.p : d.Eje.p;
+    df.e.Eej = transpose ? d.Eje.p : d.Eej.p;
+    df.e.Ee = d.Ee.p;
+    df.solve = in_vcycle && d.nc < SOLVE_CELLS && p->n_nodes <= SOLVE_ROWS && d.gchunks + d.gext <= SOLVE_SUMS;
+    if (!df.solve) {
+        count_launch();
+        launch(k_defl_solve, 1, DT, q, df.e, d.y.p);
+    }
     return df;
 }
 
 void deflated_vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, bool transpose, double* w,
                             const Queue& q) {
-    const DeflFuse df = coarse_solution(p, v, s, transpose, q);
-    vcycle_launch(p, v, s, z, df, w, q);
+    vcycle_launch(p, v, s, z, coarse_solution(p, v, s, transpose, q, deflation_gather_beside(p), true), w, q);
 }
 
 void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose,
@@ -430,8 +412,9 @@ void deflated_precond_apply(knp_problem* p, const double* v, const double* s, do
     Deflation& d = *p->defl;
     cudaStream_t st = p->stream;
     const int64_t n = p->n_nodes;
-    const DeflFuse df = coarse_solution(p, v, s, transpose, st);
-    if (p->amg->inner_cg_max_it == 0) {
+    const bool vcycle = p->amg->inner_cg_max_it == 0;
+    const DeflFuse df = coarse_solution(p, v, s, transpose, st, false, vcycle);
+    if (vcycle) {
         // one V-cycle: its first kernel forms s .* v - A Z y and its output kernel adds Z y
         vcycle_apply(p, v, s, z, &df, w);
         return;

@@ -1,5 +1,6 @@
 // Coarse correction of the potentials' near-null modes around P_0^{-1} (deflate.cu).
 #pragma once
+#include "deflate_input.h"
 #include "problem.h"
 
 namespace knp {
@@ -10,7 +11,11 @@ void deflation_prepare(knp_problem* p);
 // transpose, A^T and E^T in their places (P_0 is symmetric)
 void deflated_precond_apply(knp_problem* p, const double* v, const double* s, double* z, bool transpose = false,
                             double* w = nullptr);
-// the same with one V-cycle as P_0^{-1}, its kernels launched one by one into q (which may be capturing)
+// what forms Z^T r's partial sums (after deflation_prepare), and whether the kernel that normalises r does
+GatherArgs deflation_gather(const knp_problem* p);
+bool deflation_gather_beside(const knp_problem* p);
+// the same with one V-cycle as P_0^{-1}, its kernels launched one by one into q (which may be capturing);
+// with deflation_gather_beside the partial sums of Z^T r are there already
 void deflated_vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, bool transpose, double* w,
                             const Queue& q);
 void deflation_free(Deflation* d);

@@ -361,17 +361,22 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, 
     }
 }
 
-// v_{j+1} = (w' - sum_k h2[k] V_k) / eta with eta^2 = <w',w'> - |h2|^2 (in place), h2 the sums of the
-// second pass's partial dots (pdots; only <w', w'> without a second pass). When the second
-// Gram-Schmidt pass found nothing to remove (|h2| <= ORTH_SKIP * |w'|), the subtraction is skipped,
-// V is not read, eta = |w'|, and the host keeps h1 alone in the Hessenberg column (skip flag).
-// The last block sends the step's scalars to the host (host: pinned memory, laid out as dots, then the
-// arrival flag) while the others work: a copy node took its place in the chain before the next V-cycle.
+// v = (w' - sum_k h2[k] V_k) / eta with eta^2 = <w',w'> - |h2|^2, h2 the sums of the second pass's
+// partial dots (pdots; only <w', w'> without a second pass). When the second Gram-Schmidt pass found
+// nothing to remove (|h2| <= ORTH_SKIP * |w'|), the subtraction is skipped, V is not read, eta = |w'|, and
+// the host keeps h1 alone in the Hessenberg column (skip flag).
+// Further blocks work beside those: ga.nchunks + ga.next of them form the coarse correction's partial sums
+// of Z^T (s .* v) from w', and the last one sends the step's scalars to the host (host: pinned memory, laid
+// out as dots, then the arrival flag). A gather kernel and a copy node of their own took their time in the
+// chain before the next V-cycle. With the coarse solve in the V-cycle's first kernel as well, three steps of
+// 4,612 unknowns in 2D take 2.87 ms instead of 3.00, of 117,504 in 3D 9.79 instead of 10.00.
 constexpr double ORTH_SKIP = 1e-10;
 template <int NV>
 __global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const double* V, int64_t ldv,
                                                             const double* pdots, int nblocks, const double* dots,
-                                                            double* w, double* host) {
+                                                            const double* w, double* v, double* host,
+                                                            GatherArgs ga, const double* __restrict__ s) {
+    static_assert(RED_THREADS == DT, "the gather's blocks");
     __shared__ double h2[NV + 1];
     __shared__ double inv_s;
     __shared__ int skip_s;
@@ -405,14 +410,28 @@ __global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const do
         if (threadIdx.x == 0) *reinterpret_cast<volatile uint64_t*>(host + DOTS_LEN) = 1;
         return;
     }
-    const int64_t n2 = n4 / 2, stride = (int64_t)(gridDim.x - 1) * RED_THREADS;
+    const int ng = ga.nchunks + ga.next, nvec = (int)gridDim.x - 1 - ng;
+    if ((int)blockIdx.x >= nvec) {
+        __shared__ double sh[DT / 32];
+        const double t = block_sum(gather_share(ga, (int)blockIdx.x - nvec,
+                                                [&](int64_t i) {
+                                                    double wi = w[i];
+                                                    if (!skip)
+                                                        for (int k = 0; k < NV; ++k) wi -= h2[k] * V[k * ldv + i];
+                                                    return s[i] * (wi * inv_eta);
+                                                }),
+                                   sh);
+        if (threadIdx.x == 0) ga.part[(int)blockIdx.x - nvec] = t;
+        return;
+    }
+    const int64_t n2 = n4 / 2, stride = (int64_t)nvec * RED_THREADS;
     const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
     if (skip) {
         for (int64_t i = i0; i < n2; i += 2 * stride) {
             const bool two = i + stride < n2;
             double2 a = ld2(w, i), b = two ? ld2(w, i + stride) : a;
-            st2(w, i, make_double2(a.x * inv_eta, a.y * inv_eta));
-            if (two) st2(w, i + stride, make_double2(b.x * inv_eta, b.y * inv_eta));
+            st2(v, i, make_double2(a.x * inv_eta, a.y * inv_eta));
+            if (two) st2(v, i + stride, make_double2(b.x * inv_eta, b.y * inv_eta));
         }
     } else {
         for (int64_t i = i0; i < n2; i += stride) {
@@ -423,7 +442,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_orth_final(int64_t n4, const do
                 wi.x -= h2[k] * vk.x;
                 wi.y -= h2[k] * vk.y;
             }
-            st2(w, i, make_double2(wi.x * inv_eta, wi.y * inv_eta));
+            st2(v, i, make_double2(wi.x * inv_eta, wi.y * inv_eta));
         }
     }
 }
@@ -474,7 +493,7 @@ unsigned vec_grid(int64_t n4) {
 #define KNP_NV_CASE_k_combo_norms2(N) case N: k_combo_norms<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 #define KNP_NV_CASE_k_combo_norms3(N) case N: k_combo_norms<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 #define KNP_NV_CASE_k_orth_update_dot(N) case N: launch(k_orth_update_dot<N>, nb_red, RED_THREADS, q, KNP_ARGS); break;
-#define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec + 1, RED_THREADS, q, KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec + ga.nchunks + ga.next + 1, RED_THREADS, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_update_x(N) case N: k_update_x<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 // Launch KERNEL<nv> with the caller's grid (nb_red or nb_vec) for a runtime nv in [0, 31]
 #define KNP_LAUNCH_NV(nv, KERNEL)                                                                    \
@@ -565,15 +584,19 @@ static double norm2_dev(GmresWork& g, const double* v, cudaStream_t st) {
     return s;
 }
 
-// w = S^-1 A z_j into V_{j+1}, orthogonalised against V_0..V_j (CGS2, second pass skipped on the
+// w = S^-1 A z_j, into V_{j+1} orthogonalised against V_0..V_j (CGS2, second pass skipped on the
 // device when it has nothing to remove) and normalised; the dots of both passes land in g.dots
-static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready, const Queue& q) {
+static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose, bool w_ready, const GatherArgs& ga,
+                            const Queue& q) {
     const int64_t n4 = g.n4;
     const int nv = j + 1;
     const int nb_red = red_grid(n4);
     const unsigned nb_vec = vec_grid(n4);
     double* zj = g.Z.p + (int64_t)j * n4;
-    double* w = g.V.p + (int64_t)(j + 1) * n4;
+    // not in place where the gather reads w beside the normalisation; else in place, which keeps one vector
+    // less in the L2 cache (0.5% of a pass at 75^3)
+    double* v1 = g.V.p + nv * n4;
+    double* w = ga.part ? g.tmp.p : v1;
     op_apply(p, zj, w, p->sinv.p, nullptr, transpose, q, w_ready);
     ProfScope ps(&p->prof, KC_ORTHO, q.st);
     count_launch(3);
@@ -583,7 +606,7 @@ static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose,
 #define KNP_ARGS n4, g.V.p, n4, g.pass1(), nb_red, g.dots.p, w, g.pass2()
     KNP_LAUNCH_NV(nv, k_orth_update_dot);
 #undef KNP_ARGS
-#define KNP_ARGS n4, g.V.p, n4, g.pass2(), nb_red, g.dots.p, w, g.hh
+#define KNP_ARGS n4, g.V.p, n4, g.pass2(), nb_red, g.dots.p, w, v1, g.hh, ga, p->svec.p
     KNP_LAUNCH_NV(nv, k_orth_final);
 #undef KNP_ARGS
     KNP_CUDA(cudaGetLastError());
@@ -610,7 +633,10 @@ static void iteration_graph_launch(knp_problem* p, GmresWork& g, int j, bool tra
         const Queue q(g.cap, true);
         KNP_CUDA(cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal));
         try {
-            arnoldi_kernels(p, g, j, transpose, w_ready, q);
+            arnoldi_kernels(p, g, j, transpose, w_ready,
+                            kind == GmresWork::DEFLATED_VCYCLE && deflation_gather_beside(p) ? deflation_gather(p)
+                                                                                             : GatherArgs{},
+                            q);
             if (kind != GmresWork::NO_TAIL) tail(q);
         } catch (...) {
             cudaGraph_t tmp = nullptr;
@@ -822,7 +848,7 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
                     iteration_graph_launch(p, g, j, transpose, w_ready, tail_kind,
                                            [&](const Queue& q) { tail(v1, z1, q); });
                 else
-                    arnoldi_kernels(p, g, j, transpose, w_ready, st);
+                    arnoldi_kernels(p, g, j, transpose, w_ready, GatherArgs{}, st);
                 if (!use_graphs || tail_kind == GmresWork::NO_TAIL) precond(v1, p->svec.p, z1);
                 vc_queued = true;
                 wait_scalars(g, st);

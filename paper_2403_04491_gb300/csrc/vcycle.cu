@@ -192,19 +192,27 @@ __device__ __forceinline__ T csr_row_field(bool active, int64_t r, int t, const 
 }
 
 // first Chebyshev step from x = 0: d = c2 D^-1 b, x = d (d stored if a second step reads it). On the finest level b = s .* v (double
-// input), or s .* v - A Z y inside the coarse correction (df.y set).
-template <class T>
-__global__ void k_cheb_first(int64_t n, const double* v, const double* __restrict__ s, T* b,
+// input), or s .* v - A Z y inside the coarse correction (df.y set), whose y it forms itself with SOLVE (block
+// 0 keeps it for the last kernel). Blocks of DT threads.
+template <class T, bool SOLVE>
+__global__ void __launch_bounds__(DT) k_cheb_first(int64_t n, const double* v, const double* __restrict__ s, T* b,
                              const T* __restrict__ dinv, Coef4 c, T* __restrict__ x, T* __restrict__ d, DeflFuse df,
                              int write_d) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    V4<T> di = V4<T>::load(dinv + 4 * i), dd;
+    V4<T> di = V4<T>::load(dinv + 4 * (i < n ? i : 0)), dd;
     chain_wait();
+    const double* y = df.y;
+    if constexpr (SOLVE) {
+        __shared__ double ys[SOLVE_CELLS];
+        coarse_solve(df.e, ys);
+        if (blockIdx.x == 0 && (int)threadIdx.x <= df.e.nc) df.y[threadIdx.x] = ys[threadIdx.x];
+        y = ys;
+    }
+    if (i >= n) return;
     V4<T> bb;
     if (v && df.y) {
         double t[4];
-        defl_input(i, v, s, df, t);
+        defl_input(i, v, s, df, y, t);
         for (int f = 0; f < 4; ++f) bb.v[f] = (T)t[f];
         bb.store(b + 4 * i);
     } else if (v) {
@@ -955,8 +963,8 @@ static void smooth(DevLevel<T>& L, const std::vector<Coef4>& cs, int degree, boo
     int k0 = 0;
     if (zero_start) {
         count_launch();
-        launch(k_cheb_first<T>, nblk(L.n, 256), 256, q, L.n, v, s, L.b.p, L.dinv.p, cs[0], L.x.p, L.d.p, df,
-                                                         degree > 1);
+        launch(df.solve ? k_cheb_first<T, true> : k_cheb_first<T, false>, nblk(L.n, DT), DT, q, L.n, v, s, L.b.p,
+               L.dinv.p, cs[0], L.x.p, L.d.p, df, degree > 1);
         k0 = 1;
     }
     for (int k = k0; k < degree; ++k) cheb_step(L, cs[k], k, degree, pr, fine, q);
@@ -972,7 +980,8 @@ static void vcycle_rec(AmgDev<T>& D, int l, const double* v, const double* s, co
             // single-level hierarchy: build b from the scaled input first
             Coef4 c0{};
             count_launch();
-            launch(k_cheb_first<T>, nblk(L.n, 256), 256, q, L.n, v, s, L.b.p, L.dinv.p, c0, L.x.p, L.d.p, df, 0);
+            launch(df.solve ? k_cheb_first<T, true> : k_cheb_first<T, false>, nblk(L.n, DT), DT, q, L.n, v, s, L.b.p,
+                   L.dinv.p, c0, L.x.p, L.d.p, df, 0);
         }
         count_launch();
         launch(k_coarse<T>, nblk(4 * D.nc * 32, 256), 256, q, D.nc, D.cinv.p, L.b.p, L.x.p);
@@ -1177,7 +1186,7 @@ static void na_vcycle_rec(AmgDev<T>& D, std::vector<NaWork<T>>& W, int l, const 
         if (v) {
             Coef4 c0{};
             count_launch();
-            k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, w.b, L.dinv.p, c0, w.x, w.d, DeflFuse{}, 0);
+            k_cheb_first<T, false><<<nblk(L.n, DT), DT, 0, st>>>(L.n, v, s, w.b, L.dinv.p, c0, w.x, w.d, DeflFuse{}, 0);
         }
         count_launch();
         k_coarse<T><<<nblk(4 * D.nc * 32, 256), 256, 0, st>>>(D.nc, D.cinv.p, w.b, w.x);
@@ -1187,7 +1196,7 @@ static void na_vcycle_rec(AmgDev<T>& D, std::vector<NaWork<T>>& W, int l, const 
     NaWork<T>& wc = W[l + 1];
     const std::vector<Coef4>& cs = D.coef[l];
     count_launch();
-    k_cheb_first<T><<<nblk(L.n, 256), 256, 0, st>>>(L.n, v, s, w.b, L.dinv.p, cs[0], w.x, w.d, DeflFuse{},
+    k_cheb_first<T, false><<<nblk(L.n, DT), DT, 0, st>>>(L.n, v, s, w.b, L.dinv.p, cs[0], w.x, w.d, DeflFuse{},
                                                      D.pre > 1);
     for (int k = 1; k < D.pre; ++k) na_cheb_step(L, w, cs[k], k, D.pre, st);
     launch_resid(L, w.x, w.b, w.r, st);

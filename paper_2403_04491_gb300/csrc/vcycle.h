@@ -10,6 +10,17 @@ struct knp_problem;
 
 namespace knp {
 
+constexpr int SOLVE_CELLS = 64;   // the V-cycle's first kernel forms y for fewer cells than this
+
+// Terms of y = E^{-1} g for the arrowhead E of the coarse correction: g = Z^T r as the partial sums part
+// (those of cell j at [cchunk[j], cchunk[j + 1]), next of the extracellular space from nchunks on), and
+// 1 / E_jj, E_je, E_ej, {E_ee, 1 / Schur complement} (E_je and E_ej exchanged for the transposed operator).
+struct CoarseSolve {
+    int32_t nc = 0, nchunks = 0, next = 0;
+    const int32_t* cchunk = nullptr;
+    const double *part = nullptr, *iEjj = nullptr, *Eje = nullptr, *Eej = nullptr, *Ee = nullptr;
+};
+
 // The coarse correction's two passes around the V-cycle, done inside it (device pointers and
 // scalars; y == nullptr: none). The first kernel of the finest level forms the corrected input
 // r - A Z y from r = s .* v (deflate_input.h), and the output kernel adds Z y to the potentials.
@@ -18,10 +29,12 @@ struct DeflFuse {
     const int32_t* act = nullptr;    // node -> active row, -1 where A Z y is zero
     const double* C = nullptr;       // [active rows][8] coefficients of A Z y (or A^T Z y)
     const int32_t* xgrp = nullptr;   // active row -> group on the membrane's other side
-    const double* y = nullptr;       // [groups + 1] the coarse solution, extracellular group last
+    double* y = nullptr;             // [groups + 1] the coarse solution, extracellular group last
     int64_t N_i = 0;
     int32_t pin = -1, ext_group = 0;
     int32_t transpose = 0;           // A^T Z y in place of A Z y
+    int32_t solve = 0;               // the first kernel also forms y, from the terms below
+    CoarseSolve e;
 };
 
 // One captured V-cycle: a CUDA graph instantiated for a given (input, scale, output) triple.
