@@ -40,7 +40,7 @@ namespace knp {
 namespace {
 
 constexpr int RED_BLOCKS = 152;   // the most blocks a reduction kernel launches: one per SM (152 SMs)
-constexpr int RED_THREADS = 256;
+constexpr int RED_THREADS = 256;  // the most threads of a block
 constexpr int MAXV = 32;          // restart + 2
 constexpr int MAXW = 3 * MAXV;    // the most sums a reduction kernel forms
 constexpr int PART_LD = RED_BLOCKS + 8;   // partial[k * PART_LD + b]: block b's share of sum k
@@ -112,16 +112,16 @@ __device__ __forceinline__ void block_reduce_store(const double (&acc)[NT], doub
     __syncthreads();
     if (threadIdx.x < NT) {
         double t = 0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) t += sh[w][threadIdx.x];
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) t += sh[w][threadIdx.x];
         partial[threadIdx.x * PART_LD + blockIdx.x] = t;
     }
 }
 
-// out[k] = sum over blocks of partial[k * PART_LD + b], k < nt, by one block of RED_THREADS: each
+// out[k] = sum over blocks of partial[k * PART_LD + b], k < nt, by one block: each
 // warp takes four sums at a time. Every block of a kernel gets the same bits. out is shared memory.
 __device__ __forceinline__ void sum_partials(const double* partial, int nblocks, int nt, double* out) {
     const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
-    for (int k0 = 4 * wid; k0 < nt; k0 += 4 * (RED_THREADS / 32)) {
+    for (int k0 = 4 * wid; k0 < nt; k0 += 4 * ((int)blockDim.x / 32)) {
         double v[4] = {0.0, 0.0, 0.0, 0.0};
         for (int b = lane; b < nblocks; b += 32) {
 #pragma unroll
@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_mdot(int64_t n4, const doubl
     double acc[NV + 1];
 #pragma unroll
     for (int k = 0; k <= NV; ++k) acc[k] = 0.0;
-    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
-    for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n2; i += E * stride) {
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += E * stride) {
         double2 wi[E], vk[E][NV > 0 ? NV : 1];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_combo_norms(int64_t n4, cons
     }
     __syncthreads();
     GroupSums<NG> gu, gv;
-    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
-    const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (int64_t i = i0; i < n2; i += E * stride) {
         double2 zk[E][NV > 0 ? NV : 1], w[E];
 #pragma unroll
@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(RED_THREADS, 1) k_orth_update_dot(int64_t n4, 
     double hk[NV > 0 ? NV : 1];
 #pragma unroll
     for (int k = 0; k < NV; ++k) hk[k] = h[k];
-    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * RED_THREADS;
-    const int64_t i0 = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x;
+    const int64_t n2 = n4 / 2, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (second) {
         double acc[NV + 1];
 #pragma unroll
@@ -480,6 +480,21 @@ __global__ void __launch_bounds__(RED_THREADS) k_update_x(int64_t n4, const doub
 int red_grid(int64_t n4) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (n4 + 4 * RED_THREADS - 1) / (4 * RED_THREADS)));
 }
+// The same for the Arnoldi step's dots and the stopping test (least: 64 threads) and the update (128, for its
+// prologue's sums), in smaller blocks where 256 threads would not have a pair each on every SM: a block
+// reduction costs a warp as much as a pair of elements, so a small vector goes to more SMs and fewer warps.
+// Three steps of 4,612 unknowns in 2D 2.88 -> 2.67 ms, of the Kir problem on 97x75 7.16 -> 6.84. Smaller
+// blocks at up to two pairs per thread made 117,504 unknowns in 3D 0.3% slower, everywhere 128^3 12%.
+struct RedShape {
+    int blocks, threads;
+};
+RedShape red_shape(int64_t n4, int least) {
+    const int64_t n2 = n4 / 2;
+    int t = RED_THREADS;
+    while (t > least && n2 < (int64_t)RED_BLOCKS * t) t /= 2;
+    if (t == RED_THREADS) return {red_grid(n4), t};
+    return {(int)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (n2 + t - 1) / t)), t};
+}
 // Blocks of a kernel that leaves no partial sums: two pairs per thread, up to four blocks per SM
 unsigned vec_grid(int64_t n4) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(608, (n4 + 4 * RED_THREADS - 1) / (4 * RED_THREADS)));
@@ -489,10 +504,10 @@ unsigned vec_grid(int64_t n4) {
     X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16) X(17) X(18) X(19) \
     X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30) X(31)
 
-#define KNP_NV_CASE_k_mdot(N) case N: launch(k_mdot<N>, nb_red, RED_THREADS, q, KNP_ARGS); break;
-#define KNP_NV_CASE_k_combo_norms2(N) case N: k_combo_norms<N, 2><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_combo_norms3(N) case N: k_combo_norms<N, 3><<<nb_red, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-#define KNP_NV_CASE_k_orth_update_dot(N) case N: launch(k_orth_update_dot<N>, nb_red, RED_THREADS, q, KNP_ARGS); break;
+#define KNP_NV_CASE_k_mdot(N) case N: launch(k_mdot<N>, rs.blocks, rs.threads, q, KNP_ARGS); break;
+#define KNP_NV_CASE_k_combo_norms2(N) case N: k_combo_norms<N, 2><<<rs.blocks, rs.threads, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_combo_norms3(N) case N: k_combo_norms<N, 3><<<rs.blocks, rs.threads, 0, st>>>(KNP_ARGS); break;
+#define KNP_NV_CASE_k_orth_update_dot(N) case N: launch(k_orth_update_dot<N>, us.blocks, us.threads, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec + ga.nchunks + ga.next + 1, RED_THREADS, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_update_x(N) case N: k_update_x<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
 // Launch KERNEL<nv> with the caller's grid (nb_red or nb_vec) for a runtime nv in [0, 31]
@@ -590,7 +605,7 @@ static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose,
                             const Queue& q) {
     const int64_t n4 = g.n4;
     const int nv = j + 1;
-    const int nb_red = red_grid(n4);
+    const RedShape rs = red_shape(n4, 64), us = red_shape(n4, 128);
     const unsigned nb_vec = vec_grid(n4);
     double* zj = g.Z.p + (int64_t)j * n4;
     // not in place where the gather reads w beside the normalisation; else in place, which keeps one vector
@@ -603,10 +618,10 @@ static void arnoldi_kernels(knp_problem* p, GmresWork& g, int j, bool transpose,
 #define KNP_ARGS n4, g.V.p, n4, w, g.pass1()
     KNP_LAUNCH_NV(nv, k_mdot);
 #undef KNP_ARGS
-#define KNP_ARGS n4, g.V.p, n4, g.pass1(), nb_red, g.dots.p, w, g.pass2()
+#define KNP_ARGS n4, g.V.p, n4, g.pass1(), rs.blocks, g.dots.p, w, g.pass2()
     KNP_LAUNCH_NV(nv, k_orth_update_dot);
 #undef KNP_ARGS
-#define KNP_ARGS n4, g.V.p, n4, g.pass2(), nb_red, g.dots.p, w, v1, g.hh, ga, p->svec.p
+#define KNP_ARGS n4, g.V.p, n4, g.pass2(), us.blocks, g.dots.p, w, v1, g.hh, ga, p->svec.p
     KNP_LAUNCH_NV(nv, k_orth_final);
 #undef KNP_ARGS
     KNP_CUDA(cudaGetLastError());
@@ -707,6 +722,7 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
     }
     const double* wts = paper_test ? g.ones.p : p->swt.p;
     const int nb_red = red_grid(n4);
+    const RedShape rs = red_shape(n4, 64);
     const unsigned nb_vec = vec_grid(n4);
     // iterations from CUDA graphs, unless a kernel class is being profiled (event pairs go
     // around single launches) or graphs are switched off for the V-cycle as well; CG(P_0) waits for the
@@ -836,7 +852,7 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
                 else
                     KNP_LAUNCH_NV(j + 1, k_combo_norms2);
 #undef KNP_ARGS
-                k_reduce<<<1, RED_THREADS, 0, st>>>(g.other(), nb_red, 2 * NG, g.dots.p + CHK_OFF);
+                k_reduce<<<1, RED_THREADS, 0, st>>>(g.other(), rs.blocks, 2 * NG, g.dots.p + CHK_OFF);
             }
             const int nv = j + 1;
             if (arnoldi) {
