@@ -483,7 +483,7 @@ int red_grid(int64_t n4) {
 // The same for the Arnoldi step's dots and the stopping test (least: 64 threads) and the update (128, for its
 // prologue's sums), in smaller blocks where 256 threads would not have a pair each on every SM: a block
 // reduction costs a warp as much as a pair of elements, so a small vector goes to more SMs and fewer warps.
-// Three steps of 4,612 unknowns in 2D 2.88 -> 2.67 ms, of the Kir problem on 97x75 7.16 -> 6.84. Smaller
+// Three steps of 4,612 unknowns in 2D 2.88 -> 2.62 ms, of the Kir problem on 97x75 7.16 -> 6.77. Smaller
 // blocks at up to two pairs per thread made 117,504 unknowns in 3D 0.3% slower, everywhere 128^3 12%.
 struct RedShape {
     int blocks, threads;

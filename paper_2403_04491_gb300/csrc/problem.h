@@ -206,7 +206,7 @@ inline const cudaStream_t kProblemStream = reinterpret_cast<cudaStream_t>(~uintp
 // (on `q`, or on the problem's stream when q is the default argument); w_ready: p->op_w holds x's w
 void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale, const double* b,
               bool transpose = false, Queue q = kProblemStream, bool w_ready = false);
-// whether the forward product reads p->op_w (one thread per row)
+// whether the forward product reads p->op_w (up to four lanes per row)
 bool op_reads_w(const knp_problem* p);
 // the static per-ion values of the forward product (after the pattern and m, a are on the device)
 void op_prepare(knp_problem* p, cudaStream_t st);

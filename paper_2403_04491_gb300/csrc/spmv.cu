@@ -84,10 +84,11 @@ __device__ __forceinline__ void op_store(int64_t k, const double* out, double* _
     }
 }
 
-// y = rowscale .* (b - A x)  (b, rowscale optional), L lanes per row (lanes.h). One thread per row
-// needs w = k_op_w(x); with more lanes the kernel is bound by its chain of loads, so it forms w from
-// the x it gathers anyway (three FMAs per entry) and saves the node pass. The loads of OP_BATCH
-// entries are issued together.
+// y = rowscale .* (b - A x)  (b, rowscale optional), L lanes per row (lanes.h). One and four lanes per
+// row read w = k_op_w(x); with eight the kernel is bound by its chain of loads, so it forms w from
+// the x it gathers anyway (three FMAs per entry). Read by four lanes, 117,504 unknowns in 3D 9.89 -> 9.70 ms
+// for three steps, P2 20^3 26.3 -> 24.7 for two; by eight, the Kir problem on 97x75 6.77 -> 6.90. The loads
+// of OP_BATCH entries are issued together.
 template <int L>
 constexpr int OP_BATCH = L == 1 ? 1 : 3;
 template <int L>
@@ -121,7 +122,7 @@ __global__ void __launch_bounds__(128) k_op_apply(OpArgs A, const double* x, dou
                 const double2* xp = reinterpret_cast<const double2*>(x + 4 * (int64_t)c[u]);
                 x01[u] = xp[0];
                 x23[u] = xp[1];
-                if (L == 1) wv[u] = A.w[c[u]];
+                if (L <= 4) wv[u] = A.w[c[u]];
 #pragma unroll
                 for (int i = 0; i < KI; ++i) {
                     gv[u][i] = g0[i * ne + q];
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(128) k_op_apply(OpArgs A, const double* x, dou
         for (int u = 0; u < U; ++u) {
             if (k + u * L < w) {
                 const double phi = (c[u] == A.pin) ? 0.0 : x23[u].y;
-                if (L > 1)
+                if (L > 4)
                     wv[u] = A.z[0] * A.tau[reg][0] * x01[u].x + A.z[1] * A.tau[reg][1] * x01[u].y +
                             A.z[2] * A.tau[reg][2] * x23[u].x;
                 ag[0] += gv[u][0] * x01[u].x;
@@ -261,7 +262,7 @@ static int op_lanes(const knp_problem* p) {
     return row_lanes(p->n_nodes, (double)p->sell.n_entries / (double)std::max<int64_t>(p->n_nodes, 1));
 }
 
-bool op_reads_w(const knp_problem* p) { return op_lanes(p) == 1; }
+bool op_reads_w(const knp_problem* p) { return op_lanes(p) <= 4; }
 
 void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale, const double* b, bool transpose,
               Queue q, bool w_ready) {
@@ -299,11 +300,14 @@ void op_apply(knp_problem* p, const double* x, double* y, const double* rowscale
             launch(k_op_apply_t<4>, blocks, 128, q, A, x, y, rowscale, b);
         else
             launch(k_op_apply_t<8>, blocks, 128, q, A, x, y, rowscale, b);
-    } else if (lanes == 1) {
-        if (!w_ready) {
-            count_launch();
-            launch(k_op_w, (A.n + 255) / 256, 256, q, A, x, p->op_w.p);
-        }
+        KNP_CUDA(cudaGetLastError());
+        return;
+    }
+    if (op_reads_w(p) && !w_ready) {
+        count_launch();
+        launch(k_op_w, (A.n + 255) / 256, 256, q, A, x, p->op_w.p);
+    }
+    if (lanes == 1) {
         launch(k_op_apply<1>, blocks, 128, q, A, x, y, rowscale, b);
     } else if (lanes == 4) {
         launch(k_op_apply<4>, blocks, 128, q, A, x, y, rowscale, b);

@@ -240,9 +240,10 @@ struct VcycleOut {
     double ztau[2][3] = {};
 };
 
-// fields f0 .. f0 + F of node i
+// fields f0 .. f0 + F of node i; lanes: with one field per lane, those of the warp that call this (a node's
+// four neighbour each other), among which they form w
 template <class T, int F>
-__device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0, const VN<T, F>& x) {
+__device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0, const VN<T, F>& x, unsigned lanes = 0) {
     VN<double, F> z;
     for (int f = 0; f < F; ++f) z.v[f] = (double)x.v[f];
     const bool in = i < o.N_i;
@@ -253,6 +254,14 @@ __device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0,
             const double z0 = in ? o.ztau[0][0] : o.ztau[1][0], z1 = in ? o.ztau[0][1] : o.ztau[1][1],
                          z2 = in ? o.ztau[0][2] : o.ztau[1][2];
             o.w[i] = z0 * z.v[0] + z1 * z.v[1] + z2 * z.v[2];
+        }
+    } else if constexpr (F == 1) {
+        if (o.w && lanes) {
+            const double zt = f0 == 0 ? o.ztau[in ? 0 : 1][0] : f0 == 1 ? o.ztau[in ? 0 : 1][1] : o.ztau[in ? 0 : 1][2];
+            double w = f0 < 3 ? zt * z.v[0] : 0.0;
+            w += __shfl_xor_sync(lanes, w, 1);
+            w += __shfl_xor_sync(lanes, w, 2);
+            if (f0 == 0) o.w[i] = w;
         }
     }
 }
@@ -274,6 +283,7 @@ __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __r
     T acc[4], ax[F];
     sell_row<T, L>(i < n ? i : n - 1, t, sp, col, val, x_in, acc);
     lane_reduce4<T, L>(acc, t, ax);
+    const unsigned lanes = OUT && L > 1 ? __ballot_sync(0xffffffffu, i < n && t < 4) : 0u;
     if (i >= n || t >= 4) return;
     const int f0 = lane_field<L>(t);
     const int64_t k = 4 * i + f0;
@@ -288,7 +298,7 @@ __global__ void __launch_bounds__(128) k_cheb_sell(int64_t n, const int64_t* __r
     for (int f = 0; f < F; ++f) xx.v[f] += dd.v[f];
     if (write_d) dd.store(d + k);
     if constexpr (OUT)
-        store_out<T, F>(out, i, f0, xx);
+        store_out<T, F>(out, i, f0, xx, lanes);
     else
         xx.store(x_out + k);
 }
@@ -1032,7 +1042,7 @@ void vcycle_launch(knp_problem* p, const double* v, const double* s, double* z, 
 
 template <class T>
 static bool forms_w(const AmgDev<T>& D) {
-    return D.L.size() > 1 && D.L[0]->sell && D.L[0]->lanes == 1;
+    return D.L.size() > 1 && D.L[0]->sell;
 }
 
 bool vcycle_forms_w(const knp_problem* p) {
