@@ -5,17 +5,20 @@
 
 namespace knp {
 
-// Lanes per row of a row-product kernel over a sliced-ELL pattern: 1, 4 or 8. One thread per row
-// suffices once the rows alone give every SM enough loads in flight; a smaller matrix leaves the
-// SMs waiting on each row's chain of dependent loads, which 4 or 8 lanes shorten by that factor.
-// Lanes are added while the grid stays below LANE_THREADS (the threads that give 152 SMs 16 warps
-// each) and every lane keeps at least one entry of a mean row. Chebyshev step of the FP64 hierarchy,
-// one lane against several: 1,153 rows of 7 entries 9.3 -> 5.2 us (8 lanes), 29,376 rows of 14
-// entries 17.5 -> 10.8 us (4 lanes).
+// Lanes per row of a row-product kernel over a sliced-ELL pattern: 1, 4 or 8. More lanes shorten a row's
+// chain of dependent loads, which is what a small matrix waits for; but each row's sums over the lanes, its
+// epilogue and lanes without an entry are FP64 instructions that one thread per row does not issue. One
+// thread per row is better once the rows are many for their length, 18 per SM and entry (2D, 7 entries: from
+// 19,200 rows, 3D, 14.5: from 39,700), and always from LANE_THREADS on, where the rows alone fill the SMs.
+// Against four lanes up to LANE_THREADS in every case: 2D 68,500 rows 26.6 -> 21.8 ms (its reverse sweep
+// 63.0 -> 53.3), 3D 72,400 rows, reverse sweep, 15.5 -> 14.0; at 15 per SM and entry P2 on 80x80 (27,000 rows of
+// 11.5) was 5% slower. Eight lanes up to 4,864 rows: with four there too, the Kir problem on 97x75 is 3%
+// slower (its first coarse level) and 4,612 unknowns 0.5%; with eight up to 9,728 rows it took 6.77 ms (7,700
+// rows of 7 entries on the finest level), now 6.21.
 constexpr int64_t LANE_THREADS = 152 * 512;
 inline int row_lanes(int64_t rows, double mean_len) {
-    if (rows >= LANE_THREADS) return 1;
-    return (8 * rows <= LANE_THREADS && mean_len > 4.0) ? 8 : 4;
+    if (rows >= LANE_THREADS || rows >= 152 * 18 * mean_len) return 1;
+    return (16 * rows <= LANE_THREADS && mean_len > 4.0) ? 8 : 4;
 }
 
 // Sums of the four fields over the L lanes of a row (consecutive lanes of one warp, L a power of

@@ -23,9 +23,9 @@ def _gpu():
     __graft_entry__.build()
 
 
-# nodes: 284 (8 lanes, a partly empty warp), 9,601 and 9,997 (either side of the 8-lane limit of 9,728),
-# 74,524 and 78,397 (either side of the 4-lane limit of 77,824)
-@pytest.mark.parametrize("nx", [15, 96, 98, 271, 278])
+# nodes: 284 (8 lanes, a partly empty warp), 4,760 and 4,897 (either side of the 8-lane limit of 4,864),
+# 18,768 and 20,448 (either side of the 4-lane limit of 152 * 18 rows per entry of a mean row of 7)
+@pytest.mark.parametrize("nx", [15, 67, 68, 135, 141])
 def test_operator_products_at_the_lane_limits(nx):
     from paper_2403_04491_gb300 import problem_from_config
     cfg = make_config(1).with_nx(nx)
