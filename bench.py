@@ -287,14 +287,13 @@ def dominant_kernel_work(prob, precision):
 
 def spmv_work(prob):
     """Algorithmic bytes and FLOPs of one forward operator product y = S^-1 A x as the library
-    times it (the node pass w = sum_k z_k tau^k x^k, then k_op_apply). Bytes: per stored
+    times it (k_op_apply; w = sum_k z_k tau^k x^k comes from the V-cycle's last kernel). Bytes: per stored
     same-region entry a column index and seven FP64 values (g^1..g^3 = m + tau^k a, a, e^1..e^3),
-    per cross-region entry an index and three values, per node x (4 values) and w read by the
-    node pass and w written, then x gathered, w gathered, the row scale and y (FP64). FLOPs: 7 FMAs
-    per same-region entry, 3 per cross entry, 3 FMAs per node in the node pass and 20 per row."""
+    per cross-region entry an index and three values, per node x and w gathered, the row scale and y
+    (FP64). FLOPs: 7 FMAs per same-region entry, 3 per cross entry and 20 per row."""
     info = prob.info()
     n, nnz, nx = info["n_nodes"], info["nnz_region"], info["nnz_cross"]
-    return nnz * (4 + 56) + nx * (4 + 24) + n * (40 + 104), 14.0 * nnz + 6.0 * nx + 26.0 * n
+    return nnz * (4 + 56) + nx * (4 + 24) + n * 104, 14.0 * nnz + 6.0 * nx + 20.0 * n
 
 
 def measure(prob, torch, steps, rtol, kernel_class=None, deflate=True):
