@@ -32,6 +32,8 @@
 // application and 546 us per step for the one cell of the 64^3 workload.
 #include <algorithm>
 #include <map>
+#include <memory>
+#include <utility>
 #include <vector>
 
 #include "deflate.h"
@@ -237,8 +239,7 @@ static void make_chunks(const std::vector<int64_t>& gptr, int64_t most, std::vec
 
 static Deflation& deflation_setup(knp_problem* p) {
     if (p->defl) return *p->defl;
-    auto* d = new Deflation();
-    p->defl = d;
+    auto d = std::make_unique<Deflation>();   // the problem's once it is whole: an allocation may fail
     cudaStream_t st = p->stream;
     const knp_mesh& m = *p->mesh;
     const std::vector<int32_t>& cell = p->degree == 2 ? p2_nodes(m).node_cell_i : m.node_cell_i;
@@ -320,7 +321,8 @@ static Deflation& deflation_setup(knp_problem* p) {
     KNP_CUDA(cudaGetLastError());
     // the host tables above go out of scope here
     KNP_CUDA(cudaStreamSynchronize(st));
-    return *d;
+    p->defl = d.release();
+    return *p->defl;
 }
 
 void deflation_prepare(knp_problem* p) {
@@ -419,11 +421,13 @@ void deflated_precond_apply(knp_problem* p, const double* v, const double* s, do
         vcycle_apply(p, v, s, z, &df, w);
         return;
     }
-    if (!d.t.p) {
+    if (!d.ones.p) {
+        DArray<double> ones;   // kept last, with t there: an allocation may fail
         d.t.alloc(4 * n);
-        d.ones.alloc(4 * n);
-        k_fill_ones<<<nbk(4 * n, 256), 256, 0, st>>>(4 * n, d.ones.p);
+        ones.alloc(4 * n);
+        k_fill_ones<<<nbk(4 * n, 256), 256, 0, st>>>(4 * n, ones.p);
         count_launch();
+        d.ones = std::move(ones);
     }
     count_launch();
     k_defl_rhs<<<nbk(n, 128), 128, 0, st>>>(n, v, s, df, d.t.p);
