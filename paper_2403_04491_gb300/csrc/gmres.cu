@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <chrono>
 #include <map>
+#include <memory>
 #include <tuple>
 #include <cmath>
 #include <cstdio>
@@ -570,7 +571,7 @@ GmresWork* gmres_work(knp_problem* p, int restart) {
     if (p->gw && p->gw->restart == restart) return p->gw;
     delete p->gw;
     p->gw = nullptr;
-    auto* g = new GmresWork();
+    auto g = std::make_unique<GmresWork>();   // the problem's once it is whole: an allocation may fail
     g->restart = restart;
     g->n4 = 4 * p->n_nodes;
     g->V.alloc((restart + 1) * g->n4);
@@ -581,8 +582,8 @@ GmresWork* gmres_work(knp_problem* p, int restart) {
     g->cy.alloc(2 * MAXV);
     g->tmp.alloc(g->n4);
     KNP_CUDA(cudaMallocHost(&g->hh, DOTS_LEN * sizeof(double) + sizeof(uint64_t)));
-    p->gw = g;
-    return g;
+    p->gw = g.release();
+    return p->gw;
 }
 
 void gmres_free(GmresWork* g) { delete g; }

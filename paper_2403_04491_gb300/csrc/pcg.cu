@@ -12,6 +12,7 @@
 // level is solved exactly), as CG needs. The dot products come to the host once per inner
 // iteration.
 #include <cmath>
+#include <memory>
 #include <vector>
 
 #include "problem.h"
@@ -121,8 +122,7 @@ namespace {
 
 PcgWork& pcg_work(knp_problem* p) {
     if (!p->pcg) {
-        auto* w = new PcgWork();
-        p->pcg = w;
+        auto w = std::make_unique<PcgWork>();   // the problem's once it is whole: an allocation may fail
         const int64_t n4 = 4 * p->n_nodes;
         for (DArray<double>* v : {&w->r, &w->y, &w->pv, &w->q, &w->ones}) v->alloc(n4);
         w->partial.alloc(DOT_BLOCKS * 2 * NG);
@@ -130,6 +130,7 @@ PcgWork& pcg_work(knp_problem* p) {
         KNP_CUDA(cudaMallocHost(&w->h_dots, 2 * NG * sizeof(double)));
         count_launch();
         k_fill_one<<<nblk(n4, 256), 256, 0, p->stream>>>(n4, w->ones.p);
+        p->pcg = w.release();
     }
     return *p->pcg;
 }

@@ -39,6 +39,9 @@ def coarse_correction():
         solve(prob, False)
     return before, lambda prob: solve(prob, True), [b"k_defl", b"k_fill_ones", b"k_pcg_init"]
 
+def solver():
+    return lambda prob: hierarchy(prob, 1), lambda prob: solve(prob, False), [b"k_pcg"]
+
 before, call, watch = globals()[sys.argv[2]]()
 for w in watch:
     lib.fake_watch(w)
@@ -93,7 +96,7 @@ def run(fake_library, scenario):
     return json.loads(r.stdout.splitlines()[-1])
 
 
-@pytest.mark.parametrize("scenario", ["coarse_correction"])
+@pytest.mark.parametrize("scenario", ["coarse_correction", "solver"])
 def test_a_failed_allocation_leaves_nothing_half_built(fake_library, scenario):
     runs = run(fake_library, scenario)
     assert len(runs) > 2 and runs[-1]["code"] == 0          # every allocation of the call has failed once
