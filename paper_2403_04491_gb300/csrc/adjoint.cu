@@ -17,6 +17,7 @@
 //             Psi_k = sum_r +-_r (Lambda_r^k / z_k + Lambda_r^phi) on Gamma.
 #include <algorithm>
 #include <cmath>
+#include <memory>
 
 #include "gmres.h"
 #include "problem.h"
@@ -316,8 +317,7 @@ void adjoint_begin(knp_problem* P) {
         KNP_REQUIRE(v != KNP_MODEL_KIR, KNP_ERR_INVALID_ARG,
                     "the adjoint step covers leak and HH facets; this problem has Kir-Na/K facets");
     if (!P->adj) {
-        auto* W = new AdjointWork();
-        P->adj = W;
+        auto W = std::make_unique<AdjointWork>();   // the problem's once it is whole: an allocation may fail
         std::vector<double> elA;
         std::vector<int32_t> neptr, nelist;
         build_problem_stiffness(P, elA, neptr, nelist);
@@ -329,6 +329,7 @@ void adjoint_begin(knp_problem* P) {
         for (DArray<double>* v : {&W->rho, &W->lam, &W->rhs, &W->unew, &W->tmp}) v->alloc(4 * P->n_nodes);
         W->gam.alloc(std::max<int64_t>(1, 3 * P->n_mv));
         W->grad.alloc(std::max<int64_t>(1, 3 * P->nf));
+        P->adj = W.release();
     }
     AdjointWork* W = P->adj;
     for (DArray<double>* v : {&W->rho, &W->lam, &W->gam, &W->grad}) v->zero(P->stream);

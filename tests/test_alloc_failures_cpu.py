@@ -42,6 +42,15 @@ def coarse_correction():
 def solver():
     return lambda prob: hierarchy(prob, 1), lambda prob: solve(prob, False), [b"k_pcg"]
 
+def adjoint():
+    # the sweep's start, and a look at its (zero) result, whose kernel reads its arrays
+    def call(prob):
+        prob.adjoint_begin()
+        out = (C.c_double * prob.n_dof)()
+        p = C.cast(out, C.c_void_p)
+        knp._check(lib.knp_adjoint_get(prob.handle, knp.KNP_DEVICE, p, None, None, p))
+    return lambda prob: None, call, [b"k_eq42_out"]
+
 before, call, watch = globals()[sys.argv[2]]()
 for w in watch:
     lib.fake_watch(w)
@@ -96,7 +105,7 @@ def run(fake_library, scenario):
     return json.loads(r.stdout.splitlines()[-1])
 
 
-@pytest.mark.parametrize("scenario", ["coarse_correction", "solver"])
+@pytest.mark.parametrize("scenario", ["coarse_correction", "solver", "adjoint"])
 def test_a_failed_allocation_leaves_nothing_half_built(fake_library, scenario):
     runs = run(fake_library, scenario)
     assert len(runs) > 2 and runs[-1]["code"] == 0          # every allocation of the call has failed once
