@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <type_traits>
 
@@ -835,50 +836,54 @@ static void take_hierarchy(AmgDev<T>& D, GpuHierarchy& H, int degree, int pre, c
 
 void amg_upload(knp_problem* p, const HostHierarchy& H, int precision, int degree, int pre) {
     delete p->amg;
-    p->amg = new AmgHierarchy();
-    p->amg->precision = precision;
-    p->amg->levels = (int)H.levels.size();
-    p->amg->use_graphs = std::getenv("KNP_NO_GRAPHS") == nullptr;
+    p->amg = nullptr;
+    auto amg = std::make_unique<AmgHierarchy>();   // the problem's once it is whole: an allocation may fail
+    amg->precision = precision;
+    amg->levels = (int)H.levels.size();
+    amg->use_graphs = std::getenv("KNP_NO_GRAPHS") == nullptr;
     for (const HostLevel& L : H.levels) {
-        p->amg->nodes.push_back(L.A.n_rows);
-        p->amg->nnz.push_back(L.A.nnz());
+        amg->nodes.push_back(L.A.n_rows);
+        amg->nnz.push_back(L.A.nnz());
     }
     if (precision == KNP_PREC_FP32) {
         auto* D = new AmgDev<float>();
-        p->amg->h32 = D;
+        amg->h32 = D;
         upload_hierarchy(*D, H, degree, pre, p->stream);
     } else {
         auto* D = new AmgDev<double>();
-        p->amg->h64 = D;
+        amg->h64 = D;
         upload_hierarchy(*D, H, degree, pre, p->stream);
     }
     KNP_CUDA(cudaStreamSynchronize(p->stream));
+    p->amg = amg.release();
 }
 
 void amg_take_gpu(knp_problem* p, GpuHierarchy& H, int precision, int degree, int pre) {
     delete p->amg;
-    p->amg = new AmgHierarchy();
-    p->amg->precision = precision;
-    p->amg->levels = (int)H.levels.size();
-    p->amg->use_graphs = std::getenv("KNP_NO_GRAPHS") == nullptr;
-    p->amg->setup_on_gpu = 1;
-    p->amg->long_rows_p = H.long_rows_p;
-    p->amg->long_rows_rap = H.long_rows_rap;
+    p->amg = nullptr;
+    auto amg = std::make_unique<AmgHierarchy>();   // the problem's once it is whole: an allocation may fail
+    amg->precision = precision;
+    amg->levels = (int)H.levels.size();
+    amg->use_graphs = std::getenv("KNP_NO_GRAPHS") == nullptr;
+    amg->setup_on_gpu = 1;
+    amg->long_rows_p = H.long_rows_p;
+    amg->long_rows_rap = H.long_rows_rap;
     for (auto& L : H.levels) {
-        p->amg->nodes.push_back(L->A.n_rows);
-        p->amg->nnz.push_back(L->A.nnz);
+        amg->nodes.push_back(L->A.n_rows);
+        amg->nnz.push_back(L->A.nnz);
     }
     if (precision == KNP_PREC_FP32) {
         auto* D = new AmgDev<float>();
-        p->amg->h32 = D;
+        amg->h32 = D;
         take_hierarchy(*D, H, degree, pre, p->stream);
     } else {
         auto* D = new AmgDev<double>();
-        p->amg->h64 = D;
+        amg->h64 = D;
         take_hierarchy(*D, H, degree, pre, p->stream);
     }
     H.levels.clear();
     KNP_CUDA(cudaStreamSynchronize(p->stream));
+    p->amg = amg.release();
 }
 
 // CSR kernels with the matrix's lanes per row

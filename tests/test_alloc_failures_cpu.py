@@ -51,7 +51,19 @@ def adjoint():
         knp._check(lib.knp_adjoint_get(prob.handle, knp.KNP_DEVICE, p, None, None, p))
     return lambda prob: None, call, [b"k_eq42_out"]
 
-before, call, watch = globals()[sys.argv[2]]()
+def new_hierarchy():
+    # in place of one that is there; without a hierarchy a solve is refused
+    def after(prob):
+        prob.assemble_step()
+        try:
+            prob.solve()
+        except knp.KnpError as e:
+            assert e.code == 7, e
+        else:
+            assert False, "a solve without a hierarchy"
+    return lambda prob: hierarchy(prob, 1), lambda prob: hierarchy(prob, 1), [], after
+
+before, call, watch, *after = globals()[sys.argv[2]]()
 for w in watch:
     lib.fake_watch(w)
 out = []
@@ -66,6 +78,9 @@ for k in range(1, 200):
         code = e.code
     left = lib.fake_pending()
     lib.fake_fail_at(0)
+    if code:
+        for f in after:
+            f(prob)
     retry = 0
     try:
         call(prob)
@@ -105,7 +120,7 @@ def run(fake_library, scenario):
     return json.loads(r.stdout.splitlines()[-1])
 
 
-@pytest.mark.parametrize("scenario", ["coarse_correction", "solver", "adjoint"])
+@pytest.mark.parametrize("scenario", ["coarse_correction", "solver", "adjoint", "new_hierarchy"])
 def test_a_failed_allocation_leaves_nothing_half_built(fake_library, scenario):
     runs = run(fake_library, scenario)
     assert len(runs) > 2 and runs[-1]["code"] == 0          # every allocation of the call has failed once
