@@ -11,6 +11,7 @@
 // membrane kernels (the P2 section at the end of the anonymous namespace).
 #include <mutex>
 
+#include "element_mean.h"
 #include "p2_pairs.cuh"
 #include "problem.h"
 
@@ -108,16 +109,6 @@ __global__ void __launch_bounds__(4 * MN_NODES) k_membrane_nodes(StepParams sp, 
     const double n = w[0][lane], m = w[1][lane], hg = w[2][lane];
     mf[10 * nmv + a] = m * m * m * hg * (phiM - E[sp.ion_na]);
     mf[11 * nmv + a] = (n * n) * (n * n) * (phiM - E[sp.ion_k]);
-}
-
-// s / (D + 1), D + 1 = 3 or 4, without an FP64 division (some 20 instructions of the slow pipe each: 833 us
-// of k_elem_means at 128^3, now 365 us): a quarter is exact; a third is the product with the rounded third and one
-// FMA of its remainder, Markstein's correction, which gives the correctly rounded quotient.
-template <int D>
-__device__ __forceinline__ double mean_of_sum(double s) {
-    if constexpr (D == 3) return 0.25 * s;
-    const double third = 1.0 / 3.0, q = s * third;
-    return fma(fma(-3.0, q, s), third, q);
 }
 
 template <int D>
