@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(4 * MN_NODES) k_membrane_nodes(StepParams sp, 
     const bool in = a < nmv;
     const int64_t gi = in ? mv_g[a] : 0, ge = in ? mv_g[nmv + a] : 0;
     const double phiM = in ? u[4 * gi + 3] - u[4 * ge + 3] : 0.0;
+    double driveNa = 0.0, driveK = 0.0;   // phi_M - E of Na and K (last warp)
     if (part < 3) {
         // Hodgkin-Huxley gate (n, m, h): N_ode Rush-Larsen substeps with phi_M frozen
         if (in) {
@@ -74,11 +75,8 @@ __global__ void __launch_bounds__(4 * MN_NODES) k_membrane_nodes(StepParams sp, 
             gates_new[part * nmv + a] = x;
             w[part][lane] = x;
         }
-        __syncthreads();
-        return;
-    }
-    double ci[KI], ce[KI], E[KI], si = 0, se = 0, wi[KI], we[KI];
-    if (in) {
+    } else if (in) {
+        double ci[KI], ce[KI], E[KI], si = 0, se = 0, wi[KI], we[KI];
         for (int k = 0; k < KI; ++k) {
             ci[k] = u[4 * gi + k];
             ce[k] = u[4 * ge + k];
@@ -97,18 +95,19 @@ __global__ void __launch_bounds__(4 * MN_NODES) k_membrane_nodes(StepParams sp, 
             mf[(7 + k) * nmv + a] = phiM - E[k];
         }
         // Kir-Na/K (Section 2.4.2): the K drive rectified by f_Kir, and the pump flux density
-        const double dK = phiM - E[sp.ion_k];
+        driveNa = phiM - E[sp.ion_na];
+        driveK = phiM - E[sp.ion_k];
         const double fA = 1.0 + exp(0.433), fB = 1.0 + exp(-(0.1186 + sp.EK0) / 0.0441);
-        const double fC = 1.0 + exp((dK + 0.0185) / 0.0425), fD = 1.0 + exp(-(0.1186 + phiM) / 0.0441);
-        mf[12 * nmv + a] = dK * (fA * fB / (fC * fD) * sqrt(ce[sp.ion_k] / sp.cKe0));
+        const double fC = 1.0 + exp((driveK + 0.0185) / 0.0425), fD = 1.0 + exp(-(0.1186 + phiM) / 0.0441);
+        mf[12 * nmv + a] = driveK * (fA * fB / (fC * fD) * sqrt(ce[sp.ion_k] / sp.cKe0));
         const double na15 = ci[sp.ion_na] * sqrt(ci[sp.ion_na]), pna15 = sp.P_na * sqrt(sp.P_na);
         mf[13 * nmv + a] = sp.rho_pump * (na15 / (na15 + pna15)) * (ce[sp.ion_k] / (ce[sp.ion_k] + sp.P_k));
     }
     __syncthreads();
-    if (!in) return;
+    if (part < 3 || !in) return;
     const double n = w[0][lane], m = w[1][lane], hg = w[2][lane];
-    mf[10 * nmv + a] = m * m * m * hg * (phiM - E[sp.ion_na]);
-    mf[11 * nmv + a] = (n * n) * (n * n) * (phiM - E[sp.ion_k]);
+    mf[10 * nmv + a] = m * m * m * hg * driveNa;
+    mf[11 * nmv + a] = (n * n) * (n * n) * driveK;
 }
 
 template <int D>
