@@ -343,8 +343,9 @@ void deflation_prepare(knp_problem* p) {
 }
 
 // The solve is a block's work of 2 us in a kernel of its own of 4. The V-cycle's first kernel does it in
-// every block instead where that is less: its grid at most two blocks per SM, the sums few.
-constexpr int SOLVE_ROWS = 152 * 512, SOLVE_SUMS = 512;
+// every block instead where that is less: its grid at most two blocks per SM. The partial sums are few then
+// (a chunk per 1,024 nodes and cell: at most 140 with fewer than SOLVE_CELLS cells).
+constexpr int SOLVE_ROWS = 152 * 512;
 
 // Most blocks of a gather that runs beside the normalisation: two per SM. With more (some 470 at 75^3) the
 // scalars that each of them forms and the second vector that the normalisation then needs cost what the
@@ -396,7 +397,7 @@ static DeflFuse coarse_solution(knp_problem* p, const double* v, const double* s
     df.e.Eje = transpose ? d.Eej.p : d.Eje.p;
     df.e.Eej = transpose ? d.Eje.p : d.Eej.p;
     df.e.Ee = d.Ee.p;
-    df.solve = in_vcycle && d.nc < SOLVE_CELLS && p->n_nodes <= SOLVE_ROWS && d.gchunks + d.gext <= SOLVE_SUMS;
+    df.solve = in_vcycle && d.nc < SOLVE_CELLS && p->n_nodes <= SOLVE_ROWS;
     if (!df.solve) {
         count_launch();
         launch(k_defl_solve, 1, DT, q, df.e, d.y.p);

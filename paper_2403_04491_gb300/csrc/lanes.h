@@ -21,39 +21,33 @@ inline int row_lanes(int64_t rows, double mean_len) {
     return (16 * rows <= LANE_THREADS && mean_len > 4.0) ? 8 : 4;
 }
 
-// Sums of the four fields over the L lanes of a row (consecutive lanes of one warp, L a power of
-// two): on return out[0 .. LANE_FIELDS<L>) are the fields from lane_field<L>(t) on; the lanes from 4 on
+// Sums of the four fields over the L lanes of a row (consecutive lanes of one warp, L = 1 or a power of
+// two from 4): on return out[0 .. LANE_FIELDS<L>) are the fields from lane_field<L>(t) on; the lanes from 4 on
 // hold copies. A reduce-scatter: each halving step exchanges half of the values, so 4 lanes take
 // 3 shuffles and 3 adds instead of 8 (the adds of doubles are the scarce ones).
 template <int L>
-constexpr int LANE_FIELDS = L >= 4 ? 1 : 4 / L;
+constexpr int LANE_FIELDS = L >= 4 ? 1 : 4;
 template <int L>
 __device__ __forceinline__ int lane_field(int t) {
-    return L == 1 ? 0 : L == 2 ? 2 * t : (t & 3);
+    return L == 1 ? 0 : (t & 3);
 }
 template <class T, int L>
 __device__ __forceinline__ void lane_reduce4(const T acc[4], int t, T* out) {
+    static_assert(L == 1 || L >= 4, "lanes per row");
     if constexpr (L == 1) {
 #pragma unroll
         for (int f = 0; f < 4; ++f) out[f] = acc[f];
     } else {
-        constexpr int O = L == 2 ? 1 : 2;
-        const bool hi = (t & O) != 0;
+        const bool hi = (t & 2) != 0, odd = (t & 1) != 0;
         T a0 = hi ? acc[2] : acc[0], a1 = hi ? acc[3] : acc[1];
         const T b0 = hi ? acc[0] : acc[2], b1 = hi ? acc[1] : acc[3];
-        a0 += __shfl_xor_sync(0xffffffffu, b0, O);
-        a1 += __shfl_xor_sync(0xffffffffu, b1, O);
-        if constexpr (L == 2) {
-            out[0] = a0;
-            out[1] = a1;
-        } else {
-            const bool odd = (t & 1) != 0;
-            T a = odd ? a1 : a0;
-            a += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 1);
+        a0 += __shfl_xor_sync(0xffffffffu, b0, 2);
+        a1 += __shfl_xor_sync(0xffffffffu, b1, 2);
+        T a = odd ? a1 : a0;
+        a += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 1);
 #pragma unroll
-            for (int o = 4; o < L; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            out[0] = a;
-        }
+        for (int o = 4; o < L; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        out[0] = a;
     }
 }
 

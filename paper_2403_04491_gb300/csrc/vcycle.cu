@@ -245,6 +245,7 @@ struct VcycleOut {
 // four neighbour each other), among which they form w
 template <class T, int F>
 __device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0, const VN<T, F>& x, unsigned lanes = 0) {
+    static_assert(F == 4 || F == 1, "a thread or a lane per field");
     VN<double, F> z;
     for (int f = 0; f < F; ++f) z.v[f] = (double)x.v[f];
     const bool in = i < o.N_i;
@@ -256,7 +257,7 @@ __device__ __forceinline__ void store_out(const VcycleOut& o, int64_t i, int f0,
                          z2 = in ? o.ztau[0][2] : o.ztau[1][2];
             o.w[i] = z0 * z.v[0] + z1 * z.v[1] + z2 * z.v[2];
         }
-    } else if constexpr (F == 1) {
+    } else {
         if (o.w && lanes) {
             const double zt = f0 == 0 ? o.ztau[in ? 0 : 1][0] : f0 == 1 ? o.ztau[in ? 0 : 1][1] : o.ztau[in ? 0 : 1][2];
             double w = f0 < 3 ? zt * z.v[0] : 0.0;
