@@ -513,7 +513,7 @@ unsigned vec_grid(int64_t n4) {
 #define KNP_NV_CASE_k_orth_update_dot(N) case N: launch(k_orth_update_dot<N>, us.blocks, us.threads, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_orth_final(N) case N: launch(k_orth_final<N>, nb_vec + ga.nchunks + ga.next + 1, RED_THREADS, q, KNP_ARGS); break;
 #define KNP_NV_CASE_k_update_x(N) case N: k_update_x<N><<<nb_vec, RED_THREADS, 0, st>>>(KNP_ARGS); break;
-// Launch KERNEL<nv> with the caller's grid (nb_red or nb_vec) for a runtime nv in [0, 31]
+// Launch KERNEL<nv> for a runtime nv in [0, 31], with the caller's grid: rs or us (RedShape), or nb_vec
 #define KNP_LAUNCH_NV(nv, KERNEL)                                                                    \
     do {                                                                                             \
         switch (nv) {                                                                                \

@@ -10,11 +10,15 @@ namespace knp {
 // epilogue and lanes without an entry are FP64 instructions that one thread per row does not issue. One
 // thread per row is better once the rows are many for their length, 18 per SM and entry (2D, 7 entries: from
 // 19,200 rows, 3D, 14.5: from 39,700), and always from LANE_THREADS on, where the rows alone fill the SMs.
-// Against four lanes up to LANE_THREADS in every case: 2D 68,500 rows 26.6 -> 21.8 ms (its reverse sweep
-// 63.0 -> 53.3), 3D 72,400 rows, reverse sweep, 15.5 -> 14.0; at 15 per SM and entry P2 on 80x80 (27,000 rows of
-// 11.5) was 5% slower. Eight lanes up to 4,864 rows: with four there too, the Kir problem on 97x75 is 3%
-// slower (its first coarse level) and 4,612 unknowns 0.5%; with eight up to 9,728 rows it took 6.77 ms (7,700
-// rows of 7 entries on the finest level), now 6.21.
+// Three time steps (rtol 1e-11) with four lanes and with one, by the finest level's rows per SM and entry:
+//     2D  12.0  5.10  5.32 ms    15.2  6.20  6.10    18.7  6.95  6.55    22.0  8.81  7.86    31.5  11.3  10.1
+//     3D  10.7  7.08  7.32       14.4  8.91  8.83    17.2  9.40  9.40    20.5  11.3  11.1    32.5  14.7  13.3
+// (the 2D pass at 22.0 also in four iterations less of 86); at 15 P2 on 80x80 (27,000 rows of 11.5) is 5% slower
+// with one. Eight lanes up to 4,864 rows; three steps by the finest level's rows:
+//     2D   1,153  eight 2.10, four 2.12 ms     3,841  4.30, 4.27     5,473  4.25, 4.05     7,568  4.41, 4.01
+//     3D   1,429  eight 2.43, four 2.49        4,314  2.86, 2.78     6,128  4.40, 4.19     8,296  5.16, 4.69
+// Below the limit the two are within 3% of each other and neither always ahead: the Kir problem on 97x75 is 3%
+// slower with four (its first coarse level).
 constexpr int64_t LANE_THREADS = 152 * 512;
 inline int row_lanes(int64_t rows, double mean_len) {
     if (rows >= LANE_THREADS || rows >= 152 * 18 * mean_len) return 1;

@@ -16,7 +16,8 @@
 //     c^k row:  sum g^k x^k + sum e^k phi,     phi row:  sum a w + sum_k z_k (sum e^k phi),
 // seven FMAs per stored entry (g^k x^k, e^k phi, a w) for 60 bytes, where m, a with the
 // per-row tau take nine for 44 bytes. The transposed product keeps the m, a form.
-// One thread per row; the sliced-ELL layout makes the value loads of a warp contiguous.
+// One, four or eight lanes per row (lanes.h); the sliced-ELL layout makes the value loads of a warp
+// contiguous.
 //
 // Point pin (Remark 4.1): the stored values keep the phi_e column of the pinned node (so the
 // same-region values stay symmetric and serve the transpose too); both kernels treat that
@@ -86,8 +87,8 @@ __device__ __forceinline__ void op_store(int64_t k, const double* out, double* _
 
 // y = rowscale .* (b - A x)  (b, rowscale optional), L lanes per row (lanes.h). One and four lanes per
 // row read w = k_op_w(x); with eight the kernel is bound by its chain of loads, so it forms w from
-// the x it gathers anyway (three FMAs per entry). Read by four lanes, 117,504 unknowns in 3D 9.89 -> 9.70 ms
-// for three steps, P2 20^3 26.3 -> 24.7 for two; by eight, the Kir problem on 97x75 6.77 -> 6.90. The loads
+// the x it gathers anyway (three FMAs per entry). Read by four lanes, 117,504 unknowns in 3D 9.75 -> 9.53 ms
+// for three steps, P2 20^3 26.3 -> 24.8 for two; by eight, the Kir problem on 97x75 6.77 -> 6.90. The loads
 // of OP_BATCH entries are issued together.
 template <int L>
 constexpr int OP_BATCH = L == 1 ? 1 : 3;

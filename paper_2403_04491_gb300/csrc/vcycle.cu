@@ -640,7 +640,7 @@ AmgHierarchy::~AmgHierarchy() {
 // contiguous) if its rows are short (at most SELL_SHORT_ROW entries on average), or if they are
 // long but there are enough of them to keep the GPU busy with one thread each (at least
 // SELL_MIN_LONG_ROWS); and in either case only if padding every slice to its longest row stores
-// at most SELL_MAX_STORED entries per nonzero. Otherwise CSR with 4 S lanes per row. Measured:
+// at most SELL_MAX_STORED entries per nonzero. Otherwise CSR with 4 to 128 lanes per row. Measured:
 // the 512-cell 256^3 workload's first coarse level (1.7M rows of 58 entries) is 2.4% faster per
 // FGMRES iteration as sliced ELL; P2's first coarse level at 32^3 (19.5k rows of 143 entries, four
 // warps per SM with one thread per row) made the step 1.8 times slower.
@@ -1057,12 +1057,6 @@ bool vcycle_forms_w(const knp_problem* p) {
                        : forms_w(*static_cast<AmgDev<double>*>(p->amg->h64));
 }
 
-// z = V-cycle(P_0)(s .* v); v, s, z are [n][4] doubles on the device. The V-cycle is a fixed
-// sequence of about 15 launches, so it is captured once per (v, s, z) into a CUDA graph (on a
-// private stream, since the problem's stream may be the legacy one) and replayed on the
-// problem's stream. Each replay starts from
-// scratch (the first kernel writes b, x and d of the finest level), so replays are independent.
-// While a kernel class is being profiled the launches go out one by one.
 void p0_apply(knp_problem* p, const double* x, double* y) {
     KNP_REQUIRE(p->amg && p->amg->h64, KNP_ERR_STATE, "P_0 products need the FP64 hierarchy");
     DevLevel<double>& L = *static_cast<AmgDev<double>*>(p->amg->h64)->L[0];
@@ -1071,6 +1065,13 @@ void p0_apply(knp_problem* p, const double* x, double* y) {
     KNP_CUDA(cudaGetLastError());
 }
 
+// z = V-cycle(P_0)(s .* v); v, s, z are [n][4] doubles on the device. The V-cycle is a fixed
+// sequence of about 15 launches, so it is captured once per set of arguments (AmgHierarchy::graphs)
+// into a CUDA graph (on a private stream, since the problem's stream may be the legacy one) and
+// replayed on the problem's stream. Each replay starts from
+// scratch (the first kernel writes b, x and d of the finest level), so replays are independent.
+// While a kernel class is being profiled, and with KNP_NO_GRAPHS, the launches go out one by one.
+// (The V-cycles inside FGMRES iterations are parts of those iterations' graphs instead, gmres.cu.)
 void vcycle_apply(knp_problem* p, const double* v, const double* s, double* z, const DeflFuse* dfp, double* w) {
     KNP_REQUIRE(p->amg, KNP_ERR_STATE, "knp_amg_setup has not been called");
     AmgHierarchy& H = *p->amg;

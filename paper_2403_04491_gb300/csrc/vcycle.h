@@ -37,7 +37,7 @@ struct DeflFuse {
     CoarseSolve e;
 };
 
-// One captured V-cycle: a CUDA graph instantiated for a given (input, scale, output) triple.
+// One captured V-cycle: a CUDA graph instantiated for given arguments (AmgHierarchy::graphs).
 struct VcycleGraph {
     cudaGraphExec_t exec = nullptr;
     int launches = 0;
@@ -50,7 +50,9 @@ struct AmgHierarchy {
     std::vector<int64_t> nodes, nnz;
     void* h64 = nullptr;   // AmgDev<double>
     void* h32 = nullptr;   // AmgDev<float>
-    // CUDA graphs of the V-cycle (one per FGMRES basis slot), captured on a private stream
+    // CUDA graphs of single V-cycles, captured on a private stream: per input, scale, output, coarse
+    // solution, direction of the coarse correction and the product's w. FGMRES uses them for the first basis
+    // vector and, with CG(P_0), for all
     bool use_graphs = true;
     cudaStream_t gstream = nullptr;
     std::map<std::tuple<const double*, const double*, double*, const double*, int, double*>, VcycleGraph> graphs;

@@ -1,7 +1,7 @@
 """The kernels' choices of lanes, launch and grouping at the sizes where they change.
 
 * operator products with 8, 4 and 1 lanes per row, and with the last block and slice partly empty;
-* the V-cycle, whose last levels run in one cluster: symmetric when it smooths equally on both sides;
+* the V-cycle: symmetric when it smooths equally on both sides;
 * time steps from captured graphs against single launches.
 """
 import numpy as np
@@ -38,10 +38,9 @@ def test_operator_products_at_the_lane_limits(nx):
     assert blockwise_vector_error(pb, prob.apply_operator_transpose(x), A.T @ x) < 1e-12
 
 
-# one to four levels; from the finest level's transfers inside the cluster to none of them. P_0's field blocks
-# are independent, so each is symmetric by itself. The concentrations' blocks are mass matrices and some
-# stiffness (condition below 1e3): the dense inverse of the coarsest level is symmetric to that times eps, and
-# the rest to some tens of eps. The potentials' are nearly singular (1e9 taken).
+# one to four levels. P_0's field blocks are independent, so each is symmetric by itself. The concentrations'
+# blocks are mass matrices and some stiffness (condition below 1e3): the dense inverse of the coarsest level is
+# symmetric to that times eps, and the rest to some tens of eps. The potentials' are nearly singular (1e9 taken).
 @pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
 @pytest.mark.parametrize("config,nx", [(1, 20), (1, 32), (1, 97), (4, 256), (2, 11), (2, 29), (2, 48)])
 def test_vcycle_is_symmetric(config, nx, precision):
